@@ -528,13 +528,24 @@ __global__ void __launch_bounds__(EMPTY_THREADS) k_empty_pass(LevelDev g, int32_
   int32_t* fbase = icnt + 2 * B;  // exclusive prefixes (B + 1 each)
   int32_t* mbase = icnt + 3 * B + 1;
   int cf = 0, ce = 0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    const bool f = size[i] == 0, m = target[i] == TO_EMPTY;
+  // (warp-uniform loop) consecutive nodes mostly share an instance: the lanes
+  // of the same one are counted with one atomic.  A late iteration has hundreds
+  // of thousands of free labels, and one atomic each on B counters took 0.3 ms
+  // of a batch of 36 instances (N = 1.5 M, now 0.03 ms).
+  for (int64_t i0 = lo + (threadIdx.x & ~31); i0 < hi; i0 += blockDim.x) {
+    const int64_t i = i0 + (threadIdx.x & 31);
+    const bool in = i < hi;
+    const bool f = in && size[i] == 0, m = in && target[i] == TO_EMPTY;
     cf += f;
     ce += m;
     if (B > 1) {
-      if (f) atomicAdd(&fcnt[node_inst(g, (int32_t)i)], 1);
-      if (m) atomicAdd(&mcnt[node_inst(g, (int32_t)i)], 1);
+      const int32_t inst = in ? node_inst(g, (int32_t)i) : -1;
+      const unsigned peers = __match_any_sync(0xffffffffu, inst);
+      const int nf = __popc(__ballot_sync(0xffffffffu, f) & peers), nm = __popc(__ballot_sync(0xffffffffu, m) & peers);
+      if (in && (threadIdx.x & 31) == __ffs(peers) - 1) {
+        if (nf) atomicAdd(&fcnt[inst], nf);
+        if (nm) atomicAdd(&mcnt[inst], nm);
+      }
     }
   }
   int tf, te;
