@@ -430,6 +430,8 @@ void run_leiden(Ctx& c, const SupraGraph& G, const std::vector<InstParams>& jobs
   int32_t* iter_active = c.ws->get<int32_t>("s_iter_active", B);
   fill_i32(c, iter_active, 1, B);
   setup_null_model(S);
+  setup_tracking(S);
+  S.warm = init != nullptr;
 
   int32_t* labA = c.ws->get<int32_t>("lab_A", N0);
   int32_t* labB = c.ws->get<int32_t>("lab_B", N0);

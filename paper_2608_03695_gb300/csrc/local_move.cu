@@ -27,12 +27,14 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 
 #include "../../include/mslice.h"
 #include "decide.cuh"
 #include "solver.h"
+#include "track.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -93,36 +95,46 @@ constexpr int BUCKET_THREADS = 256;
 constexpr int BUCKET_ITEMS = 16;
 constexpr int64_t BUCKET_CHUNK = (int64_t)BUCKET_THREADS * BUCKET_ITEMS;
 constexpr int BUCKET_MAX_SEGS = 64 * NTIERS;  // segments (K * NTIERS) for K <= 64
-constexpr uint16_t BUCKET_FROZEN = 0xffff;    // segment of a node of a converged instance
 
 __device__ __forceinline__ int bucket_seg(const LevelDev& g, const uint8_t* tier, uint64_t seed, uint64_t tag,
                                           uint64_t it, uint64_t lvl, uint64_t r, int K, const int32_t* active,
                                           int64_t v) {
-  if (active && !active[node_inst(g, (int32_t)v)]) return BUCKET_FROZEN;  // converged instance: frozen
+  if (active && !active[node_inst(g, (int32_t)v)]) return SEG_FROZEN;  // converged instance: frozen
   return vertex_class(seed, tag, it, lvl, r, local_id(g, (int32_t)v), K) * NTIERS + tier[v];
 }
 
-// Step 1: segment of every node (seg, one byte) and counts[s * nchunks + chunk].
+// Step 1: segment of every node and counts[s * nchunks + chunk].  In a pruned
+// round (trk) a settled node keeps its segment, marked, and is not counted.
 __global__ void __launch_bounds__(BUCKET_THREADS)
     k_bucket_count(LevelDev g, const uint8_t* tier, uint64_t seed, uint64_t tag, uint64_t it, uint64_t lvl, uint64_t r,
-                   int K, const int32_t* active, const int32_t* r_dev, uint16_t* seg, int32_t* counts,
+                   int K, const int32_t* active, const int32_t* r_dev, TrackView trk, uint16_t* seg, int32_t* counts,
                    int64_t nchunks) {
   __shared__ int32_t cnt[BUCKET_MAX_SEGS];
   if (r_dev) r = (uint64_t)*r_dev;  // a graph replay reads its round here
   const int nseg = K * NTIERS;
+  const bool prune = track_mode(trk) == TRACK_PRUNE;
+  int settled = 0;
   for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
     for (int i = threadIdx.x; i < nseg; i += BUCKET_THREADS) cnt[i] = 0;
     __syncthreads();
     for (int k = 0; k < BUCKET_ITEMS; ++k) {
       const int64_t v = ch * BUCKET_CHUNK + (int64_t)k * BUCKET_THREADS + threadIdx.x;
       if (v >= g.N) break;
-      const int sg = bucket_seg(g, tier, seed, tag, it, lvl, r, K, active, v);
+      int sg = bucket_seg(g, tier, seed, tag, it, lvl, r, K, active, v);
+      if (prune && sg < nseg && track_settled(trk, g, (int32_t)v)) {
+        sg |= SEG_SETTLED;
+        ++settled;
+      }
       seg[v] = (uint16_t)sg;
       if (sg < nseg) atomicAdd(&cnt[sg], 1);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < nseg; i += BUCKET_THREADS) counts[(int64_t)i * nchunks + ch] = cnt[i];
     __syncthreads();
+  }
+  if (prune) {
+    settled = warp_sum(settled);
+    if ((threadIdx.x & 31) == 0 && settled) atomicAdd(&trk.state[TRACK_SETTLED], settled);
   }
 }
 
@@ -260,6 +272,7 @@ struct LMPolicy {
   SigStore sig;
   const u128* lam;
   int32_t* target;
+  TrackView trk;
 
   typedef Slot Probe;
   // Per node: own community and its size; at level 0 the node's snapshot s,
@@ -355,6 +368,8 @@ struct LMPolicy {
       if (!(vc.size_a == 1 && best.label > a && size[best.label] == 1)) t = best.label;
     }
     target[v] = t;
+    if (t == NO_MOVE && track_mode(trk) != TRACK_OFF)
+      track_record(trk, g, vc.om, v, vc.size_a == 1, has, Ga, best.G);
   }
 };
 
@@ -380,9 +395,99 @@ __device__ __forceinline__ int seg_total(const Segs& sg) {
   return t;
 }
 
-// Applies the sub-round's decisions: labels, community sizes and Sigma, and
-// resets each applied decision.  Moves to an empty community only leave here
-// (their label is assigned by k_empty_pass).
+// The bucket lists of a round, for nodes that join them while it runs.
+struct BucketLists {
+  int32_t* lists;
+  int64_t row_stride;
+  int32_t* cursors;
+  TierOff off;
+  const uint16_t* seg;
+};
+
+// Appends node u (segment sg, class and tier) to its class's list.
+__device__ __forceinline__ void bucket_append(const BucketLists& bl, int sg, int32_t u) {
+  const int q = sg / NTIERS, t = sg % NTIERS;
+  bl.lists[(int64_t)q * bl.row_stride + bl.off.off[t] + atomicAdd(&bl.cursors[sg], 1)] = u;
+}
+
+// Round start (one block): the round's tracking mode from what the round before
+// did, the budgets of every null slice and what their change costs a settled
+// node, and the round's counters.
+//   - Tracking starts when the movement, going on as in the last two rounds,
+//     is expected to stay under a twelfth of the nodes, and stops past a
+//     quarter: the movers' pushes and the drift of the null sums would leave
+//     few nodes settled for what they cost.
+//   - Pruning that leaves three nodes in four in the lists is given up until
+//     the movement has fallen to a quarter, or for a number of rounds that
+//     doubles each time (communities can swap nodes for dozens of rounds).
+//   - Levels with fewer entries, or with short rows (the decisions cost little
+//     more than the tracking) or long strength lists, are not tracked.
+constexpr int64_t TRACK_MIN_ENTRIES = 1 << 22, TRACK_MIN_DEGREE = 8;
+constexpr double TRACK_START = 1.0 / 12, TRACK_STOP = 1.0 / 4;
+constexpr int TRACK_FIRST_PAUSE = 8;
+
+__global__ void __launch_bounds__(512) k_round_begin(TrackView trk, int32_t Tn, int first, int32_t mode_init,
+                                                     int32_t* counters, const int32_t* cursors, int nseg) {
+  __shared__ int32_t mode_sh;
+  __shared__ int listed_sh;
+  if (threadIdx.x == 0) listed_sh = 0;
+  __syncthreads();
+  if (!first)
+    for (int i = threadIdx.x; i < nseg; i += blockDim.x) atomicAdd(&listed_sh, cursors[i]);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const long long moved = (long long)(((unsigned long long)(uint32_t)counters[1] << 32) | (uint32_t)counters[0]);
+    const long long listed = listed_sh, settled = trk.state[TRACK_SETTLED];
+    int32_t m = mode_init;
+    if (first) {
+      trk.state[TRACK_PAUSE] = 0;
+      trk.state[TRACK_NEXT_PAUSE] = TRACK_FIRST_PAUSE;
+      trk.state[TRACK_MOVED] = 0;
+    } else {
+      const int32_t before = trk.state[TRACK_MODE], last = trk.state[TRACK_MOVED];
+      const double active = (double)(listed + settled);
+      const double expect = last > 0 ? (double)moved * (double)moved / (double)last : (double)moved;
+      trk.state[TRACK_MOVED] = (int32_t)moved;
+      if (before == TRACK_PRUNE && listed > 3 * settled) {
+        trk.state[TRACK_PAUSE] = trk.state[TRACK_NEXT_PAUSE];
+        trk.state[TRACK_NEXT_PAUSE] = min(2 * trk.state[TRACK_NEXT_PAUSE], 1 << 20);
+        trk.state[TRACK_PAUSE_MOVED] = (int32_t)moved;
+      }
+      if (trk.state[TRACK_PAUSE] > 0) {
+        trk.state[TRACK_PAUSE]--;
+        if (4 * moved < trk.state[TRACK_PAUSE_MOVED]) trk.state[TRACK_PAUSE] = 0;
+      }
+      if (trk.state[TRACK_PAUSE] > 0)
+        m = TRACK_OFF;
+      else if (before == TRACK_OFF)
+        m = expect < TRACK_START * active ? TRACK_RECORD : TRACK_OFF;
+      else
+        m = (double)moved < TRACK_STOP * active ? TRACK_PRUNE : TRACK_OFF;
+    }
+    mode_sh = m;
+    trk.state[TRACK_MODE] = m;
+    trk.state[TRACK_PAST] = 0;
+    trk.state[TRACK_SETTLED] = 0;
+    counters[0] = counters[1] = counters[2] = 0;
+  }
+  __syncthreads();
+  const int32_t m = mode_sh;
+  if (m == TRACK_OFF) return;
+  for (int32_t s = threadIdx.x; s < Tn; s += blockDim.x) {
+    const long long E = trk.E[s], base = trk.base[s];
+    trk.E[s] = 0;
+    if (m == TRACK_RECORD) {
+      trk.B[s] = base;
+      continue;
+    }
+    // the budget: half of what moved in the round before (movement mostly
+    // falls faster than that), and the base
+    const long long B = E / 2 + base, grown = E + B - trk.B[s];
+    trk.drate[s] = grown > 0 ? (double)trk.lam[s] * (double)grown * trk.scale : 0.0;
+    trk.B[s] = B;
+  }
+}
+
 // End of a round of the device-side loop: accounts the round (acc: rounds
 // run, moves, moves of this round), advances the round index and lets the
 // loop go on while nodes moved, rounds remain, no hash region has passed half
@@ -424,17 +529,61 @@ __device__ __forceinline__ void move_slices(const LevelDev& g, SigStore& sig, in
   }
 }
 
+// Tracked rounds: the strength a mover takes through its null slices counts
+// against their budgets.  At level 0 (one slice a node, lists in node order)
+// most movers of a warp share a slice: their strengths are added up first.
+__device__ __forceinline__ void track_moved(const TrackView& trk, int32_t s, long long k) {
+  const long long old = (long long)atomicAdd((ull*)&trk.E[s], (ull)k);
+  if (old + k > trk.B[s]) trk.state[TRACK_PAST] = 1;
+}
+
+// A mover's warp takes the move off the margins of the mover's neighbours; a
+// settled one that has to decide after all joins the list of its class when
+// that is still to come in this round (it decides in the next one otherwise:
+// its class has been decided, from the state before this move).
+__device__ __forceinline__ void track_push(const TrackView& trk, const LevelDev& g, const int32_t* labels,
+                                           const BucketLists& bl, int q, int32_t v, int32_t from, int32_t to,
+                                           int64_t rb, int64_t re, int lane) {
+  const Omega om = node_omega(g, v);
+  for (int64_t e = rb + lane; e < re; e += 32) {
+    int32_t u;
+    long long w;
+    if (!edge_at(g, e, u, w, om)) continue;
+    // (the label of a neighbour that moves in this sub-round may be read before
+    // or after its move: that neighbour has to decide either way)
+    const long long d = track_drop(trk, labels[u], from, to, w);
+    if (*(volatile long long*)&trk.slack[u] < 0) continue;
+    const long long old = (long long)atomicAdd((ull*)&trk.slack[u], (ull)(-d));
+    if (old >= 0 && old < d) {
+      const int sg = bl.seg[u];
+      if ((sg & SEG_SETTLED) && sg != SEG_FROZEN) {
+        const int sgu = sg & ~(int)SEG_SETTLED;
+        if (sgu / NTIERS > q) bucket_append(bl, sgu, u);
+      }
+    }
+  }
+}
+
+// Applies the sub-round's decisions: labels, community sizes and Sigma, and
+// resets each applied decision.  Moves to an empty community only leave here
+// (their label is assigned by k_empty_pass).  Tracked rounds also lower the
+// margins of the movers' neighbours.
 __global__ void k_lm_apply(LevelDev g, Segs sg, int32_t* labels, int32_t* size, SigStore sig, int32_t* target,
-                           int32_t* counters, int32_t* inst_moved) {
+                           int32_t* counters, int32_t* inst_moved, TrackView trk, BucketLists bl, int q) {
   const int total = seg_total(sg);
+  const bool track = track_mode(trk) != TRACK_OFF;
   const int lane = threadIdx.x & 31;
+  // List items a warp takes at a time: 32, but a tracked round deals a short
+  // list out to all warps, as a warp pushes its movers one after another.
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  const int take = track ? min(32, (total + warps - 1) / warps) : 32;
   int local = 0, local_empty = 0;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < total;
-       base += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * take; base < total;
+       base += (int64_t)warps * take) {
     const int64_t idx = base + lane;
     int32_t v = 0, t = NO_MOVE, a = 0;
-    int64_t b = 0, e = 0;
-    if (idx < total && seg_item(sg, idx, v)) t = target[v];
+    int64_t b = 0, e = 0, rb = 0, re = 0;
+    if (lane < take && idx < total && seg_item(sg, idx, v)) t = target[v];
 #if MSLICE_CHECKED
     if (t != NO_MOVE && (t >= g.N || (t < 0 && t != TO_EMPTY))) {
       atomicOr(g.chk, ERR_BOUNDS);
@@ -447,6 +596,37 @@ __global__ void k_lm_apply(LevelDev g, Segs sg, int32_t* labels, int32_t* size, 
       atomicSub(&size[a], 1);
       slice_range(g, v, b, e);
       if (e - b <= 32) move_slices(g, sig, v, a, t, b, e, 0, 1);
+      if (track) {
+        rb = g.rowptr[v];
+        re = g.rowptr[v + 1];
+        trk.slack[v] = TRACK_DEAD;
+      }
+    }
+    if (track) {
+      const unsigned mv = __ballot_sync(0xffffffffu, t != NO_MOVE);
+      if (mv && g.is0) {
+        const int32_t s = t != NO_MOVE ? node_slice0(g, v) : -1;
+        const long long k = t != NO_MOVE ? g.k0[v] : 0;
+        const int32_t s0 = __shfl_sync(0xffffffffu, s, __ffs(mv) - 1);
+        const long long k0 = warp_sum(s == s0 ? k : 0ll);
+        if (lane == 0)
+          track_moved(trk, s0, k0);
+        if (t != NO_MOVE && s != s0) track_moved(trk, s, k);
+      } else if (t != NO_MOVE) {
+        for (int64_t j = b; j < e; ++j) {
+          int32_t s;
+          long long k;
+          slice_entry(g, v, j, s, k);
+          track_moved(trk, s, k);
+        }
+      }
+      for (unsigned m = mv; m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        const int32_t vs = __shfl_sync(0xffffffffu, v, src), as = __shfl_sync(0xffffffffu, a, src),
+                      ts = __shfl_sync(0xffffffffu, t, src);
+        const int64_t rbs = __shfl_sync(0xffffffffu, rb, src), res = __shfl_sync(0xffffffffu, re, src);
+        track_push(trk, g, labels, bl, q, vs, as, ts, rbs, res, lane);
+      }
     }
     unsigned wide = __ballot_sync(0xffffffffu, t != NO_MOVE && e - b > 32);
     while (wide) {
@@ -512,10 +692,31 @@ __device__ __forceinline__ T block_scan_excl(T x, T* sm, T& total) {
 //   freelist: all free labels in ascending order; mrank: movers' global ranks
 //   icnt:     4*B + 2 ints (per-instance counts, then their prefixes); zero
 //             on entry and left zero on exit
+// In a pruned round whose movement has passed a budget it first lets the
+// settled nodes of the next class rejoin its lists (see track.cuh).
 __global__ void __launch_bounds__(EMPTY_THREADS) k_empty_pass(LevelDev g, int32_t B, int32_t* target, int32_t* labels,
                                                               int32_t* size, SigStore sig, int32_t* counters,
                                                               int32_t* blk, int32_t* freelist, int32_t* mrank,
-                                                              int32_t* icnt) {
+                                                              int32_t* icnt, TrackView trk, BucketLists bl,
+                                                              int q_next) {
+  if (trk.state && trk.state[TRACK_MODE] == TRACK_PRUNE && trk.state[TRACK_PAST]) {
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < g.N; v += (int64_t)gridDim.x * blockDim.x) {
+      const int sg = bl.seg[v];
+      if (!(sg & SEG_SETTLED) || sg == SEG_FROZEN) continue;
+      const int sgv = sg & ~(int)SEG_SETTLED;
+      if (sgv / NTIERS != q_next || trk.slack[v] < 0) continue;
+      int64_t b, e;
+      slice_range(g, (int32_t)v, b, e);
+      bool past = false;
+      for (int64_t j = b; j < e && !past; ++j) {
+        int32_t s;
+        long long k;
+        slice_entry(g, (int32_t)v, j, s, k);
+        past = trk.E[s] > trk.B[s];
+      }
+      if (past) bucket_append(bl, sgv, (int32_t)v);
+    }
+  }
   const int n_empty = counters[2];
   if (n_empty == 0) return;
   __shared__ int32_t sm[33];
@@ -755,27 +956,48 @@ static std::vector<int64_t> null_slice_nodes(const Solver& S) {
   return out;
 }
 
-// Largest mass of a null slice, the bound on every sum its table keys hold:
-// 2m_s (Q_MS), the node count n (CPM, whose strengths are 1) or the
-// instance's 2M' in units of 1/omega_den (the global model).
-static int64_t null_slice_mass_max(const Solver& S) {
+// Mass of every null slice, the bound on every sum its table keys hold: 2m_s
+// (Q_MS), the node count n (CPM, whose strengths are 1) or the instance's 2M'
+// in units of 1/omega_den (the global model; INT64_MAX past 2^62).
+static std::vector<int64_t> null_slice_masses(const Solver& S) {
   const SupraGraph& G = *S.G0;
-  int64_t mx = 0;
+  std::vector<int64_t> out(S.Tn > 0 ? S.Tn : 1, 0);
   for (int32_t i = 0; i < G.B; ++i) {
     const InstInfo& in = G.inst[i];
-    if (S.p.cpm) {
-      mx = std::max<int64_t>(mx, in.n);
-    } else if (S.p.global_null) {
+    if (S.p.global_null) {
       u128 sum2m = 0;
       for (int32_t s = in.soff; s < in.soff + in.T; ++s) sum2m += (u128)(ull)G.two_m_host[s];
       const u128 m = (u128)(ull)S.od_h[i] * sum2m + (u128)(ull)S.csum_h[i];
-      mx = m >= ((u128)1 << 62) ? INT64_MAX : std::max<int64_t>(mx, (int64_t)m);
-      if (mx == INT64_MAX) break;
+      if (i < (int32_t)out.size()) out[i] = m >= ((u128)1 << 62) ? INT64_MAX : (int64_t)m;
     } else {
-      for (int32_t s = in.soff; s < in.soff + in.T; ++s) mx = std::max<int64_t>(mx, G.two_m_host[s]);
+      for (int32_t s = in.soff; s < in.soff + in.T && s < (int32_t)out.size(); ++s)
+        out[s] = S.p.cpm ? in.n : G.two_m_host[s];
     }
   }
-  return mx;
+  return out;
+}
+
+// What the margins of local moving are kept against (see track.cuh), once per
+// solve.  A slice's smallest budget is 1/256 of its mass: movement within it
+// costs a settled node under 1% of its strength in margin, and a quiet round
+// stays inside it.  Slices of a handful of edges get a 1/16, up to 8.
+void setup_tracking(Solver& S) {
+  Ctx& c = *S.c;
+  const SupraGraph& G = *S.G0;
+  const std::vector<int64_t> mass = null_slice_masses(S);
+  S.track_base_h.resize(mass.size());
+  for (size_t s = 0; s < mass.size(); ++s)
+    S.track_base_h[s] = std::max<int64_t>(mass[s] >> 8, std::min<int64_t>(mass[s] >> 4, 8));
+  S.track_base = c.ws->get<long long>("s_track_base", mass.size());
+  check_cuda(cudaMemcpyAsync(S.track_base, S.track_base_h.data(), mass.size() * sizeof(long long),
+                             cudaMemcpyHostToDevice, c.stream), "copy");
+  S.total_strength = 0;
+  for (int32_t i = 0; i < G.B; ++i) {
+    const InstInfo& in = G.inst[i];
+    double sum2m = 0;
+    for (int32_t s = in.soff; s < in.soff + in.T; ++s) sum2m += (double)G.two_m_host[s];
+    S.total_strength += (double)S.od_h[i] * sum2m + (double)S.csum_h[i];
+  }
 }
 
 void configure_stores(Solver& S, int64_t N) {
@@ -818,7 +1040,8 @@ void configure_stores(Solver& S, int64_t N) {
     S.region_T = T;
   }
   // 8-byte slots when no null slice's mass reaches 2^32 (no sum can)
-  bool narrow = null_slice_mass_max(S) < ((int64_t)1 << 32);
+  bool narrow = true;
+  for (int64_t m : null_slice_masses(S)) narrow = narrow && m < ((int64_t)1 << 32);
   if (const char* e = std::getenv("MSLICE_WIDE_SLOTS")) narrow = narrow && std::atoi(e) == 0;
   S.sig_h.narrow = S.kr_h.narrow = narrow ? 1 : 0;
   S.sig_h.nregions = S.kr_h.nregions = (int32_t)(S.region_h.size() - 1);
@@ -863,11 +1086,16 @@ TierSegs bucket_segments(Solver& S, int q) {
   return sg;
 }
 
-void bucket(Solver& S, const Level& L, uint64_t tag, int it, int lvl, int r, const int32_t* active,
-            const int32_t* r_dev) {
-  Ctx& c = *S.c;
+static TierOff tier_offsets(const Solver& S) {
   TierOff to;
   for (int t = 0; t < NTIERS; ++t) to.off[t] = S.tier_off[t];
+  return to;
+}
+
+static void bucket_tracked(Solver& S, const Level& L, uint64_t tag, int it, int lvl, int r, const int32_t* active,
+                           const int32_t* r_dev, const TrackView& trk) {
+  Ctx& c = *S.c;
+  const TierOff to = tier_offsets(S);
   const int64_t N = L.d.N;
   if (N == 0) {
     check_cuda(cudaMemsetAsync(S.cursors, 0, NTIERS * S.p.K * sizeof(int32_t), c.stream), "memset");
@@ -876,10 +1104,36 @@ void bucket(Solver& S, const Level& L, uint64_t tag, int it, int lvl, int r, con
   const int64_t nchunks = (N + BUCKET_CHUNK - 1) / BUCKET_CHUNK;
   const unsigned grid = (unsigned)std::min<int64_t>(nchunks, fixed_grid(16));
   launch(c, k_bucket_count, dim3(grid), dim3(BUCKET_THREADS), 0, L.d, (const uint8_t*)S.tier, S.p.seed, tag,
-         (uint64_t)it, (uint64_t)lvl, (uint64_t)r, S.p.K, active, r_dev, S.bseg, S.bcounts, nchunks);
+         (uint64_t)it, (uint64_t)lvl, (uint64_t)r, S.p.K, active, r_dev, trk, S.bseg, S.bcounts, nchunks);
   launch(c, k_bucket_scan, dim3(S.p.K * NTIERS), dim3(1024), 0, S.bcounts, nchunks, S.cursors);
   launch(c, k_bucket_write, dim3(grid), dim3(BUCKET_THREADS), 0, L.d.N, (const uint16_t*)S.bseg,
          (const int32_t*)S.bcounts, nchunks, S.p.K, S.lists, (int64_t)S.N0, to);
+}
+
+void bucket(Solver& S, const Level& L, uint64_t tag, int it, int lvl, int r, const int32_t* active,
+            const int32_t* r_dev) {
+  bucket_tracked(S, L, tag, it, lvl, r, active, r_dev, TrackView{});
+}
+
+// The tracking state of a level (see track.cuh).  Margins live in a
+// refinement array, which is only read after local moving.  Their unit is set
+// so that a node of average strength has about 2^20 of them.
+static TrackView track_view(Solver& S, const Level& L) {
+  Ctx& c = *S.c;
+  TrackView t;
+  t.state = c.ws->get<int32_t>("s_track_state", TRACK_WORDS);
+  t.slack = S.Wsel;
+  t.E = c.ws->get<long long>("s_track_E", S.Tn);
+  t.B = c.ws->get<long long>("s_track_B", S.Tn);
+  t.drate = c.ws->get<double>("s_track_drate", S.Tn);
+  t.base = S.track_base;
+  t.lam = S.lam;
+  const double avg = S.total_strength / (double)(L.d.N > 0 ? L.d.N : 1);
+  int bits = 0;
+  while (bits < 60 && avg > (double)(1ll << bits)) ++bits;
+  t.F = std::max(-40, std::min(16, 20 - bits));
+  t.scale = std::ldexp(1.0, t.F - 63);
+  return t;
 }
 
 // Chooses the degree cuts of the decision tiers for this solve: every
@@ -1004,6 +1258,20 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
   polh.sig = pol.sig;
   polh.lam = pol.lam;
   polh.target = pol.target;
+  // Margins are recorded once few nodes move: from the level's first round,
+  // except where the level starts from singletons (its first rounds move most
+  // nodes), and not on a level whose tier cuts are still being tuned.
+  const bool from_singletons = lvl == 0 && it == 0 && !S.warm;
+  // (MSLICE_TRACK_MIN_ENTRIES: tracks every level of that many entries)
+  const char* track_min = std::getenv("MSLICE_TRACK_MIN_ENTRIES");
+  const bool worth = track_min ? L.nnz >= std::atoll(track_min)
+                               : L.nnz >= TRACK_MIN_ENTRIES && L.nnz >= TRACK_MIN_DEGREE * (int64_t)N &&
+                                     L.ns <= 4 * (int64_t)N;
+  const TrackView trk = (!worth || (S.p.autotune && lvl == 0)) ? TrackView{} : track_view(S, L);
+  const int32_t mode_init = from_singletons ? TRACK_OFF : TRACK_RECORD;
+  pol.trk = polh.trk = trk;
+  const BucketLists bl{S.lists, (int64_t)S.N0, S.cursors, tier_offsets(S), S.bseg};
+  bool first_round = true;
   auto decide = [&](const TierSegs& sg) {
     if (S.sig.d)
       decide_all(c, pol, sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
@@ -1026,8 +1294,12 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
   //         the enclosing graph loop (r_dev holds the round).
   enum class RoundEnd { HOST, LOOP };
   auto round_body = [&](int r, const int32_t* r_dev, bool prof, RoundEnd end, cudaGraphConditionalHandle h) {
-    check_cuda(cudaMemsetAsync(S.counters, 0, 3 * sizeof(int32_t), c.stream), "memset");
-    bucket(S, L, 0, it, lvl, r, active, r_dev);
+    if (trk.state)
+      launch(c, k_round_begin, dim3(1), dim3(512), 0, trk, S.Tn, (int)first_round, mode_init, S.counters,
+             (const int32_t*)S.cursors, S.p.K * NTIERS);
+    else
+      check_cuda(cudaMemsetAsync(S.counters, 0, 3 * sizeof(int32_t), c.stream), "memset");
+    bucket_tracked(S, L, 0, it, lvl, r, active, r_dev, trk);
     for (int q = 0; q < S.p.K; ++q) {
       const Segs sg = bucket_segments(S, q);
       if (prof) {
@@ -1042,9 +1314,9 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
         decide(sg);
       }
       launch(c, k_lm_apply, dim3(fixed_grid(4)), dim3(APPLY_THREADS), 0, L.d, sg, labels, S.size, S.sig, S.target,
-             S.counters, batch ? S.inst_moved : nullptr);
+             S.counters, batch ? S.inst_moved : nullptr, trk, bl, q);
       launch_coop(c, k_empty_pass, dim3(S.empty_grid), dim3(EMPTY_THREADS), 0, L.d, S.B, S.target, labels, S.size,
-                  S.sig, S.counters, S.empty_blk, S.freelist, S.tmp32b, S.inst_cnt);
+                  S.sig, S.counters, S.empty_blk, S.freelist, S.tmp32b, S.inst_cnt, trk, bl, q + 1);
     }
     if (batch)
       launch(c, k_round_freeze, dim3(grid_for(S.B, 256)), dim3(256), 0, S.lm_active, S.inst_moved, S.B);
@@ -1144,8 +1416,10 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
     S.lm_rounds++;
     S.lm_edges += L.nnz_eff;
     const bool prof = c.profile && lvl == 0;
+    const size_t spans = prof ? c.prof_spans->size() : 0;
     if (prof) c.prof_bytes += 12 * L.nnz_eff + 40 * (int64_t)N;
     round_body(r, nullptr, prof, RoundEnd::HOST, cudaGraphConditionalHandle{});
+    first_round = false;
     sync(c);
     struct {
       int64_t moved;
@@ -1161,6 +1435,17 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
     rebuild = !S.sig.d && rb.used > 0;  // a region has taken half of its slots
     out.rounds++;
     out.moves += rb.moved;
+    if (prof && trk.state) {
+      // the decision timing covers the rounds in which every node decides
+      if (*static_cast<const int32_t*>(readback(c, trk.state + TRACK_MODE, sizeof(int32_t))) == TRACK_PRUNE) {
+        for (size_t k = spans; k < c.prof_spans->size(); ++k) {
+          cudaEventDestroy((*c.prof_spans)[k].first);
+          cudaEventDestroy((*c.prof_spans)[k].second);
+        }
+        c.prof_spans->resize(spans);
+        c.prof_bytes -= 12 * L.nnz_eff + 40 * (int64_t)N;
+      }
+    }
     ++r;
     if (rb.moved == 0) break;
     if (r == max_rounds) out.capped = true;

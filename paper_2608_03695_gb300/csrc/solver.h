@@ -94,6 +94,13 @@ struct Solver {
   int32_t* inst_moved = nullptr;   // per instance: moved in the current round
   int32_t* round_dev = nullptr;    // the round the device-side round loop is at
   long long* loop_acc = nullptr;   // device-side round loop: rounds run, moves, moves of the last round
+  // tracking of settled nodes (track.cuh): smallest budget per null slice, the
+  // strength of all nodes in units of 1/od, and whether the solve started from
+  // given labels
+  long long* track_base = nullptr;
+  std::vector<long long> track_base_h;
+  double total_strength = 0;
+  bool warm = false;
   int32_t* wqueue = nullptr;       // work counters of the decision kernels, one per degree tier
   int64_t* goff = nullptr;      // global-tier table offsets
   int32_t* gkeys = nullptr;
@@ -143,6 +150,9 @@ void clear_store(Solver& S, const SigStore& st);
 
 // Degree tiers, global-tier scratch; once per level.
 void prepare_level(Solver& S, const Level& L);
+
+// Local moving's settled-node tracking; once per solve, after setup_null_model.
+void setup_tracking(Solver& S);
 
 struct MoveOut {
   int64_t rounds = 0, moves = 0;
