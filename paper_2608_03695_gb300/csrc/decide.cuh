@@ -99,16 +99,20 @@ __host__ __device__ __forceinline__ int degree_tier(int64_t d, const TierCuts& c
 }
 
 // Aggregated nodes carry a list of (snapshot, strength) entries, and scoring
-// one candidate walks that list once (the null term sums over snapshots).
-// On long sequences late-level nodes hold thousands of entries, so a node
-// whose (degree + 1) * entries reaches SLICE_WORK_BLOCK is decided by a
-// block-per-node tier, whose threads then split each candidate's walk
-// (slice_parallel) instead of taking one candidate each.
-constexpr int64_t SLICE_WORK_BLOCK = 4096;
+// one candidate walks that list once (the null term sums over snapshots).  On
+// long sequences late-level nodes hold up to thousands of entries.  A node's
+// lookups number (degree + 1) * entries at most; from SLICE_WORK_WARP on a warp
+// decides it and from SLICE_WORK_BLOCK a block, whose threads split each
+// candidate's walk, so that no lane walks more than a few dozen entries (a node
+// just below the next tier held a sub-round for hundreds of dependent lookups).
+constexpr int64_t SLICE_WORK_WARP = 128, SLICE_WORK_BLOCK = 2048;
 
 __host__ __device__ __forceinline__ int work_tier(int64_t d, int64_t nslices, const TierCuts& c) {
   const int t = degree_tier(d, c);
-  if (t < NTIERS - 2 && nslices > 1 && (d + 1) * nslices >= SLICE_WORK_BLOCK) return NTIERS - 2;
+  if (nslices > 1 && t < NTIERS - 2) {
+    if ((d + 1) * nslices >= SLICE_WORK_BLOCK) return NTIERS - 2;
+    if ((d + 1) * nslices >= SLICE_WORK_WARP) return t > 2 ? t : 2;
+  }
   return t;
 }
 
@@ -368,6 +372,98 @@ __global__ void __launch_bounds__(GROUP_THREADS, Pol::MIN_BLOCKS)
   }
 }
 
+// Sum of one u128 per lane over aligned runs of `width` lanes (a power of two).
+__device__ __forceinline__ u128 lanes_sum_u128(u128 x, int width, unsigned mask) {
+  ull lo = (ull)x, hi = (ull)(x >> 64);
+  for (int m = width >> 1; m >= 1; m >>= 1) {
+    const ull l2 = __shfl_xor_sync(mask, lo, m), h2 = __shfl_xor_sync(mask, hi, m);
+    const ull nl = lo + l2;
+    hi += h2 + (nl < lo ? 1ull : 0ull);
+    lo = nl;
+  }
+  return ((u128)hi << 64) | lo;
+}
+
+// One node decided by a group of G lanes (gl: rank, gmask: lanes) with a table
+// of 2^BITS slots in shared memory, all free on entry and left free (CL: room
+// for half of them; ncand: 0 on entry and left 0).
+// An aggregated node's candidates each walk its (snapshot, strength) list.
+// With fewer candidates than lanes the idle lanes share the walks: `sub` lanes
+// take one candidate (the walk is a chain of dependent lookups, so this cuts
+// the node's latency by about sub).
+template <class Pol, int G, int BITS, int EPL>
+__device__ __forceinline__ void group_decide_node(const Pol& pol, int32_t v, int32_t* K, long long* V, uint16_t* CL,
+                                                  int32_t* ncand, int gl, unsigned gmask) {
+  if (!pol.begin(v)) {
+    if (gl == 0) pol.skip(v);
+    return;
+  }
+  const int64_t beg = pol.g.rowptr[v], end = pol.g.rowptr[v + 1];
+  const typename Pol::VCtx vc = pol.vctx(v);
+  for (int64_t base = beg; base < end; base += G * EPL) {
+    int32_t keys[EPL];
+    long long ws[EPL];
+    bool ok[EPL];
+#pragma unroll
+    for (int j = 0; j < EPL; ++j) {
+      const int64_t e = base + j * G + gl;
+      ok[j] = e < end && pol.edge(v, vc, e, keys[j], ws[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < EPL; ++j) {
+      if (ok[j]) {
+        bool fresh;
+        const int slot = table_add_slot(K, V, BITS, keys[j], ws[j], fresh);
+#if MSLICE_CHECKED
+        if (slot < 0) atomicOr(pol.g.chk, ERR_BOUNDS);
+#endif
+        if (fresh) CL[atomicAdd(ncand, 1)] = (uint16_t)slot;
+      }
+    }
+  }
+  __syncwarp(gmask);
+  const int n = *ncand;
+  const int32_t own = pol.own_key(v);
+  const int64_t ns = pol.slice_count(v);
+  int sub = 1;
+  while (2 * sub <= G && 2 * sub * n <= G && 2 * sub <= ns) sub *= 2;
+  Cand c{0, INT32_MAX};
+  i128 Gown = 0;
+  if (sub > 1) {
+    const int j = gl / sub, slot = j < n ? CL[j] : 0;
+    const int32_t key = j < n ? K[slot] : own;
+    const u128 ns_sum =
+        lanes_sum_u128(key != own ? pol.null_part(v, vc, key, false, gl % sub, sub) : (u128)0, sub, gmask);
+    if (key != own && gl % sub == 0) c = pol.cand_ns(v, vc, key, V[slot], ns_sum);
+  } else {
+    for (int j = gl; j < n; j += G) {
+      const int slot = CL[j];
+      const int32_t key = K[slot];
+      if (key != own) {
+        const Cand x = ns > 1 ? pol.cand_ns(v, vc, key, V[slot], pol.null_part(v, vc, key, false, 0, 1))
+                              : pol.cand(v, vc, key, V[slot], pol.probe(v, vc, key));
+        if (better(x, c)) c = x;
+      }
+    }
+  }
+  if (ns > 1 && pol.own_walks_slices()) {
+    const u128 ns_own = lanes_sum_u128(pol.null_part(v, vc, own, true, gl, G), G, gmask);
+    if (gl == 0) Gown = pol.own_ns(v, vc, table_get(K, V, BITS, own), ns_own);
+  } else if (gl == 0) {
+    Gown = pol.own(v, vc, table_get(K, V, BITS, own));
+  }
+  c = group_best<G>(c, gmask);
+  if (gl == 0) pol.finish(v, c, c.label != INT32_MAX ? table_get(K, V, BITS, c.label) : 0, Gown, vc);
+  __syncwarp(gmask);
+  for (int j = gl; j < n; j += G) {
+    const int slot = CL[j];
+    K[slot] = -1;
+    V[slot] = 0;
+  }
+  if (gl == 0) *ncand = 0;
+  __syncwarp(gmask);
+}
+
 __device__ __forceinline__ int table_bits_for_degree(int64_t deg) {
   int bits = 1;
   while ((1ll << bits) < 2 * deg) ++bits;
@@ -413,32 +509,49 @@ __device__ __forceinline__ void block_decide_node(const Pol& pol, int32_t v, int
   __syncthreads();
   const int n = *ncand;
   const int32_t own = pol.own_key(v);
-  if (slice_parallel(n, pol.slice_count(v), NT)) {
-    // every thread walks a share of the slice list for each candidate in
-    // turn; thread 0 keeps the best
+  const int64_t ns = pol.slice_count(v);
+  if (ns > 1) {
+    // The n candidates, and staying as one more, walk the node's list with `sub`
+    // threads each: all at once when they fit the block (sub > 32: whole warps,
+    // whose sums meet in usm), a thread each otherwise.
+    const bool walk_own = pol.own_walks_slices();
+    const int m = n + (walk_own ? 1 : 0);
+    int sub = 1;
+    while (2 * sub <= NT && 2 * sub * m <= NT && 2 * sub <= ns) sub *= 2;
     Cand c{0, INT32_MAX};
-    for (int j = 0; j < n; ++j) {
-      const int slot = cl[j];
-      const int32_t k = hk[slot];
-      if (k == own) continue;
-      const u128 ns =
-          block_sum_u128<NT / 32>(pol.null_part(v, vc, k, false, threadIdx.x, NT), usm);
-      if (threadIdx.x == 0) {
-        const Cand x = pol.cand_ns(v, vc, k, hv[slot], ns);
-        if (better(x, c)) c = x;
+    for (int j0 = 0; j0 < m; j0 += NT / sub) {
+      const int j = j0 + (int)threadIdx.x / sub;
+      const bool stay = j == n;
+      const int slot = j < n ? cl[j] : 0;
+      const int32_t k = j < n ? hk[slot] : own;
+      const bool walks = j < m && (stay || k != own);
+      u128 x = walks ? pol.null_part(v, vc, k, stay, threadIdx.x % sub, sub) : (u128)0;
+      x = lanes_sum_u128(x, sub < 32 ? sub : 32, 0xffffffffu);
+      if (sub > 32) {
+        const int w = threadIdx.x >> 5;
+        if ((threadIdx.x & 31) == 0) {
+          usm[2 * w] = (ull)x;
+          usm[2 * w + 1] = (ull)(x >> 64);
+        }
+        __syncthreads();
+        x = 0;
+        if (threadIdx.x % sub == 0)
+          for (int i = 0; i < sub / 32; ++i) x += ((u128)usm[2 * (w + i) + 1] << 64) | usm[2 * (w + i)];
+      }
+      if (walks && threadIdx.x % sub == 0) {
+        if (stay) {
+          *own_sm = pol.own_ns(v, vc, table_get(hk, hv, bits, own), x);
+        } else {
+          const Cand y = pol.cand_ns(v, vc, k, hv[slot], x);
+          if (better(y, c)) c = y;
+        }
       }
     }
-    i128 Go = 0;
-    if (pol.own_walks_slices()) {
-      const u128 ns =
-          block_sum_u128<NT / 32>(pol.null_part(v, vc, own, true, threadIdx.x, NT), usm);
-      if (threadIdx.x == 0) Go = pol.own_ns(v, vc, table_get(hk, hv, bits, own), ns);
-    } else if (threadIdx.x == 0) {
-      Go = pol.own(v, vc, table_get(hk, hv, bits, own));
-    }
+    if (!walk_own && threadIdx.x == 0) *own_sm = pol.own(v, vc, table_get(hk, hv, bits, own));
+    const Cand best = block_best<NT / 32>(c, red);
     if (threadIdx.x == 0) {
-      const long long Wb = c.label != INT32_MAX ? table_get(hk, hv, bits, c.label) : 0;
-      pol.finish(v, c, Wb, Go, vc);
+      const long long Wb = best.label != INT32_MAX ? table_get(hk, hv, bits, best.label) : 0;
+      pol.finish(v, best, Wb, *own_sm, vc);
     }
   } else {
     Cand c{0, INT32_MAX};
@@ -527,6 +640,67 @@ __device__ __forceinline__ void gtable_add(int32_t* hk, long long* hv, int bits,
   atomicOr(status, ERR_HASH_FULL);
 }
 
+// One node decided by a block of NT threads with its table in global scratch at
+// goff[v].
+template <class Pol, int NT>
+__device__ __forceinline__ void block_decide_scratch(const Pol& pol, int32_t v, int32_t* gkeys, long long* gvals,
+                                                     const int64_t* goff, unsigned* status, Cand* red, ull* usm,
+                                                     i128* own_sm) {
+  const typename Pol::VCtx vc = pol.vctx(v);
+  const int64_t beg = pol.g.rowptr[v], end = pol.g.rowptr[v + 1];
+  const int bits = table_bits_for_degree(end - beg);
+  const int64_t S = 1ll << bits;
+  int32_t* hk = gkeys + goff[v];
+  long long* hv = gvals + goff[v];
+  for (int64_t i = threadIdx.x; i < S; i += NT) {
+    hk[i] = -1;
+    hv[i] = 0;
+  }
+  __syncthreads();
+  for (int64_t e = beg + threadIdx.x; e < end; e += NT) {
+    int32_t key;
+    long long w;
+    if (pol.edge(v, vc, e, key, w)) gtable_add(hk, hv, bits, key, w, status);
+  }
+  __syncthreads();
+  const int32_t own = pol.own_key(v);
+  if (slice_parallel(end - beg, pol.slice_count(v), NT)) {
+    // (the degree bounds the candidates) the block splits each
+    // candidate's slice walk; thread 0 keeps the best
+    Cand c{0, INT32_MAX};
+    for (int64_t i = 0; i < S; ++i) {
+      const int32_t k = hk[i];
+      if (k < 0 || k == own) continue;
+      const u128 ns =
+          block_sum_u128<NT / 32>(pol.null_part(v, vc, k, false, threadIdx.x, NT), usm);
+      if (threadIdx.x == 0) {
+        const Cand x = pol.cand_ns(v, vc, k, hv[i], ns);
+        if (better(x, c)) c = x;
+      }
+    }
+    i128 Go = 0;
+    if (pol.own_walks_slices()) {
+      const u128 ns =
+          block_sum_u128<NT / 32>(pol.null_part(v, vc, own, true, threadIdx.x, NT), usm);
+      if (threadIdx.x == 0) Go = pol.own_ns(v, vc, table_get(hk, hv, bits, own), ns);
+    } else if (threadIdx.x == 0) {
+      Go = pol.own(v, vc, table_get(hk, hv, bits, own));
+    }
+    if (threadIdx.x == 0) {
+      const long long Wb = c.label != INT32_MAX ? table_get(hk, hv, bits, c.label) : 0;
+      pol.finish(v, c, Wb, Go, vc);
+    }
+  } else {
+    if (threadIdx.x == 0) *own_sm = pol.own(v, vc, table_get(hk, hv, bits, own));
+    const Cand best = block_best<NT / 32>(score_range(pol, v, vc, own, hk, hv, S), red);
+    if (threadIdx.x == 0) {
+      const long long Wb = best.label != INT32_MAX ? table_get(hk, hv, bits, best.label) : 0;
+      pol.finish(v, best, Wb, *own_sm, vc);
+    }
+  }
+  __syncthreads();
+}
+
 // Tier 4: one block of NT threads per node.  A node whose table fits
 // 2^TIER4_SMEM_BITS slots (degree up to 4096) keeps it in dynamic shared
 // memory (one block per SM), as tier 3 does; a larger one uses global
@@ -564,59 +738,7 @@ __global__ void __launch_bounds__(NT) k_decide_global(Pol pol, const int32_t* li
       block_decide_node<Pol, NT>(pol, v, shk, shv, scl, &ncand, red, usm, &own_sm);
       continue;
     }
-    const typename Pol::VCtx vc = pol.vctx(v);
-    const int64_t beg = pol.g.rowptr[v], end = pol.g.rowptr[v + 1];
-    const int bits = table_bits_for_degree(end - beg);
-    const int64_t S = 1ll << bits;
-    int32_t* hk = gkeys + goff[v];
-    long long* hv = gvals + goff[v];
-    for (int64_t i = threadIdx.x; i < S; i += NT) {
-      hk[i] = -1;
-      hv[i] = 0;
-    }
-    __syncthreads();
-    for (int64_t e = beg + threadIdx.x; e < end; e += NT) {
-      int32_t key;
-      long long w;
-      if (pol.edge(v, vc, e, key, w)) gtable_add(hk, hv, bits, key, w, status);
-    }
-    __syncthreads();
-    const int32_t own = pol.own_key(v);
-    if (slice_parallel(end - beg, pol.slice_count(v), NT)) {
-      // (the degree bounds the candidates) the block splits each
-      // candidate's slice walk; thread 0 keeps the best
-      Cand c{0, INT32_MAX};
-      for (int64_t i = 0; i < S; ++i) {
-        const int32_t k = hk[i];
-        if (k < 0 || k == own) continue;
-        const u128 ns =
-            block_sum_u128<NT / 32>(pol.null_part(v, vc, k, false, threadIdx.x, NT), usm);
-        if (threadIdx.x == 0) {
-          const Cand x = pol.cand_ns(v, vc, k, hv[i], ns);
-          if (better(x, c)) c = x;
-        }
-      }
-      i128 Go = 0;
-      if (pol.own_walks_slices()) {
-        const u128 ns =
-            block_sum_u128<NT / 32>(pol.null_part(v, vc, own, true, threadIdx.x, NT), usm);
-        if (threadIdx.x == 0) Go = pol.own_ns(v, vc, table_get(hk, hv, bits, own), ns);
-      } else if (threadIdx.x == 0) {
-        Go = pol.own(v, vc, table_get(hk, hv, bits, own));
-      }
-      if (threadIdx.x == 0) {
-        const long long Wb = c.label != INT32_MAX ? table_get(hk, hv, bits, c.label) : 0;
-        pol.finish(v, c, Wb, Go, vc);
-      }
-    } else {
-      if (threadIdx.x == 0) own_sm = pol.own(v, vc, table_get(hk, hv, bits, own));
-      const Cand best = block_best<NT / 32>(score_range(pol, v, vc, own, hk, hv, S), red);
-      if (threadIdx.x == 0) {
-        const long long Wb = best.label != INT32_MAX ? table_get(hk, hv, bits, best.label) : 0;
-        pol.finish(v, best, Wb, own_sm, vc);
-      }
-    }
-    __syncthreads();
+    block_decide_scratch<Pol, NT>(pol, v, gkeys, gvals, goff, status, red, usm, &own_sm);
   }
 }
 

@@ -1,0 +1,355 @@
+// Resident rounds of local moving: one cooperative launch runs a level's rounds
+// until nothing moves (or the host has to step in), with grid barriers where
+// the host-driven rounds of local_move.cu have kernel boundaries.
+//
+// A host-driven round is about 28 launches and a synchronisation, 160 us however
+// little there is to decide; most rounds of most levels (all of a small graph's,
+// and the pruned tail of a large level) have a few microseconds of work.  Here a
+// round costs 2K + 1 grid barriers.  The price is occupancy: every degree tier
+// is decided by the same blocks of 512 threads, one per SM (their tables take
+// 107 KB of shared memory), which keeps fewer nodes in flight than the tiers'
+// own kernels; rounds with more than RESIDENT_MAX_WORK to decide
+// are left to those (see local_move()).
+//
+// Double buffering by the round's parity replaces the clearing launches: lists'
+// lengths, move counts and tracking words of the other parity are cleared by
+// block 0 between the round's first and second barrier, when every block has
+// read what it needs of them.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "../../include/mslice.h"
+#include "lm.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace mslice {
+
+namespace {
+
+constexpr int RT = 512;              // threads per block
+constexpr int RW = RT / 32;
+constexpr int R_SLOTS = TIER4_SMEM_SLOTS;  // table slots per block: 512 per warp
+constexpr int R_PER_WARP = R_SLOTS / RW;
+constexpr int R_BUCKET_ITEMS = 4;
+static_assert(R_PER_WARP == 1 << T2_BITS, "a warp's share of the block's table is tier 2's table");
+
+// Device words of a launch.
+struct ResidentCtl {
+  ull moved[2];            // moves of the round, by parity (moves to empty communities apart)
+  int32_t empties[2][64];  // moves to empty communities per sub-round
+  // results
+  long long rounds, moves, last_moved, last_listed;
+};
+
+struct ResidentArgs {
+  LevelDev g;
+  int32_t *labels, *size, *target;
+  SigStore sig;
+  const uint8_t* tier;
+  uint16_t* seg;
+  int32_t* lists;
+  int64_t row_stride;
+  TierOff off;
+  int32_t* cursors;    // 2 x K x NTIERS
+  int32_t* inst_moved; // 2 x B (nullptr: single solve)
+  int32_t* lm_active;
+  const int32_t* active;
+  int32_t B;
+  TrackView trk;       // of even rounds
+  int32_t Tn;
+  int32_t mode_init, first;      // first: the level's first round is this launch's
+  long long prev_moved, prev_listed;  // of the round before this launch
+  uint64_t seed, it, lvl;
+  int32_t r0, r_end, K;
+  long long max_listed;          // leave after a round that listed more nodes
+  int32_t *gkeys;
+  long long* gvals;
+  const int64_t* goff;
+  unsigned* status;
+  const ull* sig_used;           // nullptr: dense tables
+  int32_t *blk, *freelist, *mrank, *icnt;
+  ResidentCtl* ctl;
+};
+
+__device__ __forceinline__ void resident_bar() {
+  if (gridDim.x == 1)
+    __syncthreads();
+  else
+    cg::this_grid().sync();
+}
+
+// Lists the nodes that decide in this round (one block's share at a time:
+// segments counted in shared memory, one reservation per block and segment).
+__device__ __forceinline__ void resident_bucket(const ResidentArgs& a, const TrackView& trk, bool prune,
+                                                const int32_t* prev_moved, const BucketLists& bl, uint64_t r,
+                                                int32_t* cnt, int32_t* base) {
+  const int nseg = a.K * NTIERS;
+  const int64_t chunk = (int64_t)RT * R_BUCKET_ITEMS;
+  int settled = 0;
+  for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < a.g.N; c0 += (int64_t)gridDim.x * chunk) {
+    for (int i = threadIdx.x; i < nseg; i += RT) cnt[i] = 0;
+    __syncthreads();
+    int sg[R_BUCKET_ITEMS], rank[R_BUCKET_ITEMS];
+#pragma unroll
+    for (int k = 0; k < R_BUCKET_ITEMS; ++k) {
+      const int64_t v = c0 + (int64_t)k * RT + threadIdx.x;
+      sg[k] = SEG_FROZEN;
+      if (v >= a.g.N) continue;
+      const bool idle = prev_moved && !prev_moved[node_inst(a.g, (int32_t)v)];
+      int s = idle ? (int)SEG_FROZEN
+                   : bucket_seg(a.g, a.tier, a.seed, 0, a.it, a.lvl, r, a.K, a.active, v);
+      if (prune && s < nseg && track_settled(trk, a.g, (int32_t)v)) {
+        s |= SEG_SETTLED;
+        ++settled;
+      }
+      a.seg[v] = (uint16_t)s;
+      sg[k] = s;
+      if (s < nseg) rank[k] = atomicAdd(&cnt[s], 1);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nseg; i += RT) base[i] = cnt[i] ? atomicAdd(&bl.cursors[i], cnt[i]) : 0;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < R_BUCKET_ITEMS; ++k)
+      if (sg[k] < nseg) {
+        const int q = sg[k] / NTIERS, t = sg[k] % NTIERS;
+        bl.lists[(int64_t)q * bl.row_stride + bl.off.off[t] + base[sg[k]] + rank[k]] =
+            (int32_t)(c0 + (int64_t)k * RT + threadIdx.x);
+      }
+    __syncthreads();
+  }
+  if (prune) {
+    settled = warp_sum(settled);
+    if ((threadIdx.x & 31) == 0 && settled) atomicAdd(&trk.state[TRACK_SETTLED], settled);
+  }
+}
+
+template <class Pol>
+__global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  long long* hv = reinterpret_cast<long long*>(smem);
+  int32_t* hk = reinterpret_cast<int32_t*>(smem + R_SLOTS * sizeof(long long));
+  uint16_t* cl = reinterpret_cast<uint16_t*>(smem + R_SLOTS * (sizeof(long long) + sizeof(int32_t)));
+  __shared__ int32_t ncand[RW * 4];
+  __shared__ int32_t block_ncand;
+  __shared__ Cand red[RW];
+  __shared__ ull usm[2 * RW];
+  __shared__ i128 own_sm;
+  __shared__ int32_t seg_cnt[64 * NTIERS], seg_base[64 * NTIERS];
+  __shared__ int32_t mode_sh;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < R_SLOTS; i += RT) {
+    hk[i] = -1;
+    hv[i] = 0;
+  }
+  for (int i = threadIdx.x; i < RW * 4; i += RT) ncand[i] = 0;
+  if (threadIdx.x == 0) block_ncand = 0;
+  const int nseg = a.K * NTIERS;
+  long long moved = a.prev_moved, listed = a.prev_listed, moves = 0;
+  int32_t r = a.r0;
+  for (;;) {
+    const int p = r & 1;
+    TrackView trk = a.trk;
+    int32_t mode = TRACK_OFF;
+    if (a.trk.state) {
+      trk.state = a.trk.state + p * TRACK_WORDS;
+      trk.E = a.trk.E + (int64_t)p * a.Tn;
+      trk.B = a.trk.B + (int64_t)p * a.Tn;
+      trk.Ep = a.trk.E + (int64_t)(1 - p) * a.Tn;
+      trk.Bp = a.trk.B + (int64_t)(1 - p) * a.Tn;
+      if (threadIdx.x == 0) {
+        const TrackState st =
+            track_next(a.trk.state + (1 - p) * TRACK_WORDS, a.first && r == a.r0, a.mode_init, moved, listed);
+        mode_sh = st.mode;
+        if (blockIdx.x == 0) track_store(trk.state, st);
+      }
+      __syncthreads();
+      mode = mode_sh;
+      track_budgets(trk, mode, a.Tn, blockIdx.x * RT + threadIdx.x, gridDim.x * RT);
+    }
+    const BucketLists bl{a.lists, a.row_stride, a.cursors + p * nseg, a.off, a.seg};
+    const bool first_here = r == a.r0;
+    resident_bucket(a, trk, mode == TRACK_PRUNE,
+                    a.inst_moved && !first_here ? a.inst_moved + (1 - p) * a.B : nullptr, bl, (uint64_t)r, seg_cnt,
+                    seg_base);
+    resident_bar();
+    pol.trk = trk;
+    if (blockIdx.x == 0) {
+      // the other parity's words: read by every block before the barrier above
+      if (a.inst_moved)
+        for (int32_t i = threadIdx.x; i < a.B; i += RT) {
+          if (!first_here && !a.inst_moved[(1 - p) * a.B + i]) a.lm_active[i] = 0;
+          a.inst_moved[(1 - p) * a.B + i] = 0;
+        }
+      for (int i = threadIdx.x; i < nseg; i += RT) a.cursors[(1 - p) * nseg + i] = 0;
+      for (int i = threadIdx.x; i < a.K; i += RT) a.ctl->empties[1 - p][i] = 0;
+      if (threadIdx.x == 0) {
+        a.ctl->moved[1 - p] = 0;
+        if (a.trk.state)
+          a.trk.state[(1 - p) * TRACK_WORDS + TRACK_PAST] = a.trk.state[(1 - p) * TRACK_WORDS + TRACK_SETTLED] = 0;
+      }
+    }
+    for (int q = 0; q < a.K; ++q) {
+      TierSegs sg;
+#pragma unroll
+      for (int t = 0; t < NTIERS; ++t) {
+        sg.list[t] = a.lists + (int64_t)q * a.row_stride + a.off.off[t];
+        sg.count[t] = bl.cursors + q * NTIERS + t;
+      }
+      // ---- decisions: a block per node of tiers 4 and 3, a warp of tier 2, 8
+      // lanes of tiers 1 and 0 (the last blocks take the first of the short ones)
+      for (int t = NTIERS - 1; t >= NTIERS - 2; --t) {
+        const int n = *sg.count[t];
+        for (int i = blockIdx.x; i < n; i += gridDim.x) {
+          const int32_t v = sg.list[t][i];
+          __syncthreads();
+          if (table_bits_for_degree(a.g.rowptr[v + 1] - a.g.rowptr[v]) <= TIER4_SMEM_BITS)
+            block_decide_node<Pol, RT>(pol, v, hk, hv, cl, &block_ncand, red, usm, &own_sm);
+          else
+            block_decide_scratch<Pol, RT>(pol, v, a.gkeys, a.gvals, a.goff, a.status, red, usm, &own_sm);
+        }
+      }
+      __syncthreads();
+      const int gw = (gridDim.x - 1 - blockIdx.x) * RW + w, warps = gridDim.x * RW;
+      {
+        const int n = *sg.count[2];
+        for (int i = gw; i < n; i += warps)
+          group_decide_node<Pol, 32, T2_BITS, 2>(pol, sg.list[2][i], hk + w * R_PER_WARP, hv + w * R_PER_WARP,
+                                                 cl + w * (R_PER_WARP / 2), &ncand[w * 4], lane, 0xffffffffu);
+      }
+      {
+        const int n0 = *sg.count[0], n = n0 + *sg.count[1];
+        const int gi = lane >> 3, gl = lane & 7;
+        const unsigned gmask = 0xffu << (gi * 8);
+        const int o = w * R_PER_WARP + gi * 64, oc = w * (R_PER_WARP / 2) + gi * 32;
+        for (int i = gw * 4 + gi; i < n; i += warps * 4)
+          group_decide_node<Pol, 8, 6, 4>(pol, i < n0 ? sg.list[0][i] : sg.list[1][i - n0], hk + o, hv + o, cl + oc,
+                                          &ncand[w * 4 + gi], gl, gmask);
+        __syncwarp();
+      }
+      resident_bar();
+      lm_apply(a.g, sg, a.labels, a.size, a.sig, a.target, &a.ctl->moved[p], &a.ctl->empties[p][q],
+               a.inst_moved ? a.inst_moved + p * a.B : nullptr, trk, bl, q);
+      resident_bar();
+      const bool past = mode == TRACK_PRUNE && trk.state[TRACK_PAST];
+      const bool empties = a.ctl->empties[p][q] > 0;
+      if (past) track_rescan(trk, a.g, bl, q + 1);
+      if (empties)
+        lm_empty(a.g, a.B, a.target, a.labels, a.size, a.sig, a.blk, a.freelist, a.mrank, a.icnt,
+                 [] { resident_bar(); });
+      else if (past)
+        resident_bar();
+    }
+    // ---- end of the round (every block reads the same words; nobody writes
+    // them before the next round's first barrier)
+    moved = (long long)a.ctl->moved[p];
+    for (int q = 0; q < a.K; ++q) moved += a.ctl->empties[p][q];
+    listed = 0;
+    for (int i = 0; i < nseg; ++i) listed += bl.cursors[i];
+    moves += moved;
+    ++r;
+    if (moved == 0 || r >= a.r_end || listed > a.max_listed || (a.sig_used && *a.sig_used) || *a.status) break;
+  }
+  if (blockIdx.x == 0) {
+    if (a.inst_moved) {
+      const int p = (r - 1) & 1;
+      for (int32_t i = threadIdx.x; i < a.B; i += RT) {
+        if (!a.inst_moved[p * a.B + i]) a.lm_active[i] = 0;
+        a.inst_moved[p * a.B + i] = 0;
+      }
+    }
+    if (threadIdx.x == 0) {
+      a.ctl->rounds = r - a.r0;
+      a.ctl->moves = moves;
+      a.ctl->last_moved = moved;
+      a.ctl->last_listed = listed;
+    }
+  }
+}
+
+template <class Pol>
+void launch_rounds(Ctx& c, const Pol& pol, const ResidentArgs& a, int32_t N, int32_t big, int32_t sms) {
+  const size_t bytes = TIER4_SMEM_BYTES;
+  check_cuda(cudaFuncSetAttribute(k_lm_rounds<Pol>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
+             "resident rounds' shared memory");
+  // a block or a warp per node of a sub-round, up to one block per SM: fewer
+  // blocks make the barriers cheaper
+  const int64_t blocks = ((int64_t)big + a.K - 1) / a.K, warps = ((int64_t)(N - big) + a.K - 1) / a.K;
+  const int64_t want = blocks + (warps + RW - 1) / RW;
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, sms));
+  launch_coop(c, k_lm_rounds<Pol>, dim3(grid), dim3(RT), bytes, pol, a);
+}
+
+}  // namespace
+
+void resident_rounds(Solver& S, const Level& L, int32_t* labels, int it, int lvl, const TrackView& trk,
+                     const ResidentIn& in, const int32_t* active, ResidentOut& out) {
+  Ctx& c = *S.c;
+  ResidentArgs a{};
+  a.g = L.d;
+  a.labels = labels;
+  a.size = S.size;
+  a.target = S.target;
+  a.sig = S.sig;
+  a.tier = S.tier;
+  a.seg = S.bseg;
+  a.lists = S.lists;
+  a.row_stride = S.N0;
+  a.off = tier_offsets(S);
+  a.cursors = S.cursors;
+  a.inst_moved = S.B > 1 ? S.inst_moved : nullptr;
+  a.lm_active = S.lm_active;
+  a.active = active;
+  a.B = S.B;
+  a.trk = trk;
+  a.Tn = S.Tn;
+  a.mode_init = in.mode_init;
+  a.first = in.first ? 1 : 0;
+  a.prev_moved = in.prev_moved;
+  a.prev_listed = in.prev_listed;
+  a.seed = S.p.seed;
+  a.it = (uint64_t)it;
+  a.lvl = (uint64_t)lvl;
+  a.r0 = in.r;
+  a.r_end = in.r_end;
+  a.K = S.p.K;
+  a.max_listed = in.max_listed;
+  a.gkeys = S.gkeys;
+  a.gvals = S.gvals;
+  a.goff = S.goff;
+  a.status = c.d_status;
+  a.sig_used = S.sig.d ? nullptr : S.sig_used;
+  a.blk = S.empty_blk;
+  a.freelist = S.freelist;
+  a.mrank = S.tmp32b;
+  a.icnt = S.inst_cnt;
+  a.ctl = reinterpret_cast<ResidentCtl*>(c.ws->get_bytes("s_resident", sizeof(ResidentCtl)));
+  check_cuda(cudaMemsetAsync(a.ctl, 0, sizeof(ResidentCtl), c.stream), "memset");
+  check_cuda(cudaMemsetAsync(S.cursors, 0, 2 * (size_t)S.p.K * NTIERS * sizeof(int32_t), c.stream), "memset");
+  if (S.sig.d)
+    launch_rounds(c, lm_policy<true>(S, L, labels, trk), a, L.d.N, S.tier_cnt[3] + S.tier_cnt[4], S.sms);
+  else
+    launch_rounds(c, lm_policy<false>(S, L, labels, trk), a, L.d.N, S.tier_cnt[3] + S.tier_cnt[4], S.sms);
+  char* h = static_cast<char*>(c.pinned);
+  check_cuda(cudaMemcpyAsync(h, &a.ctl->rounds, 4 * sizeof(long long), cudaMemcpyDeviceToHost, c.stream), "copy");
+  check_cuda(cudaMemcpyAsync(h + 32, S.sig_used, sizeof(ull), cudaMemcpyDeviceToHost, c.stream), "copy");
+  check_cuda(cudaMemcpyAsync(h + 40, c.d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream), "copy");
+  sync(c);
+  struct {
+    long long rounds, moves, last_moved, last_listed;
+    ull used;
+    unsigned status;
+  } rb;
+  std::memcpy(&rb, h, sizeof(rb));
+  out.rounds = rb.rounds;
+  out.moves = rb.moves;
+  out.last_moved = rb.last_moved;
+  out.last_listed = rb.last_listed;
+  out.used = rb.used;
+  out.status = rb.status;
+}
+
+}  // namespace mslice

@@ -16,8 +16,7 @@
 // W(R,C\R) is maintained incrementally: when the set M of nodes joins R,
 //   W(R u M, C\(R u M)) = W(R,C\R) + sum_{v in M} [W(v,C\v) - 2 W(v,R)]
 //                         - sum_{v in M} W(v, M\v).
-#include "decide.cuh"
-#include "solver.h"
+#include "lm.cuh"
 
 namespace mslice {
 
@@ -222,16 +221,7 @@ struct RefPolicy {
   __device__ int64_t slice_count(int32_t v) const { return g.is0 ? 0 : g.sptr[v + 1] - g.sptr[v]; }
   __device__ bool own_walks_slices() const { return false; }
   __device__ u128 null_part(int32_t v, const VCtx&, int32_t X, bool, int t, int nt) const {
-    int64_t b, e;
-    slice_range(g, v, b, e);
-    u128 acc = 0;
-    for (int64_t j = b + t; j < e; j += nt) {
-      int32_t s;
-      long long k;
-      slice_entry(g, v, j, s, k);
-      acc += lam_k_x(lam, s, k, sst_get<DENSE>(kr, X, s));
-    }
-    return acc;
+    return null_sum_part<DENSE>(g, lam, kr, v, X, false, t, nt);
   }
   __device__ Cand cand_ns(int32_t, const VCtx& vc, int32_t X, long long W, const u128& ns) const {
     const unsigned long long d = desc[X];
@@ -835,8 +825,7 @@ unsigned fixed_grid(int per_sm) { return 152u * (unsigned)per_sm; }
 
 }  // namespace
 
-void bucket(Solver& S, const Level& L, uint64_t tag, int it, int lvl, int r, const int32_t* active,
-            const int32_t* r_dev = nullptr);
+void bucket(Solver& S, const Level& L, uint64_t tag, int it, int lvl, int r, const int32_t* active);
 TierSegs bucket_segments(Solver& S, int q);
 
 // Launches the randomised decisions of one sub-round: the tiers decide

@@ -75,11 +75,12 @@ struct Solver {
   uint8_t* tier = nullptr;
   uint8_t* cls = nullptr;       // refinement class of every node of the level
   int32_t* lists = nullptr;     // K rows of N0 entries: nodes bucketed by class and tier
-  int32_t* cursors = nullptr;   // bucket sizes per (class, tier) segment (device)
+  int32_t* cursors = nullptr;   // bucket sizes per (class, tier) segment (device; two sets: resident rounds)
   uint16_t* bseg = nullptr;     // segment of every node in the round being bucketed
   int32_t* bcounts = nullptr;   // per segment and chunk of nodes: counts, then offsets
   int32_t* counters = nullptr;  // [0] moves in round (low), [1] moves (high), [2] moves to empty in sub-round
   ull* sig_used = nullptr;      // Sigma slots taken since its last rebuild
+  int32_t sms = 1;              // multiprocessors of the device
   int32_t empty_grid = 0;       // co-resident grid of the empty-community pass
   int32_t* empty_blk = nullptr;
   int32_t* inst_cnt = nullptr;  // per-instance counts of the empty-community pass
@@ -91,9 +92,7 @@ struct Solver {
   long long *gn_d = nullptr, *gd_d = nullptr, *on_d = nullptr, *od_d = nullptr;
   int32_t* inst_active = nullptr;  // per instance: 1 while not converged (nullptr: all active)
   int32_t* lm_active = nullptr;    // per instance: still moving in this level's local moving
-  int32_t* inst_moved = nullptr;   // per instance: moved in the current round
-  int32_t* round_dev = nullptr;    // the round the device-side round loop is at
-  long long* loop_acc = nullptr;   // device-side round loop: rounds run, moves, moves of the last round
+  int32_t* inst_moved = nullptr;   // per instance: moved in the current round (two sets: resident rounds)
   // tracking of settled nodes (track.cuh): smallest budget per null slice, the
   // strength of all nodes in units of 1/od, and whether the solve started from
   // given labels

@@ -58,7 +58,7 @@ enum {
   TRACK_NEXT_PAUSE = 4,  // length of the next pause
   TRACK_MOVED = 5,       // moves of the round before the last
   TRACK_PAUSE_MOVED = 6, // moves of the round that started the pause
-  TRACK_WORDS = 7
+  TRACK_WORDS = 8
 };
 
 struct TrackView {
@@ -66,8 +66,9 @@ struct TrackView {
   long long* slack = nullptr;     // margins in units of 2^-F weight units, net of the round's budgets
   long long* E = nullptr;         // per null slice: strength moved in this round
   long long* B = nullptr;         // per null slice: budget of this round
+  const long long* Ep = nullptr;  // the same of the round before (rounds alternate between two sets)
+  const long long* Bp = nullptr;
   const long long* base = nullptr;  // per null slice: smallest budget
-  double* drate = nullptr;        // per null slice: margin per unit of nd*k that the round's new budget costs
   const u128* lam = nullptr;
   int F = 0;                      // margin unit: 2^-F weight units
   double scale = 0;               // 2^(F-63): margin units per 2^64 of key, doubled
@@ -79,7 +80,7 @@ __device__ __forceinline__ int32_t track_mode(const TrackView& t) { return t.sta
 // the node past every rounding of the products that made it (relative 2^-53
 // each).
 __device__ __forceinline__ long long track_cost(double xp, double xn) {
-  const double up = xp * (1.0 + 0x1p-40) + 1.0, down = xn * (1.0 - 0x1p-40) - 1.0;
+  const double up = xp > 0 ? xp * (1.0 + 0x1p-40) + 1.0 : 0.0, down = xn * (1.0 - 0x1p-40) - 1.0;
   const long long c = up >= 0x1p60 ? 1ll << 60 : (long long)ceil(up);
   const long long d = down >= 0x1p60 ? 1ll << 60 : down > 0 ? (long long)down : 0;
   return c - d;
@@ -128,8 +129,23 @@ __device__ __forceinline__ void track_record(const TrackView& t, const LevelDev&
   t.slack[v] = m;
 }
 
-// Round start: charges the node's margin with the change of the budgets
-// (drate) and says whether the node is settled for the round.
+// A round's budget of a null slice: half of what moved in the round before
+// (movement mostly falls faster than that), and the smallest budget.
+__device__ __forceinline__ long long track_budget(const TrackView& t, int32_t s) { return t.Ep[s] / 2 + t.base[s]; }
+
+// Round start: the budgets of slices first, first + step, ...; nothing has
+// moved yet.
+__device__ __forceinline__ void track_budgets(const TrackView& t, int32_t mode, int32_t Tn, int32_t first,
+                                              int32_t step) {
+  if (mode == TRACK_OFF) return;
+  for (int32_t s = first; s < Tn; s += step) {
+    t.E[s] = 0;
+    t.B[s] = mode == TRACK_RECORD ? t.base[s] : track_budget(t, s);
+  }
+}
+
+// Round start: charges the node's margin with the last round's movement and the
+// change of the budgets, and says whether the node is settled for the round.
 __device__ __forceinline__ bool track_settled(const TrackView& t, const LevelDev& g, int32_t v) {
   long long m = t.slack[v];
   if (m < 0) return false;
@@ -140,12 +156,13 @@ __device__ __forceinline__ bool track_settled(const TrackView& t, const LevelDev
     int32_t s;
     long long k;
     slice_entry(g, v, j, s, k);
-    x += (double)k * t.drate[s];
+    // (a budget that shrinks is not credited: the cap of a node alone in its
+    // community has to hold)
+    const long long grown = t.Ep[s] + track_budget(t, s) - t.Bp[s];
+    if (grown > 0) x += (double)t.lam[s] * (double)k * (double)grown;
   }
-  // (a budget that shrinks is not credited: the cap of a node alone in its
-  // community has to hold)
   if (x > 0) {
-    m -= track_cost(x * (double)null_scale(g, node_omega(g, v)), 0.0);
+    m -= track_cost(x * (double)null_scale(g, node_omega(g, v)) * t.scale, 0.0);
     if (m < 0) m = TRACK_DEAD;
     t.slack[v] = m;
   }
