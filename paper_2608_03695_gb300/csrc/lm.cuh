@@ -616,6 +616,11 @@ inline TrackView track_at(const TrackView& trk, int32_t Tn, int r) {
   return t;
 }
 
+// Work to decide in a round (entries, and a node counted as so many) up to
+// which rounds are resident, and the same for a level's refinement.
+constexpr int64_t RESIDENT_MAX_WORK = (int64_t)1 << 22, RESIDENT_NODE_WORK = 16;
+constexpr int64_t RESIDENT_REFINE_WORK = (int64_t)1 << 21;
+
 // Rounds in one launch (lm_rounds.cu): from round r, up to r_end, while nodes
 // move, no hash region needs a rebuild and no round lists more than max_listed
 // nodes.  Synchronises.

@@ -15,26 +15,14 @@
 // lengths, move counts and tracking words of the other parity are cleared by
 // block 0 between the round's first and second barrier, when every block has
 // read what it needs of them.
-#include <cooperative_groups.h>
-
-#include <algorithm>
 #include <cstring>
 
 #include "../../include/mslice.h"
-#include "lm.cuh"
-
-namespace cg = cooperative_groups;
+#include "resident.cuh"
 
 namespace mslice {
 
 namespace {
-
-constexpr int RT = 512;              // threads per block
-constexpr int RW = RT / 32;
-constexpr int R_SLOTS = TIER4_SMEM_SLOTS;  // table slots per block: 512 per warp
-constexpr int R_PER_WARP = R_SLOTS / RW;
-constexpr int R_BUCKET_ITEMS = 4;
-static_assert(R_PER_WARP == 1 << T2_BITS, "a warp's share of the block's table is tier 2's table");
 
 // Device words of a launch.
 struct ResidentCtl {
@@ -73,59 +61,6 @@ struct ResidentArgs {
   int32_t *blk, *freelist, *mrank, *icnt;
   ResidentCtl* ctl;
 };
-
-__device__ __forceinline__ void resident_bar() {
-  if (gridDim.x == 1)
-    __syncthreads();
-  else
-    cg::this_grid().sync();
-}
-
-// Lists the nodes that decide in this round (one block's share at a time:
-// segments counted in shared memory, one reservation per block and segment).
-__device__ __forceinline__ void resident_bucket(const ResidentArgs& a, const TrackView& trk, bool prune,
-                                                const int32_t* prev_moved, const BucketLists& bl, uint64_t r,
-                                                int32_t* cnt, int32_t* base) {
-  const int nseg = a.K * NTIERS;
-  const int64_t chunk = (int64_t)RT * R_BUCKET_ITEMS;
-  int settled = 0;
-  for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < a.g.N; c0 += (int64_t)gridDim.x * chunk) {
-    for (int i = threadIdx.x; i < nseg; i += RT) cnt[i] = 0;
-    __syncthreads();
-    int sg[R_BUCKET_ITEMS], rank[R_BUCKET_ITEMS];
-#pragma unroll
-    for (int k = 0; k < R_BUCKET_ITEMS; ++k) {
-      const int64_t v = c0 + (int64_t)k * RT + threadIdx.x;
-      sg[k] = SEG_FROZEN;
-      if (v >= a.g.N) continue;
-      const bool idle = prev_moved && !prev_moved[node_inst(a.g, (int32_t)v)];
-      int s = idle ? (int)SEG_FROZEN
-                   : bucket_seg(a.g, a.tier, a.seed, 0, a.it, a.lvl, r, a.K, a.active, v);
-      if (prune && s < nseg && track_settled(trk, a.g, (int32_t)v)) {
-        s |= SEG_SETTLED;
-        ++settled;
-      }
-      a.seg[v] = (uint16_t)s;
-      sg[k] = s;
-      if (s < nseg) rank[k] = atomicAdd(&cnt[s], 1);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nseg; i += RT) base[i] = cnt[i] ? atomicAdd(&bl.cursors[i], cnt[i]) : 0;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < R_BUCKET_ITEMS; ++k)
-      if (sg[k] < nseg) {
-        const int q = sg[k] / NTIERS, t = sg[k] % NTIERS;
-        bl.lists[(int64_t)q * bl.row_stride + bl.off.off[t] + base[sg[k]] + rank[k]] =
-            (int32_t)(c0 + (int64_t)k * RT + threadIdx.x);
-      }
-    __syncthreads();
-  }
-  if (prune) {
-    settled = warp_sum(settled);
-    if ((threadIdx.x & 31) == 0 && settled) atomicAdd(&trk.state[TRACK_SETTLED], settled);
-  }
-}
 
 template <class Pol>
 __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
@@ -172,9 +107,24 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
     }
     const BucketLists bl{a.lists, a.row_stride, a.cursors + p * nseg, a.off, a.seg};
     const bool first_here = r == a.r0;
-    resident_bucket(a, trk, mode == TRACK_PRUNE,
-                    a.inst_moved && !first_here ? a.inst_moved + (1 - p) * a.B : nullptr, bl, (uint64_t)r, seg_cnt,
-                    seg_base);
+    const bool prune = mode == TRACK_PRUNE;
+    const int32_t* prev_moved = a.inst_moved && !first_here ? a.inst_moved + (1 - p) * a.B : nullptr;
+    int settled = 0;
+    resident_list(a.g.N, nseg, a.lists, a.row_stride, a.off, bl.cursors, seg_cnt, seg_base, [&](int32_t v) {
+      int s = prev_moved && !prev_moved[node_inst(a.g, v)]
+                  ? (int)SEG_FROZEN
+                  : bucket_seg(a.g, a.tier, a.seed, 0, a.it, a.lvl, (uint64_t)r, a.K, a.active, v);
+      if (prune && s < nseg && track_settled(trk, a.g, v)) {
+        s |= SEG_SETTLED;
+        ++settled;
+      }
+      a.seg[v] = (uint16_t)s;
+      return s;
+    });
+    if (prune) {
+      settled = warp_sum(settled);
+      if (lane == 0 && settled) atomicAdd(&trk.state[TRACK_SETTLED], settled);
+    }
     resident_bar();
     pol.trk = trk;
     if (blockIdx.x == 0) {
@@ -193,43 +143,24 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
       }
     }
     for (int q = 0; q < a.K; ++q) {
-      TierSegs sg;
-#pragma unroll
-      for (int t = 0; t < NTIERS; ++t) {
-        sg.list[t] = a.lists + (int64_t)q * a.row_stride + a.off.off[t];
-        sg.count[t] = bl.cursors + q * NTIERS + t;
-      }
-      // ---- decisions: a block per node of tiers 4 and 3, a warp of tier 2, 8
-      // lanes of tiers 1 and 0 (the last blocks take the first of the short ones)
-      for (int t = NTIERS - 1; t >= NTIERS - 2; --t) {
-        const int n = *sg.count[t];
-        for (int i = blockIdx.x; i < n; i += gridDim.x) {
-          const int32_t v = sg.list[t][i];
-          __syncthreads();
-          if (table_bits_for_degree(a.g.rowptr[v + 1] - a.g.rowptr[v]) <= TIER4_SMEM_BITS)
-            block_decide_node<Pol, RT>(pol, v, hk, hv, cl, &block_ncand, red, usm, &own_sm);
-          else
-            block_decide_scratch<Pol, RT>(pol, v, a.gkeys, a.gvals, a.goff, a.status, red, usm, &own_sm);
-        }
-      }
-      __syncthreads();
-      const int gw = (gridDim.x - 1 - blockIdx.x) * RW + w, warps = gridDim.x * RW;
-      {
-        const int n = *sg.count[2];
-        for (int i = gw; i < n; i += warps)
-          group_decide_node<Pol, 32, T2_BITS, 2>(pol, sg.list[2][i], hk + w * R_PER_WARP, hv + w * R_PER_WARP,
-                                                 cl + w * (R_PER_WARP / 2), &ncand[w * 4], lane, 0xffffffffu);
-      }
-      {
-        const int n0 = *sg.count[0], n = n0 + *sg.count[1];
-        const int gi = lane >> 3, gl = lane & 7;
-        const unsigned gmask = 0xffu << (gi * 8);
-        const int o = w * R_PER_WARP + gi * 64, oc = w * (R_PER_WARP / 2) + gi * 32;
-        for (int i = gw * 4 + gi; i < n; i += warps * 4)
-          group_decide_node<Pol, 8, 6, 4>(pol, i < n0 ? sg.list[0][i] : sg.list[1][i - n0], hk + o, hv + o, cl + oc,
-                                          &ncand[w * 4 + gi], gl, gmask);
-        __syncwarp();
-      }
+      const TierSegs sg = resident_segs(a.lists, a.row_stride, a.off, bl.cursors, q);
+      resident_deal(
+          sg,
+          [&](int32_t v) {
+            if (table_bits_for_degree(a.g.rowptr[v + 1] - a.g.rowptr[v]) <= TIER4_SMEM_BITS)
+              block_decide_node<Pol, RT>(pol, v, hk, hv, cl, &block_ncand, red, usm, &own_sm);
+            else
+              block_decide_scratch<Pol, RT>(pol, v, a.gkeys, a.gvals, a.goff, a.status, red, usm, &own_sm);
+          },
+          [&](int32_t v) {
+            group_decide_node<Pol, 32, T2_BITS, 2>(pol, v, hk + w * R_PER_WARP, hv + w * R_PER_WARP,
+                                                   cl + w * (R_PER_WARP / 2), &ncand[w * 4], lane, 0xffffffffu);
+          },
+          [&](int32_t v, int gi, int gl) {
+            const int o = w * R_PER_WARP + gi * 64;
+            group_decide_node<Pol, 8, 6, 4>(pol, v, hk + o, hv + o, cl + w * (R_PER_WARP / 2) + gi * 32,
+                                            &ncand[w * 4 + gi], gl, 0xffu << (gi * 8));
+          });
       resident_bar();
       lm_apply(a.g, sg, a.labels, a.size, a.sig, a.target, &a.ctl->moved[p], &a.ctl->empties[p][q],
                a.inst_moved ? a.inst_moved + p * a.B : nullptr, trk, bl, q);
@@ -271,15 +202,10 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
 }
 
 template <class Pol>
-void launch_rounds(Ctx& c, const Pol& pol, const ResidentArgs& a, int32_t N, int32_t big, int32_t sms) {
+void launch_rounds(Ctx& c, const Pol& pol, const ResidentArgs& a, unsigned grid) {
   const size_t bytes = TIER4_SMEM_BYTES;
   check_cuda(cudaFuncSetAttribute(k_lm_rounds<Pol>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
              "resident rounds' shared memory");
-  // a block or a warp per node of a sub-round, up to one block per SM: fewer
-  // blocks make the barriers cheaper
-  const int64_t blocks = ((int64_t)big + a.K - 1) / a.K, warps = ((int64_t)(N - big) + a.K - 1) / a.K;
-  const int64_t want = blocks + (warps + RW - 1) / RW;
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, sms));
   launch_coop(c, k_lm_rounds<Pol>, dim3(grid), dim3(RT), bytes, pol, a);
 }
 
@@ -329,10 +255,11 @@ void resident_rounds(Solver& S, const Level& L, int32_t* labels, int it, int lvl
   a.ctl = reinterpret_cast<ResidentCtl*>(c.ws->get_bytes("s_resident", sizeof(ResidentCtl)));
   check_cuda(cudaMemsetAsync(a.ctl, 0, sizeof(ResidentCtl), c.stream), "memset");
   check_cuda(cudaMemsetAsync(S.cursors, 0, 2 * (size_t)S.p.K * NTIERS * sizeof(int32_t), c.stream), "memset");
+  const unsigned grid = resident_grid(L.d.N, (int64_t)S.tier_cnt[3] + S.tier_cnt[4], S.p.K, S.sms);
   if (S.sig.d)
-    launch_rounds(c, lm_policy<true>(S, L, labels, trk), a, L.d.N, S.tier_cnt[3] + S.tier_cnt[4], S.sms);
+    launch_rounds(c, lm_policy<true>(S, L, labels, trk), a, grid);
   else
-    launch_rounds(c, lm_policy<false>(S, L, labels, trk), a, L.d.N, S.tier_cnt[3] + S.tier_cnt[4], S.sms);
+    launch_rounds(c, lm_policy<false>(S, L, labels, trk), a, grid);
   char* h = static_cast<char*>(c.pinned);
   check_cuda(cudaMemcpyAsync(h, &a.ctl->rounds, 4 * sizeof(long long), cudaMemcpyDeviceToHost, c.stream), "copy");
   check_cuda(cudaMemcpyAsync(h + 32, S.sig_used, sizeof(ull), cudaMemcpyDeviceToHost, c.stream), "copy");

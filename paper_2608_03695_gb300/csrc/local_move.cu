@@ -42,9 +42,6 @@ namespace {
 
 constexpr int APPLY_THREADS = 256;
 constexpr int EMPTY_THREADS = 512;
-// Work to decide in a round (entries, and a node counted as so many) up to
-// which rounds are resident.
-constexpr int64_t RESIDENT_MAX_WORK = (int64_t)1 << 22, RESIDENT_NODE_WORK = 16;
 
 unsigned fixed_grid(int per_sm) { return 152u * (unsigned)per_sm; }
 

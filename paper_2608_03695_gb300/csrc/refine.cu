@@ -16,7 +16,7 @@
 // W(R,C\R) is maintained incrementally: when the set M of nodes joins R,
 //   W(R u M, C\(R u M)) = W(R,C\R) + sum_{v in M} [W(v,C\v) - 2 W(v,R)]
 //                         - sum_{v in M} W(v, M\v).
-#include "lm.cuh"
+#include "resident.cuh"
 
 namespace mslice {
 
@@ -31,8 +31,9 @@ __device__ __forceinline__ u128 lam_k_x(const u128* lam, int32_t s, long long k,
 // the lanes share; fewer at level 0, whose rows are short and whose nodes
 // hold one snapshot each, so a warp takes several nodes at once).
 template <int G>
-__global__ void k_ref_init(LevelDev g, const int32_t* P, SigStore sig, const u128* lam, int32_t* R, int32_t* sizeR,
-                           long long* Wc, long long* Wout, uint8_t* elig, SigStore kr, long long* PR) {
+__device__ __forceinline__ void ref_init(const LevelDev& g, const int32_t* P, const SigStore& sig, const u128* lam,
+                                         int32_t* R, int32_t* sizeR, long long* Wc, long long* Wout, uint8_t* elig,
+                                         const SigStore& kr, long long* PR) {
   const int lane = threadIdx.x & 31, gl = lane % G;
   const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (lane - gl));
   const int64_t groups = ((int64_t)gridDim.x * blockDim.x) / G;
@@ -79,6 +80,12 @@ __global__ void k_ref_init(LevelDev g, const int32_t* P, SigStore sig, const u12
   }
 }
 
+template <int G>
+__global__ void k_ref_init(LevelDev g, const int32_t* P, SigStore sig, const u128* lam, int32_t* R, int32_t* sizeR,
+                           long long* Wc, long long* Wout, uint8_t* elig, SigStore kr, long long* PR) {
+  ref_init<G>(g, P, sig, lam, R, sizeR, Wc, Wout, elig, kr, PR);
+}
+
 __global__ void k_classes(LevelDev g, uint64_t seed, uint64_t it, uint64_t lvl, int K, uint8_t* cls) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < g.N; v += (int64_t)gridDim.x * blockDim.x)
     cls[v] = (uint8_t)vertex_class(seed, 1, it, lvl, 0, local_id(g, (int32_t)v), K);
@@ -108,8 +115,9 @@ __global__ void k_rhs_accum(SigStore kr, const int32_t* sizeR, const int32_t* P,
 // node's instance's.)
 // Also packs what a candidate probe reads of sub-community L, as of the
 // sub-round start, into one word: size | class << 32 | well-connected << 40.
-__global__ void k_wc(LevelDev g, const int32_t* sizeR, const long long* Wout, const ull* rhs, const uint8_t* elig,
-                     const uint8_t* cls, uint8_t* wc, unsigned long long* desc) {
+__device__ __forceinline__ void ref_wc(const LevelDev& g, const int32_t* sizeR, const long long* Wout, const ull* rhs,
+                                       const uint8_t* elig, const uint8_t* cls, uint8_t* wc,
+                                       unsigned long long* desc) {
   for (int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; L < g.N; L += (int64_t)gridDim.x * blockDim.x) {
     const int32_t sz = sizeR[L];
     uint8_t f = 0;
@@ -123,6 +131,11 @@ __global__ void k_wc(LevelDev g, const int32_t* sizeR, const long long* Wout, co
     wc[L] = f;
     desc[L] = (unsigned long long)(uint32_t)sz | ((unsigned long long)cls[L] << 32) | ((unsigned long long)f << 40);
   }
+}
+
+__global__ void k_wc(LevelDev g, const int32_t* sizeR, const long long* Wout, const ull* rhs, const uint8_t* elig,
+                     const uint8_t* cls, uint8_t* wc, unsigned long long* desc) {
+  ref_wc(g, sizeR, Wout, rhs, elig, cls, wc, desc);
 }
 
 template <bool DENSE>
@@ -561,6 +574,46 @@ __device__ int32_t rand_choose(const Pol& pol, int32_t v, const typename Pol::VC
   return chosen;
 }
 
+// One node decided by G lanes (gl: rank, base: first lane, gmask: lanes) with
+// tables of 2^BITS slots (K, V, weights WT; CL: room for half of them) in shared
+// memory, all free on entry and left free.
+template <bool DENSE, int G, int BITS>
+__device__ __forceinline__ void ref_random_group_node(const RefPolicy<DENSE>& pol, int32_t v, const RandParams& rp,
+                                                      int32_t* K, long long* V, ull* WT, uint16_t* CL, int32_t* ncand,
+                                                      int gl, int base, unsigned gmask) {
+  if (!pol.begin(v)) {
+    if (gl == 0) pol.skip(v);
+    return;
+  }
+  const typename RefPolicy<DENSE>::VCtx vc = pol.vctx(v);
+  for (int64_t e = pol.g.rowptr[v] + gl; e < pol.g.rowptr[v + 1]; e += G) {
+    int32_t key;
+    long long wgt;
+    if (pol.edge(v, vc, e, key, wgt)) {
+      bool fresh;
+      const int slot = table_add_slot(K, V, BITS, key, wgt, fresh);
+#if MSLICE_CHECKED
+      if (slot < 0) atomicOr(pol.g.chk, ERR_BOUNDS);
+#endif
+      if (fresh) CL[atomicAdd(ncand, 1)] = (uint16_t)slot;
+    }
+  }
+  __syncwarp(gmask);
+  const int n = *ncand;
+  long long Wb;
+  const int32_t X =
+      rand_choose<RefPolicy<DENSE>, G>(pol, v, vc, rp, K, V, WT, CL, n, BITS, gl, base, gmask, nullptr, Wb);
+  if (gl == 0) pol.finish(v, Cand{0, X}, Wb, 0, vc);
+  __syncwarp(gmask);
+  for (int j = gl; j < n; j += G) {
+    const int slot = CL[j];
+    K[slot] = -1;
+    V[slot] = 0;
+  }
+  if (gl == 0) *ncand = 0;
+  __syncwarp(gmask);
+}
+
 // Randomised decisions, degree tiers 0-2: G lanes per node, 2^BITS-slot
 // tables per group in shared memory, with the weights beside them; the
 // distinct target labels are listed as their slots are claimed, and only
@@ -594,37 +647,75 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS)
   const int count = *count_ptr;
   for (int idx = blockIdx.x * NG + gx; idx < count; idx += gridDim.x * NG) {
     const int32_t v = list[idx];
-    if (!pol.begin(v)) {
-      if (gl == 0) pol.skip(v);
-      continue;
-    }
-    const typename RefPolicy<DENSE>::VCtx vc = pol.vctx(v);
-    for (int64_t e = pol.g.rowptr[v] + gl; e < pol.g.rowptr[v + 1]; e += G) {
+    ref_random_group_node<DENSE, G, BITS>(pol, v, rp, K, V, WT, CL, &ncand[gx], gl, gi * G, gmask);
+  }
+}
+
+// One node decided by a block of NT threads, with its tables in shared memory
+// (2^bits slots, all free on entry and left free) or in global scratch at
+// goff[v].
+template <bool DENSE, int NT>
+__device__ __forceinline__ void ref_random_block_node(const RefPolicy<DENSE>& pol, int32_t v, const RandParams& rp,
+                                                      int32_t* hk, long long* hv, ull* hw, uint16_t* cl,
+                                                      int32_t* ncand, u128* sm128, int32_t* gkeys, long long* gvals,
+                                                      ull* gwts, const int64_t* goff, unsigned* status,
+                                                      bool in_global) {
+  if (!pol.begin(v)) {
+    if (threadIdx.x == 0) pol.skip(v);
+    return;
+  }
+  const typename RefPolicy<DENSE>::VCtx vc = pol.vctx(v);
+  const int64_t beg = pol.g.rowptr[v], end = pol.g.rowptr[v + 1];
+  long long Wb;
+  int32_t X;
+  if (!in_global) {
+    const int bits = table_bits_for_degree(end - beg);
+    for (int64_t e = beg + threadIdx.x; e < end; e += NT) {
       int32_t key;
       long long wgt;
       if (pol.edge(v, vc, e, key, wgt)) {
         bool fresh;
-        const int slot = table_add_slot(K, V, BITS, key, wgt, fresh);
+        const int slot = table_add_slot(hk, hv, bits, key, wgt, fresh);
 #if MSLICE_CHECKED
         if (slot < 0) atomicOr(pol.g.chk, ERR_BOUNDS);
 #endif
-        if (fresh) CL[atomicAdd(&ncand[gx], 1)] = (uint16_t)slot;
+        if (fresh) cl[atomicAdd(ncand, 1)] = (uint16_t)slot;
       }
     }
-    __syncwarp(gmask);
-    const int n = ncand[gx];
-    long long Wb;
-    const int32_t X =
-        rand_choose<RefPolicy<DENSE>, G>(pol, v, vc, rp, K, V, WT, CL, n, BITS, gl, gi * G, gmask, nullptr, Wb);
-    if (gl == 0) pol.finish(v, Cand{0, X}, Wb, 0, vc);
-    __syncwarp(gmask);
-    for (int j = gl; j < n; j += G) {
-      const int slot = CL[j];
-      K[slot] = -1;
-      V[slot] = 0;
+    __syncthreads();
+    const int n = *ncand;
+    X = rand_choose<RefPolicy<DENSE>, NT>(pol, v, vc, rp, hk, hv, hw, cl, n, bits, threadIdx.x, 0, 0xffffffffu,
+                                           sm128, Wb);
+    if (threadIdx.x == 0) pol.finish(v, Cand{0, X}, Wb, 0, vc);
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += NT) {
+      const int slot = cl[j];
+      hk[slot] = -1;
+      hv[slot] = 0;
     }
-    if (gl == 0) ncand[gx] = 0;
-    __syncwarp(gmask);
+    if (threadIdx.x == 0) *ncand = 0;
+    __syncthreads();
+  } else {
+    const int bits = table_bits_for_degree(end - beg);
+    const int64_t S = 1ll << bits;
+    int32_t* K = gkeys + goff[v];
+    long long* V = gvals + goff[v];
+    ull* WT = gwts + goff[v];
+    for (int64_t i = threadIdx.x; i < S; i += NT) {
+      K[i] = -1;
+      V[i] = 0;
+    }
+    __syncthreads();
+    for (int64_t e = beg + threadIdx.x; e < end; e += NT) {
+      int32_t key;
+      long long wgt;
+      if (pol.edge(v, vc, e, key, wgt)) gtable_add(K, V, bits, key, wgt, status);
+    }
+    __syncthreads();
+    X = rand_choose<RefPolicy<DENSE>, NT>(pol, v, vc, rp, K, V, WT, nullptr, S, bits, threadIdx.x, 0, 0xffffffffu,
+                                           sm128, Wb);
+    if (threadIdx.x == 0) pol.finish(v, Cand{0, X}, Wb, 0, vc);
+    __syncthreads();
   }
 }
 
@@ -653,63 +744,8 @@ __global__ void __launch_bounds__(256) k_ref_random_block(RefPolicy<DENSE> pol, 
   const int count = *count_ptr;
   for (int idx = blockIdx.x; idx < count; idx += gridDim.x) {
     const int32_t v = list[idx];
-    if (!pol.begin(v)) {
-      if (threadIdx.x == 0) pol.skip(v);
-      continue;
-    }
-    const typename RefPolicy<DENSE>::VCtx vc = pol.vctx(v);
-    const int64_t beg = pol.g.rowptr[v], end = pol.g.rowptr[v + 1];
-    long long Wb;
-    int32_t X;
-    if (!in_global) {
-      const int bits = table_bits_for_degree(end - beg);
-      for (int64_t e = beg + threadIdx.x; e < end; e += 256) {
-        int32_t key;
-        long long wgt;
-        if (pol.edge(v, vc, e, key, wgt)) {
-          bool fresh;
-          const int slot = table_add_slot(hk, hv, bits, key, wgt, fresh);
-#if MSLICE_CHECKED
-          if (slot < 0) atomicOr(pol.g.chk, ERR_BOUNDS);
-#endif
-          if (fresh) cl[atomicAdd(&ncand, 1)] = (uint16_t)slot;
-        }
-      }
-      __syncthreads();
-      const int n = ncand;
-      X = rand_choose<RefPolicy<DENSE>, 256>(pol, v, vc, rp, hk, hv, hw, cl, n, bits, threadIdx.x, 0, 0xffffffffu,
-                                             sm128, Wb);
-      if (threadIdx.x == 0) pol.finish(v, Cand{0, X}, Wb, 0, vc);
-      __syncthreads();
-      for (int j = threadIdx.x; j < n; j += 256) {
-        const int slot = cl[j];
-        hk[slot] = -1;
-        hv[slot] = 0;
-      }
-      if (threadIdx.x == 0) ncand = 0;
-      __syncthreads();
-    } else {
-      const int bits = table_bits_for_degree(end - beg);
-      const int64_t S = 1ll << bits;
-      int32_t* K = gkeys + goff[v];
-      long long* V = gvals + goff[v];
-      ull* WT = gwts + goff[v];
-      for (int64_t i = threadIdx.x; i < S; i += 256) {
-        K[i] = -1;
-        V[i] = 0;
-      }
-      __syncthreads();
-      for (int64_t e = beg + threadIdx.x; e < end; e += 256) {
-        int32_t key;
-        long long wgt;
-        if (pol.edge(v, vc, e, key, wgt)) gtable_add(K, V, bits, key, wgt, status);
-      }
-      __syncthreads();
-      X = rand_choose<RefPolicy<DENSE>, 256>(pol, v, vc, rp, K, V, WT, nullptr, S, bits, threadIdx.x, 0, 0xffffffffu,
-                                             sm128, Wb);
-      if (threadIdx.x == 0) pol.finish(v, Cand{0, X}, Wb, 0, vc);
-      __syncthreads();
-    }
+    ref_random_block_node<DENSE, 256>(pol, v, rp, hk, hv, hw, cl, &ncand, sm128, gkeys, gvals, gwts, goff, status,
+                                      in_global != 0);
   }
 }
 
@@ -761,9 +797,9 @@ __device__ __forceinline__ bool seg3_item_in(const Segs3& sg, int64_t idx, int32
 // Applies the sub-round's refinement moves of tiers [T0, T1): G lanes per
 // node (8 for the short rows of the low tiers, a warp otherwise).
 template <int G, int T0, int T1>
-__global__ void k_ref_apply(LevelDev g, Segs3 sg, const int32_t* P, const int32_t* target, const long long* Wc,
-                            const long long* Wsel, int32_t* R, int32_t* sizeR, long long* Wout, SigStore kr,
-                            long long* PR) {
+__device__ __forceinline__ void ref_apply(const LevelDev& g, const Segs3& sg, const int32_t* P, const int32_t* target,
+                                          const long long* Wc, const long long* Wsel, int32_t* R, int32_t* sizeR,
+                                          long long* Wout, const SigStore& kr, long long* PR) {
   const int lane = threadIdx.x & 31, gl = lane % G;
   const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (lane - gl));
   const int total = seg3_total_in<T0, T1>(sg);
@@ -812,13 +848,182 @@ __global__ void k_ref_apply(LevelDev g, Segs3 sg, const int32_t* P, const int32_
   }
 }
 
-__global__ void k_ref_reset(Segs3 sg, int32_t* target) {
+template <int G, int T0, int T1>
+__global__ void k_ref_apply(LevelDev g, Segs3 sg, const int32_t* P, const int32_t* target, const long long* Wc,
+                            const long long* Wsel, int32_t* R, int32_t* sizeR, long long* Wout, SigStore kr,
+                            long long* PR) {
+  ref_apply<G, T0, T1>(g, sg, P, target, Wc, Wsel, R, sizeR, Wout, kr, PR);
+}
+
+__device__ __forceinline__ void ref_reset(const Segs3& sg, int32_t* target) {
   const int total = seg3_total(sg);
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
     int32_t v;
     if (seg3_item(sg, idx, v)) target[v] = NO_MOVE;
   }
+}
+
+__global__ void k_ref_reset(Segs3 sg, int32_t* target) { ref_reset(sg, target); }
+
+// ---------------------------------------------------------------------------
+// The whole refinement of a small level in one cooperative launch: about 45
+// launches (0.35 ms, however small the level) become 4 K + 1 grid barriers.
+// The right-hand sides of well-connectedness are summed over the members,
+//   sum_s Lambda_s K_{R,s} (K_{C,s} - K_{R,s})
+//     = sum_{v in R} sum_s Lambda_s k_{v,s} (K_{C,s} - K_{R,s}),
+// so no pass over the whole table (sized for level 0) is needed.
+struct RefArgs {
+  LevelDev g;
+  const int32_t* P;
+  SigStore sig, kr;
+  const u128* lam;
+  int32_t *R, *sizeR, *target;
+  long long *Wc, *Wout, *Wsel, *PR;
+  unsigned long long* desc;
+  uint8_t *elig, *wc, *cls;
+  ull* rhs;
+  const uint8_t* tier;
+  const int32_t* active;
+  int32_t* lists;
+  int64_t row_stride;
+  TierOff off;
+  int32_t* cursors;  // zero on entry
+  uint64_t seed, it, lvl;
+  int32_t K;
+  int32_t* gkeys;
+  long long* gvals;
+  ull* gwts;
+  const int64_t* goff;
+  unsigned* status;
+  RandParams rp;
+};
+
+template <bool DENSE>
+__device__ __forceinline__ u128 ref_rhs_part(const RefArgs& a, int32_t v, int32_t Rl, int t, int nt) {
+  int64_t b, e;
+  slice_range(a.g, v, b, e);
+  const int32_t C = a.P[v];
+  u128 acc = 0;
+  for (int64_t j = b + t; j < e; j += nt) {
+    int32_t s;
+    long long k;
+    slice_entry(a.g, v, j, s, k);
+    acc += lam_k_x(a.lam, s, k, sst_get<DENSE>(a.sig, C, s) - sst_get<DENSE>(a.kr, Rl, s));
+  }
+  return acc;
+}
+
+template <bool DENSE, bool RANDOM>
+__global__ void __launch_bounds__(RT, 1) k_refine(RefPolicy<DENSE> pol, RefArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  long long* hv = reinterpret_cast<long long*>(smem);
+  ull* hw = reinterpret_cast<ull*>(hv + R_SLOTS);  // RANDOM only
+  int32_t* hk = reinterpret_cast<int32_t*>(smem + (RANDOM ? 2 : 1) * R_SLOTS * sizeof(long long));
+  uint16_t* cl = reinterpret_cast<uint16_t*>(hk + R_SLOTS);
+  __shared__ int32_t ncand[RW * 4];
+  __shared__ int32_t block_ncand;
+  __shared__ Cand red[RW];
+  __shared__ ull usm[2 * RW];
+  __shared__ i128 own_sm;
+  __shared__ u128 sm128[RW + 1];
+  __shared__ int32_t seg_cnt[64 * NTIERS], seg_base[64 * NTIERS];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t tid = (int64_t)blockIdx.x * RT + threadIdx.x, threads = (int64_t)gridDim.x * RT;
+  for (int i = threadIdx.x; i < R_SLOTS; i += RT) {
+    hk[i] = -1;
+    hv[i] = 0;
+  }
+  for (int i = threadIdx.x; i < RW * 4; i += RT) ncand[i] = 0;
+  if (threadIdx.x == 0) block_ncand = 0;
+  if (a.g.is0)
+    ref_init<8>(a.g, a.P, a.sig, a.lam, a.R, a.sizeR, a.Wc, a.Wout, a.elig, a.kr, a.PR);
+  else
+    ref_init<32>(a.g, a.P, a.sig, a.lam, a.R, a.sizeR, a.Wc, a.Wout, a.elig, a.kr, a.PR);
+  for (int64_t i = tid; i < 2 * (int64_t)a.g.N; i += threads) a.rhs[i] = 0;
+  resident_list(a.g.N, a.K * NTIERS, a.lists, a.row_stride, a.off, a.cursors, seg_cnt, seg_base, [&](int32_t v) {
+    const int cls = vertex_class(a.seed, 1, a.it, a.lvl, 0, local_id(a.g, v), a.K);
+    a.cls[v] = (uint8_t)cls;
+    if (a.active && !a.active[node_inst(a.g, v)]) return (int)SEG_FROZEN;
+    return cls * NTIERS + (int)a.tier[v];
+  });
+  resident_bar();
+  for (int q = 0; q < a.K; ++q) {
+    // well-connectedness of every sub-community at the sub-round start
+    if (q > 0) {
+      ref_reset(resident_segs(a.lists, a.row_stride, a.off, a.cursors, q - 1), a.target);
+      if (a.g.is0) {
+        for (int64_t v = tid; v < a.g.N; v += threads) {
+          const int32_t Rl = a.R[v];
+          if (a.sizeR[Rl] > 1) atomic_add_u128(&a.rhs[2 * (int64_t)Rl], ref_rhs_part<DENSE>(a, (int32_t)v, Rl, 0, 1));
+        }
+      } else {
+        for (int64_t v = tid >> 5; v < a.g.N; v += threads >> 5) {
+          const int32_t Rl = a.R[v];
+          if (a.sizeR[Rl] <= 1) continue;  // (uniform per warp)
+          const u128 x = warp_sum_u128(ref_rhs_part<DENSE>(a, (int32_t)v, Rl, lane, 32));
+          if (lane == 0) atomic_add_u128(&a.rhs[2 * (int64_t)Rl], x);
+        }
+      }
+      resident_bar();
+    }
+    ref_wc(a.g, a.sizeR, a.Wout, a.rhs, a.elig, a.cls, a.wc, a.desc);
+    resident_bar();
+    pol.q = q;
+    const Segs3 sg = resident_segs(a.lists, a.row_stride, a.off, a.cursors, q);
+    for (int64_t i = tid; i < 2 * (int64_t)a.g.N; i += threads) a.rhs[i] = 0;  // (read before the barrier above)
+    if constexpr (RANDOM) {
+      auto by_warp = [&](int32_t v) {
+        const int o = w * R_PER_WARP;
+        ref_random_group_node<DENSE, 32, T2_BITS>(pol, v, a.rp, hk + o, hv + o, hw + o, cl + w * (R_PER_WARP / 2),
+                                                  &ncand[w * 4], lane, 0, 0xffffffffu);
+      };
+      // (a warp for the low tiers too: most of a node's work is per candidate)
+      const int gw = blockIdx.x * RW + w, warps = gridDim.x * RW;
+      const int n0 = *sg.count[0], n = n0 + *sg.count[1];
+      for (int i = gw; i < n; i += warps) by_warp(i < n0 ? sg.list[0][i] : sg.list[1][i - n0]);
+      for (int t = NTIERS - 2; t < NTIERS; ++t) {
+        const int m = *sg.count[t];
+        for (int i = blockIdx.x; i < m; i += gridDim.x) {
+          __syncthreads();
+          const int32_t v = sg.list[t][i];
+          const bool big = table_bits_for_degree(a.g.rowptr[v + 1] - a.g.rowptr[v]) > TIER4_SMEM_BITS;
+          ref_random_block_node<DENSE, RT>(pol, v, a.rp, hk, hv, hw, cl, &block_ncand, sm128, a.gkeys, a.gvals, a.gwts,
+                                           a.goff, a.status, big);
+        }
+      }
+      __syncthreads();
+      const int m2 = *sg.count[2];
+      for (int i = gw; i < m2; i += warps) by_warp(sg.list[2][i]);
+    } else {
+      resident_deal(
+          sg,
+          [&](int32_t v) {
+            if (!pol.begin(v)) {
+              if (threadIdx.x == 0) pol.skip(v);
+            } else if (table_bits_for_degree(a.g.rowptr[v + 1] - a.g.rowptr[v]) <= TIER4_SMEM_BITS) {
+              block_decide_node<RefPolicy<DENSE>, RT>(pol, v, hk, hv, cl, &block_ncand, red, usm, &own_sm);
+            } else {
+              block_decide_scratch<RefPolicy<DENSE>, RT>(pol, v, a.gkeys, a.gvals, a.goff, a.status, red, usm, &own_sm);
+            }
+          },
+          [&](int32_t v) {
+            group_decide_node<RefPolicy<DENSE>, 32, T2_BITS, 2>(pol, v, hk + w * R_PER_WARP, hv + w * R_PER_WARP,
+                                                                cl + w * (R_PER_WARP / 2), &ncand[w * 4], lane,
+                                                                0xffffffffu);
+          },
+          [&](int32_t v, int gi, int gl) {
+            const int o = w * R_PER_WARP + gi * 64;
+            group_decide_node<RefPolicy<DENSE>, 8, 6, 4>(pol, v, hk + o, hv + o, cl + w * (R_PER_WARP / 2) + gi * 32,
+                                                         &ncand[w * 4 + gi], gl, 0xffu << (gi * 8));
+          });
+    }
+    resident_bar();
+    ref_apply<8, 0, 2>(a.g, sg, a.P, a.target, a.Wc, a.Wsel, a.R, a.sizeR, a.Wout, a.kr, a.PR);
+    ref_apply<32, 2, NTIERS>(a.g, sg, a.P, a.target, a.Wc, a.Wsel, a.R, a.sizeR, a.Wout, a.kr, a.PR);
+    resident_bar();
+  }
+  ref_reset(resident_segs(a.lists, a.row_stride, a.off, a.cursors, a.K - 1), a.target);
 }
 
 unsigned fixed_grid(int per_sm) { return 152u * (unsigned)per_sm; }
@@ -879,13 +1084,16 @@ static void refine_impl(Solver& S, const Level& L, const int32_t* P, int it, int
   if (N == 0) return;
   clear_store(S, S.kr);
   long long* PR = c.ws->get<long long>("ref_PR", N);
-  if (L.d.is0)
-    launch(c, k_ref_init<8>, dim3(fixed_grid(8)), dim3(256), 0, L.d, P, S.sig, (const u128*)S.lam, S.R, S.sizeR,
-           S.Wc, S.Wout, S.elig, S.kr, PR);
-  else
-    launch(c, k_ref_init<32>, dim3(fixed_grid(8)), dim3(256), 0, L.d, P, S.sig, (const u128*)S.lam, S.R, S.sizeR,
-           S.Wc, S.Wout, S.elig, S.kr, PR);
-  bucket(S, L, 1, it, lvl, 0, S.inst_active);
+  const bool resident = L.nnz + RESIDENT_NODE_WORK * (int64_t)N <= RESIDENT_REFINE_WORK;
+  if (!resident) {
+    if (L.d.is0)
+      launch(c, k_ref_init<8>, dim3(fixed_grid(8)), dim3(256), 0, L.d, P, S.sig, (const u128*)S.lam, S.R, S.sizeR,
+             S.Wc, S.Wout, S.elig, S.kr, PR);
+    else
+      launch(c, k_ref_init<32>, dim3(fixed_grid(8)), dim3(256), 0, L.d, P, S.sig, (const u128*)S.lam, S.R, S.sizeR,
+             S.Wc, S.Wout, S.elig, S.kr, PR);
+    bucket(S, L, 1, it, lvl, 0, S.inst_active);
+  }
   RefPolicy<DENSE> pol;
   pol.g = L.d;
   pol.P = P;
@@ -901,6 +1109,52 @@ static void refine_impl(Solver& S, const Level& L, const int32_t* P, int it, int
   pol.target = S.target;
   pol.Wsel = S.Wsel;
   pol.cls = S.cls;
+  const RandParams rp{S.p.seed, (uint64_t)it, (uint64_t)lvl, S.rdiv, (ull)S.p.theta_den};
+  if (resident) {
+    RefArgs a{};
+    a.g = L.d;
+    a.P = P;
+    a.sig = S.sig;
+    a.kr = S.kr;
+    a.lam = S.lam;
+    a.R = S.R;
+    a.sizeR = S.sizeR;
+    a.target = S.target;
+    a.Wc = S.Wc;
+    a.Wout = S.Wout;
+    a.Wsel = S.Wsel;
+    a.PR = PR;
+    a.desc = desc;
+    a.elig = S.elig;
+    a.wc = S.wc;
+    a.cls = S.cls;
+    a.rhs = S.rhs;
+    a.tier = S.tier;
+    a.active = S.inst_active;
+    a.lists = S.lists;
+    a.row_stride = S.N0;
+    a.off = tier_offsets(S);
+    a.cursors = S.cursors;
+    a.seed = S.p.seed;
+    a.it = (uint64_t)it;
+    a.lvl = (uint64_t)lvl;
+    a.K = S.p.K;
+    a.gkeys = S.gkeys;
+    a.gvals = S.gvals;
+    a.gwts = S.gwts;
+    a.goff = S.goff;
+    a.status = c.d_status;
+    a.rp = rp;
+    check_cuda(cudaMemsetAsync(S.cursors, 0, (size_t)S.p.K * NTIERS * sizeof(int32_t), c.stream), "memset");
+    const bool random = S.p.theta_num > 0;
+    const size_t bytes = TIER4_SMEM_BYTES + (random ? R_SLOTS * sizeof(ull) : 0);
+    const auto k = random ? k_refine<DENSE, true> : k_refine<DENSE, false>;
+    check_cuda(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
+               "resident refinement's shared memory");
+    launch_coop(c, k, dim3(resident_grid(N, (int64_t)S.tier_cnt[3] + S.tier_cnt[4], S.p.K, S.sms)), dim3(RT), bytes,
+                pol, a);
+    return;
+  }
   launch(c, k_classes, dim3(fixed_grid(8)), dim3(256), 0, L.d, S.p.seed, (uint64_t)it, (uint64_t)lvl, S.p.K, S.cls);
   for (int q = 0; q < S.p.K; ++q) {
     // well-connectedness of every sub-community at the sub-round start
@@ -914,7 +1168,7 @@ static void refine_impl(Solver& S, const Level& L, const int32_t* P, int it, int
     pol.q = q;
     const Segs3 sg = bucket_segments(S, q);
     if (S.p.theta_num > 0) {
-      random_all<DENSE>(S, pol, sg, RandParams{S.p.seed, (uint64_t)it, (uint64_t)lvl, S.rdiv, (ull)S.p.theta_den});
+      random_all<DENSE>(S, pol, sg, rp);
     } else {
       decide_all(c, pol, sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
     }
