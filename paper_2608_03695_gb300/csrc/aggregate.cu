@@ -15,7 +15,7 @@
 #include <cstring>
 
 #include "../../include/mslice.h"
-#include "solver.h"
+#include "resident.cuh"
 
 namespace mslice {
 
@@ -119,8 +119,109 @@ __device__ __forceinline__ int64_t gtab_add(int32_t* hk, long long* hv, int64_t 
   return -1;
 }
 
-// One warp per new node x (tier 0).  Members are fetched 32 at a time with
-// their row bounds; lanes stride over each member's entries.
+// One row by a warp (at most CW_MAX stored and snapshot entries).  Members are
+// fetched 32 at a time with their row bounds; lanes stride over each member's
+// entries.  K, V (2^CW_BITS slots), CL and *ncl: the warp's shared table, free on
+// entry and left free.
+struct RowOut {
+  const int64_t *eoff, *soff;  // the rows' places in the upper-bound layout
+  int32_t* tcol;
+  long long* tw;
+  int32_t* ecnt;
+  int32_t* tsidx;
+  long long* tsval;
+  int32_t* scnt;
+};
+
+__device__ __forceinline__ void contract_row_warp(const LevelDev& g, const int32_t* xmap, const int64_t* moff,
+                                                  const int32_t* mem, int32_t x, int32_t* K, long long* V,
+                                                  uint16_t* CL, int32_t* ncl, const RowOut& o) {
+  constexpr int SLOTS = 1 << CW_BITS;
+  const int lane = threadIdx.x & 31;
+  const int64_t mb = moff[x], me = moff[x + 1];
+  int n = 0;
+  for (int64_t j0 = mb; j0 < me; j0 += 32) {
+    const int64_t jj = j0 + lane;
+    int32_t mv = 0;
+    int64_t rb = 0, re = 0;
+    if (jj < me) {
+      mv = mem[jj];
+      rb = g.rowptr[mv];
+      re = g.rowptr[mv + 1];
+    }
+    const int cm = (int)min((int64_t)32, me - j0);
+    for (int t = 0; t < cm; ++t) {
+      const int32_t v = __shfl_sync(0xffffffffu, mv, t);
+      const int64_t b = __shfl_sync(0xffffffffu, rb, t), e = __shfl_sync(0xffffffffu, re, t);
+      const Omega om = node_omega(g, v);
+      for (int64_t base = b; base < e; base += 32) {
+        const int64_t i = base + lane;
+        bool fresh = false;
+        int64_t slot = 0;
+        if (i < e) {
+          int32_t u;
+          long long W;
+          if (edge_at(g, i, u, W, om)) {
+            const int32_t y = xmap[u];
+            if (y != x) slot = ctab_add(K, V, SLOTS, y, W, fresh);
+#if MSLICE_CHECKED
+            if (y != x && slot < 0) atomicOr(g.chk, ERR_BOUNDS);
+#endif
+          }
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, fresh);
+        if (fresh) CL[n + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)slot;
+        n += __popc(bal);
+      }
+    }
+  }
+  __syncwarp();
+  const int64_t eo = o.eoff[x];
+  for (int k = lane; k < n; k += 32) {
+    const int slot = CL[k];
+    o.tcol[eo + k] = K[slot];
+    o.tw[eo + k] = V[slot];
+    K[slot] = -1;
+    V[slot] = 0;
+  }
+  if (lane == 0) o.ecnt[x] = n;
+  __syncwarp();
+  // snapshot strengths: lane per member
+  for (int64_t j = mb + lane; j < me; j += 32) {
+    const int32_t v = mem[j];
+    int64_t b, e;
+    slice_range(g, v, b, e);
+    for (int64_t q = b; q < e; ++q) {
+      int32_t sl;
+      long long k;
+      slice_entry(g, v, q, sl, k);
+      bool fresh;
+      const int64_t slot = ctab_add(K, V, SLOTS, sl, k, fresh);
+#if MSLICE_CHECKED
+          if (slot < 0) atomicOr(g.chk, ERR_BOUNDS);
+#endif
+      if (fresh) CL[atomicAdd(ncl, 1)] = (uint16_t)slot;
+    }
+  }
+  __syncwarp();
+  const int ns = *ncl;
+  const int64_t so = o.soff[x];
+  for (int k = lane; k < ns; k += 32) {
+    const int slot = CL[k];
+    o.tsidx[so + k] = K[slot];
+    o.tsval[so + k] = V[slot];
+    K[slot] = -1;
+    V[slot] = 0;
+  }
+  __syncwarp();
+  if (lane == 0) {
+    o.scnt[x] = ns;
+    *ncl = 0;
+  }
+  __syncwarp();
+}
+
+// One warp per new node x (tier 0).
 __global__ void __launch_bounds__(CW_WARPS * 32)
     k_contract_warp(LevelDev g, const int32_t* xmap, const int64_t* moff, const int32_t* mem, const int32_t* list,
                     const int32_t* count_ptr, const int64_t* eoff, const int64_t* soff, int32_t* tcol, long long* tw,
@@ -143,88 +244,8 @@ __global__ void __launch_bounds__(CW_WARPS * 32)
   const int count = *count_ptr;
   const int64_t warps = (int64_t)gridDim.x * CW_WARPS;
   for (int64_t idx = (int64_t)blockIdx.x * CW_WARPS + w; idx < count; idx += warps) {
-    const int32_t x = list[idx];
-    const int64_t mb = moff[x], me = moff[x + 1];
-    int n = 0;
-    for (int64_t j0 = mb; j0 < me; j0 += 32) {
-      const int64_t jj = j0 + lane;
-      int32_t mv = 0;
-      int64_t rb = 0, re = 0;
-      if (jj < me) {
-        mv = mem[jj];
-        rb = g.rowptr[mv];
-        re = g.rowptr[mv + 1];
-      }
-      const int cm = (int)min((int64_t)32, me - j0);
-      for (int t = 0; t < cm; ++t) {
-        const int32_t v = __shfl_sync(0xffffffffu, mv, t);
-        const int64_t b = __shfl_sync(0xffffffffu, rb, t), e = __shfl_sync(0xffffffffu, re, t);
-        const Omega om = node_omega(g, v);
-        for (int64_t base = b; base < e; base += 32) {
-          const int64_t i = base + lane;
-          bool fresh = false;
-          int64_t slot = 0;
-          if (i < e) {
-            int32_t u;
-            long long W;
-            if (edge_at(g, i, u, W, om)) {
-              const int32_t y = xmap[u];
-              if (y != x) slot = ctab_add(K, V, SLOTS, y, W, fresh);
-#if MSLICE_CHECKED
-              if (y != x && slot < 0) atomicOr(g.chk, ERR_BOUNDS);
-#endif
-            }
-          }
-          const unsigned bal = __ballot_sync(0xffffffffu, fresh);
-          if (fresh) CL[n + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)slot;
-          n += __popc(bal);
-        }
-      }
-    }
-    __syncwarp();
-    const int64_t eo = eoff[x];
-    for (int k = lane; k < n; k += 32) {
-      const int slot = CL[k];
-      tcol[eo + k] = K[slot];
-      tw[eo + k] = V[slot];
-      K[slot] = -1;
-      V[slot] = 0;
-    }
-    if (lane == 0) ecnt[x] = n;
-    __syncwarp();
-    // snapshot strengths: lane per member
-    for (int64_t j = mb + lane; j < me; j += 32) {
-      const int32_t v = mem[j];
-      int64_t b, e;
-      slice_range(g, v, b, e);
-      for (int64_t q = b; q < e; ++q) {
-        int32_t sl;
-        long long k;
-        slice_entry(g, v, q, sl, k);
-        bool fresh;
-        const int64_t slot = ctab_add(K, V, SLOTS, sl, k, fresh);
-#if MSLICE_CHECKED
-            if (slot < 0) atomicOr(g.chk, ERR_BOUNDS);
-#endif
-        if (fresh) CL[atomicAdd(&ncl[w], 1)] = (uint16_t)slot;
-      }
-    }
-    __syncwarp();
-    const int ns = ncl[w];
-    const int64_t so = soff[x];
-    for (int k = lane; k < ns; k += 32) {
-      const int slot = CL[k];
-      tsidx[so + k] = K[slot];
-      tsval[so + k] = V[slot];
-      K[slot] = -1;
-      V[slot] = 0;
-    }
-    __syncwarp();
-    if (lane == 0) {
-      scnt_out[x] = ns;
-      ncl[w] = 0;
-    }
-    __syncwarp();
+    contract_row_warp(g, xmap, moff, mem, list[idx], K, V, CL, &ncl[w],
+                      RowOut{eoff, soff, tcol, tw, ecnt, tsidx, tsval, scnt_out});
   }
 }
 
@@ -527,7 +548,9 @@ __global__ void k_next_inst(LevelDev g, const int32_t* R, const int32_t* newid, 
     const int32_t x = newid[R[v]];
     const int32_t i = g.inst[v];
     inst_next[x] = i;
-    atomicMin(&off_next[i], x);
+    // (most nodes find a smaller id there: one atomic each on B words took
+    // 0.15 ms of a level of 0.7 M nodes)
+    if (x < off_next[i]) atomicMin(&off_next[i], x);
   }
 }
 
@@ -536,12 +559,330 @@ __global__ void k_compose(const int32_t* R, const int32_t* newid, int64_t N0, in
     node_of0[v] = newid[R[node_of0[v]]];
 }
 
-__global__ void k_max_deg(const int64_t* rowptr, int32_t N, int32_t* mx) {
-  int32_t m = 0;
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x)
-    m = max(m, (int32_t)(rowptr[v + 1] - rowptr[v]));
-  for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(mx, m);
+// ---------------------------------------------------------------------------
+// The whole aggregation of a small level in one cooperative launch: the path
+// below is about 28 launches and three synchronisations (0.26 ms however small
+// the level); here they are eight grid barriers and one synchronisation, with
+// outputs allocated by upper bound.  Rows are summed by a warp or a block; a row
+// that needs more distinct targets than the block's table holds, or is so long
+// that one block would hold up the level, sends the level to the general path.
+// The next level's degree tiers are found on the way.
+constexpr int64_t RESIDENT_ROW_MAX = 1 << 15;  // entries of a row one block sums
+
+struct AggCtl {
+  int32_t np, general, nblock, pad_;
+  int32_t tier[NTIERS], pad2_[3];
+  int64_t mu, ms;
+};
+
+struct AggArgs {
+  LevelDev g;
+  const int32_t *R, *sizeR, *P;
+  int32_t T;  // null slices
+  int32_t *newid, *minid, *xmap, *mcnt, *scnt, *mem, *big;
+  long long* dsum;
+  int64_t *moff, *eoff, *soff;
+  int32_t *tcol, *ecnt, *tsidx, *scnt_out;
+  long long *tw, *tsval;
+  int64_t *rowptr, *sptr;
+  int32_t *col, *sidx;
+  long long *W, *sval;
+  int32_t* next_labels;
+  int32_t *inst_next, *off_next;
+  int32_t B;
+  uint8_t* tier;
+  TierCuts cuts;
+  long long* blk;  // 3 words per block
+  AggCtl* ctl;
+};
+
+// Exclusive prefix of this block's share over the blocks (blk[0..gridDim.x)),
+// and the total over all blocks.
+__device__ __forceinline__ long long blocks_before(const long long* blk, long long* sm, long long& total) {
+  long long before = 0, all = 0;
+  for (int b = threadIdx.x; b < gridDim.x; b += RT) {
+    const long long x = blk[b];
+    all += x;
+    if (b < blockIdx.x) before += x;
+  }
+  long long tb;
+  block_scan_excl(before, sm, tb);
+  block_scan_excl(all, sm, total);
+  return tb;
+}
+
+__global__ void __launch_bounds__(RT, 1) k_aggregate(AggArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  long long* hv = reinterpret_cast<long long*>(smem);
+  int32_t* hk = reinterpret_cast<int32_t*>(smem + R_SLOTS * sizeof(long long));
+  uint16_t* cl = reinterpret_cast<uint16_t*>(hk + R_SLOTS);
+  __shared__ long long sm[33];
+  __shared__ int32_t ncl[RW];
+  __shared__ int32_t ncnt, tiers[NTIERS];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t tid = (int64_t)blockIdx.x * RT + threadIdx.x, threads = (int64_t)gridDim.x * RT;
+  const int32_t N = a.g.N;
+  const int nb = gridDim.x;
+  for (int i = threadIdx.x; i < R_SLOTS; i += RT) {
+    hk[i] = -1;
+    hv[i] = 0;
+  }
+  if (threadIdx.x < RW) ncl[threadIdx.x] = 0;
+  if (threadIdx.x < NTIERS) tiers[threadIdx.x] = 0;
+  // ---- new ids: ranks of the present sub-community labels
+  {
+    const int32_t chunk = (N + nb - 1) / nb;
+    const int32_t lo = min((int64_t)N, (int64_t)blockIdx.x * chunk), hi = min((int64_t)N, (int64_t)lo + chunk);
+    long long cnt = 0, tot;
+    for (int32_t i = lo + threadIdx.x; i < hi; i += RT) cnt += a.sizeR[i] > 0;
+    block_scan_excl(cnt, sm, tot);
+    if (threadIdx.x == 0) a.blk[blockIdx.x] = tot;
+    for (int64_t i = tid; i <= N; i += threads) {
+      a.mcnt[i] = a.scnt[i] = 0;
+      a.dsum[i] = 0;
+      if (i < N) a.minid[i] = INT32_MAX;
+    }
+    resident_bar();
+    long long np;
+    long long at = blocks_before(a.blk, sm, np);
+    if (tid == 0) a.ctl->np = (int32_t)np;
+    if (np == N) return;  // (every block alike) nothing merged
+    for (int32_t base = lo; base < hi; base += RT) {
+      const int32_t i = base + threadIdx.x;
+      const long long f = i < hi && a.sizeR[i] > 0 ? 1 : 0;
+      long long t;
+      const long long r = block_scan_excl(f, sm, t);
+      if (i < hi) a.newid[i] = (int32_t)(at + r);
+      at += t;
+    }
+    if (a.inst_next)
+      for (int64_t i = tid; i <= a.B; i += threads) a.off_next[i] = (int32_t)np;
+  }
+  resident_bar();
+  // ---- members, entries and snapshot entries of every new node
+  for (int64_t v = tid; v < N; v += threads) {
+    const int32_t x = a.newid[a.R[v]];
+    a.xmap[v] = x;
+    atomicAdd(&a.mcnt[x], 1);
+    atomicAdd((ull*)&a.dsum[x], (ull)(a.g.rowptr[v + 1] - a.g.rowptr[v]));
+    int64_t b, e;
+    slice_range(a.g, (int32_t)v, b, e);
+    if (e > b) atomicAdd(&a.scnt[x], (int32_t)(e - b));
+    atomicMin(&a.minid[a.P[v]], x);
+    if (a.inst_next) {
+      const int32_t i = a.g.inst[v];
+      a.inst_next[x] = i;
+      if (x < a.off_next[i]) atomicMin(&a.off_next[i], x);
+    }
+  }
+  resident_bar();
+  const int32_t Np = a.ctl->np;
+  const int32_t chunk = (Np + nb - 1) / nb;
+  const int32_t lo = min((int64_t)Np, (int64_t)blockIdx.x * chunk), hi = min((int64_t)Np, (int64_t)lo + chunk);
+  {
+    long long m = 0, d = 0, c = 0, t;
+    for (int32_t x = lo + threadIdx.x; x < hi; x += RT) {
+      const long long dx = a.dsum[x], cx = a.scnt[x];
+      m += a.mcnt[x];
+      d += dx;
+      c += cx;
+      if (max(dx, cx) > CW_MAX) {
+        a.big[atomicAdd(&a.ctl->nblock, 1)] = x;
+        // slots: distinct targets, and snapshots (addressed directly up to
+        // R_SLOTS of them)
+        if (min(dx, (long long)Np) > R_SLOTS / 2 || (a.T > R_SLOTS && min(cx, (long long)a.T) > R_SLOTS / 2) ||
+            max(dx, cx) > RESIDENT_ROW_MAX)
+          a.ctl->general = 1;
+      }
+    }
+    block_scan_excl(m, sm, t);
+    if (threadIdx.x == 0) a.blk[blockIdx.x] = t;
+    block_scan_excl(d, sm, t);
+    if (threadIdx.x == 0) a.blk[nb + blockIdx.x] = t;
+    block_scan_excl(c, sm, t);
+    if (threadIdx.x == 0) a.blk[2 * nb + blockIdx.x] = t;
+  }
+  resident_bar();
+  if (a.ctl->general) return;  // (every block alike)
+  {
+    long long tm, td, tc;
+    long long am = blocks_before(a.blk, sm, tm), ad = blocks_before(a.blk + nb, sm, td),
+              ac = blocks_before(a.blk + 2 * nb, sm, tc);
+    for (int32_t base = lo; base < hi; base += RT) {
+      const int32_t x = base + threadIdx.x;
+      const bool in = x < hi;
+      long long t;
+      const long long rm = block_scan_excl(in ? (long long)a.mcnt[x] : 0ll, sm, t);
+      if (in) {
+        a.moff[x] = am + rm;
+        a.mcnt[x] = 0;  // (fill counts of the member lists)
+      }
+      am += t;
+      const long long rd = block_scan_excl(in ? a.dsum[x] : 0ll, sm, t);
+      if (in) a.eoff[x] = ad + rd;
+      ad += t;
+      const long long rc = block_scan_excl(in ? (long long)a.scnt[x] : 0ll, sm, t);
+      if (in) a.soff[x] = ac + rc;
+      ac += t;
+    }
+    if (tid == 0) a.moff[Np] = tm;
+    for (int64_t v = tid; v < N; v += threads) a.next_labels[a.xmap[v]] = a.minid[a.P[v]];
+  }
+  resident_bar();
+  for (int64_t v = tid; v < N; v += threads) {
+    const int32_t x = a.xmap[v];
+    a.mem[a.moff[x] + atomicAdd(&a.mcnt[x], 1)] = (int32_t)v;
+  }
+  resident_bar();
+  // ---- rows: a block each for the long ones, then a warp each
+  const RowOut o{a.eoff, a.soff, a.tcol, a.tw, a.ecnt, a.tsidx, a.tsval, a.scnt_out};
+  const int nbig = a.ctl->nblock;
+  for (int i = blockIdx.x; i < nbig; i += nb) {
+    const int32_t x = a.big[i];
+    if (threadIdx.x == 0) ncnt = 0;
+    __syncthreads();
+    const int64_t mb = a.moff[x], me = a.moff[x + 1];
+    for (int64_t j = mb + w; j < me; j += RW) {
+      const int32_t v = a.mem[j];
+      const int64_t b = a.g.rowptr[v], e = a.g.rowptr[v + 1];
+      const Omega om = node_omega(a.g, v);
+      for (int64_t q = b + lane; q < e; q += 32) {
+        int32_t u;
+        long long W;
+        if (edge_at(a.g, q, u, W, om)) {
+          const int32_t y = a.xmap[u];
+          if (y != x) {
+            bool fresh;
+            const int64_t slot = ctab_add(hk, hv, R_SLOTS, y, W, fresh);
+#if MSLICE_CHECKED
+            if (slot < 0) atomicOr(a.g.chk, ERR_BOUNDS);
+#endif
+            if (fresh) cl[atomicAdd(&ncnt, 1)] = (uint16_t)slot;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    const int n = ncnt;
+    for (int k = threadIdx.x; k < n; k += RT) {
+      const int slot = cl[k];
+      a.tcol[a.eoff[x] + k] = hk[slot];
+      a.tw[a.eoff[x] + k] = hv[slot];
+      hk[slot] = -1;
+      hv[slot] = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      a.ecnt[x] = n;
+      ncnt = 0;
+    }
+    __syncthreads();
+    if (a.T <= R_SLOTS) {
+      for (int64_t j = mb + w; j < me; j += RW) {
+        const int32_t v = a.mem[j];
+        int64_t b, e;
+        slice_range(a.g, v, b, e);
+        for (int64_t q = b + lane; q < e; q += 32) {
+          int32_t sl;
+          long long k;
+          slice_entry(a.g, v, q, sl, k);
+          atomicAdd((ull*)&hv[sl], (ull)k);  // (strengths are positive)
+        }
+      }
+      __syncthreads();
+      for (int sl = threadIdx.x; sl < a.T; sl += RT) {
+        const long long k = hv[sl];
+        if (k == 0) continue;
+        const int at = atomicAdd(&ncnt, 1);
+        a.tsidx[a.soff[x] + at] = sl;
+        a.tsval[a.soff[x] + at] = k;
+        hv[sl] = 0;
+      }
+    } else {
+      for (int64_t j = mb + w; j < me; j += RW) {
+        const int32_t v = a.mem[j];
+        int64_t b, e;
+        slice_range(a.g, v, b, e);
+        for (int64_t q = b + lane; q < e; q += 32) {
+          int32_t sl;
+          long long k;
+          slice_entry(a.g, v, q, sl, k);
+          bool fresh;
+          const int64_t slot = ctab_add(hk, hv, R_SLOTS, sl, k, fresh);
+#if MSLICE_CHECKED
+          if (slot < 0) atomicOr(a.g.chk, ERR_BOUNDS);
+#endif
+          if (fresh) cl[atomicAdd(&ncnt, 1)] = (uint16_t)slot;
+        }
+      }
+      __syncthreads();
+      for (int k = threadIdx.x; k < ncnt; k += RT) {
+        const int slot = cl[k];
+        a.tsidx[a.soff[x] + k] = hk[slot];
+        a.tsval[a.soff[x] + k] = hv[slot];
+        hk[slot] = -1;
+        hv[slot] = 0;
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) a.scnt_out[x] = ncnt;
+    __syncthreads();
+  }
+  for (int32_t x = (nb - 1 - blockIdx.x) * RW + w; x < Np; x += nb * RW)
+    if (max(a.dsum[x], (long long)a.scnt[x]) <= CW_MAX)
+      contract_row_warp(a.g, a.xmap, a.moff, a.mem, x, hk + w * R_PER_WARP, hv + w * R_PER_WARP,
+                        cl + w * (R_PER_WARP / 2), &ncl[w], o);
+  resident_bar();
+  // ---- the rows' final places; the next level's tiers
+  {
+    long long d = 0, c = 0, t;
+    for (int32_t x = lo + threadIdx.x; x < hi; x += RT) {
+      d += a.ecnt[x];
+      c += a.scnt_out[x];
+    }
+    block_scan_excl(d, sm, t);
+    if (threadIdx.x == 0) a.blk[blockIdx.x] = t;
+    block_scan_excl(c, sm, t);
+    if (threadIdx.x == 0) a.blk[nb + blockIdx.x] = t;
+  }
+  resident_bar();
+  long long td, tc;
+  long long ad = blocks_before(a.blk, sm, td), ac = blocks_before(a.blk + nb, sm, tc);
+  for (int32_t base = lo; base < hi; base += RT) {
+    const int32_t x = base + threadIdx.x;
+    const bool in = x < hi;
+    const int n = in ? a.ecnt[x] : 0, ns = in ? a.scnt_out[x] : 0;
+    long long t;
+    const long long rd = block_scan_excl((long long)n, sm, t);
+    if (in) a.rowptr[x] = ad + rd;
+    ad += t;
+    const long long rc = block_scan_excl((long long)ns, sm, t);
+    if (in) a.sptr[x] = ac + rc;
+    ac += t;
+    if (in) {
+      const int tr = work_tier(n, ns, a.cuts);
+      a.tier[x] = (uint8_t)tr;
+      atomicAdd(&tiers[tr], 1);
+    }
+  }
+  __syncthreads();
+  for (int32_t x = lo + w; x < hi; x += RW) {
+    const int64_t from = a.eoff[x], to = a.rowptr[x], sfrom = a.soff[x], sto = a.sptr[x];
+    const int n = a.ecnt[x], ns = a.scnt_out[x];
+    for (int k = lane; k < n; k += 32) {
+      a.col[to + k] = a.tcol[from + k];
+      a.W[to + k] = a.tw[from + k];
+    }
+    for (int k = lane; k < ns; k += 32) {
+      a.sidx[sto + k] = a.tsidx[sfrom + k];
+      a.sval[sto + k] = a.tsval[sfrom + k];
+    }
+  }
+  if (threadIdx.x < NTIERS && tiers[threadIdx.x]) atomicAdd(&a.ctl->tier[threadIdx.x], tiers[threadIdx.x]);
+  if (tid == 0) {
+    a.rowptr[Np] = a.ctl->mu = td;
+    a.sptr[Np] = a.ctl->ms = tc;
+  }
 }
 
 unsigned gsz(int64_t n) {
@@ -552,10 +893,112 @@ unsigned gsz(int64_t n) {
 
 }  // namespace
 
+// What every aggregated level shares with the level it came from.
+static void next_level(const Level& L, Level& next, int32_t Np, int64_t mu, int64_t ms, const int64_t* rowptr,
+                       const int32_t* col, const long long* W, const int64_t* sptr, const int32_t* sidx,
+                       const long long* sval, const int32_t* inst, const int32_t* inst_off) {
+  next = Level{};
+  next.d.N = Np;
+  next.d.is0 = 0;
+  next.d.on = L.d.on;
+  next.d.od = L.d.od;
+  next.d.global_null = L.d.global_null;
+  next.d.on_i = L.d.on_i;
+  next.d.od_i = L.d.od_i;
+  next.d.chk = L.d.chk;
+  next.d.inst = inst;
+  next.d.inst_off = inst_off;
+  next.d.rowptr = rowptr;
+  next.d.col = col;
+  next.d.W = W;
+  next.d.sptr = sptr;
+  next.d.sidx = sidx;
+  next.d.sval = sval;
+  next.nnz = next.nnz_eff = mu;
+  next.ns = ms;
+}
+
+// Levels up to this many work units (entries, and RESIDENT_NODE_WORK a node) are
+// aggregated in one launch.
+constexpr int64_t RESIDENT_AGGREGATE_WORK = (int64_t)1 << 21;
+
+enum class Resident { DONE, SAME, GENERAL };  // SAME: nothing merged; GENERAL: not for one launch
+
+static Resident aggregate_resident(Solver& S, const Level& L, const int32_t* P, Level& next, const std::string& slot,
+                                   int32_t* next_labels, int32_t* node_of0) {
+  Ctx& c = *S.c;
+  const int32_t N = L.d.N;
+  const size_t n1 = (size_t)N + 1, nnz = (size_t)std::max<int64_t>(1, L.nnz), ns = (size_t)std::max<int64_t>(1, L.ns);
+  AggArgs a{};
+  a.g = L.d;
+  a.R = S.R;
+  a.sizeR = S.sizeR;
+  a.P = P;
+  a.T = S.Tn;
+  a.newid = S.tmp32b;
+  a.minid = S.tmp32a;
+  a.xmap = c.ws->get<int32_t>("ag_xmap", N);
+  a.mcnt = c.ws->get<int32_t>("ag_mcnt", n1);
+  a.scnt = c.ws->get<int32_t>("ag_scnt", n1);
+  a.dsum = c.ws->get<long long>("ag_dsum", n1);
+  a.moff = c.ws->get<int64_t>("ag_moff", n1);
+  a.eoff = c.ws->get<int64_t>("ag_eoff", n1);
+  a.soff = c.ws->get<int64_t>("ag_soff", n1);
+  a.mem = c.ws->get<int32_t>("ag_mem", N);
+  a.big = S.freelist;
+  a.tcol = c.ws->get<int32_t>("ag_tcol", nnz);
+  a.tw = c.ws->get<long long>("ag_tw", nnz);
+  a.tsidx = c.ws->get<int32_t>("ag_tsidx", ns);
+  a.tsval = c.ws->get<long long>("ag_tsval", ns);
+  a.ecnt = c.ws->get<int32_t>("ag_ecnt", n1);
+  a.scnt_out = c.ws->get<int32_t>("ag_scnt_out", n1);
+  a.rowptr = c.ws->get<int64_t>(slot + "_rowptr", n1);
+  a.sptr = c.ws->get<int64_t>(slot + "_sptr", n1);
+  a.col = c.ws->get<int32_t>(slot + "_col", nnz);
+  a.W = c.ws->get<long long>(slot + "_W", nnz);
+  a.sidx = c.ws->get<int32_t>(slot + "_sidx", ns);
+  a.sval = c.ws->get<long long>(slot + "_sval", ns);
+  a.next_labels = next_labels;
+  a.B = S.B;
+  if (L.d.inst) {
+    a.inst_next = c.ws->get<int32_t>(slot + "_inst", (size_t)N);
+    a.off_next = c.ws->get<int32_t>(slot + "_ioff", (size_t)S.B + 1);
+  }
+  a.tier = S.tier;
+  a.cuts = S.p.cuts;
+  a.blk = c.ws->get<long long>("ag_blk", 3 * (size_t)S.sms);
+  a.ctl = reinterpret_cast<AggCtl*>(c.ws->get_bytes("ag_ctl", sizeof(AggCtl)));
+  check_cuda(cudaMemsetAsync(a.ctl, 0, sizeof(AggCtl), c.stream), "memset");
+  check_cuda(cudaFuncSetAttribute(k_aggregate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TIER4_SMEM_BYTES),
+             "resident aggregation's shared memory");
+  const int64_t want = std::max<int64_t>((L.nnz + 4095) / 4096, (N + RT - 1) / RT);
+  launch_coop(c, k_aggregate, dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(want, S.sms))), dim3(RT),
+              TIER4_SMEM_BYTES, a);
+  AggCtl h;
+  std::memcpy(&h, readback(c, a.ctl, sizeof(AggCtl)), sizeof(AggCtl));
+  if (h.np == N) return Resident::SAME;
+  if (h.general) return Resident::GENERAL;
+  if (node_of0)
+    launch(c, k_compose, dim3(gsz(S.N0)), dim3(256), 0, (const int32_t*)S.R, (const int32_t*)a.newid, S.N0, node_of0);
+  next_level(L, next, h.np, h.mu, h.ms, a.rowptr, a.col, a.W, a.sptr, a.sidx, a.sval, a.inst_next, a.off_next);
+  // (a level with top-tier nodes still lays out their scratch tables)
+  next.tiers_known = h.tier[NTIERS - 1] == 0;
+  for (int t = 0; t < NTIERS; ++t) next.tier_cnt[t] = h.tier[t];
+  return Resident::DONE;
+}
+
 bool aggregate(Solver& S, const Level& L, const int32_t* P, Level& next, const std::string& slot,
                int32_t* next_labels, int32_t* node_of0, int64_t* checksum) {
   Ctx& c = *S.c;
   const int32_t N = L.d.N;
+  if (L.nnz + RESIDENT_NODE_WORK * (int64_t)N <= RESIDENT_AGGREGATE_WORK) {
+    const Resident r = aggregate_resident(S, L, P, next, slot, next_labels, node_of0);
+    if (r == Resident::SAME) return false;
+    if (r == Resident::DONE) {
+      if (checksum) *checksum = (int64_t)level_checksum(S, next);
+      return true;
+    }
+  }
   // new ids = ranks of the present sub-community labels
   int32_t* flag = S.tmp32a;
   int32_t* newid = S.tmp32b;
@@ -683,33 +1126,15 @@ bool aggregate(Solver& S, const Level& L, const int32_t* P, Level& next, const s
          (const int64_t*)soff, (const int32_t*)scnt_out, (const int64_t*)sptr, (const int32_t*)tsidx,
          (const long long*)tsval, sidx, sval);
 
-  next.d = LevelDev{};
-  next.d.N = Np;
-  next.d.is0 = 0;
-  next.d.on = L.d.on;
-  next.d.od = L.d.od;
-  next.d.global_null = L.d.global_null;
-  next.d.on_i = L.d.on_i;
-  next.d.od_i = L.d.od_i;
-  next.d.chk = L.d.chk;
+  int32_t *inst_next = nullptr, *off_next = nullptr;
   if (L.d.inst) {
-    int32_t* inst_next = c.ws->get<int32_t>(slot + "_inst", (size_t)Np);
-    int32_t* off_next = c.ws->get<int32_t>(slot + "_ioff", (size_t)S.B + 1);
+    inst_next = c.ws->get<int32_t>(slot + "_inst", (size_t)Np);
+    off_next = c.ws->get<int32_t>(slot + "_ioff", (size_t)S.B + 1);
     fill_i32(c, off_next, Np, (int64_t)S.B + 1);
     launch(c, k_next_inst, dim3(gsz(N)), dim3(256), 0, L.d, (const int32_t*)S.R, (const int32_t*)newid, inst_next,
            off_next);
-    next.d.inst = inst_next;
-    next.d.inst_off = off_next;
   }
-  next.d.rowptr = rowptr;
-  next.d.col = col;
-  next.d.W = W;
-  next.nnz = mu;
-  next.nnz_eff = mu;
-  next.d.sptr = sptr;
-  next.d.sidx = sidx;
-  next.d.sval = sval;
-  next.ns = ms;
+  next_level(L, next, Np, mu, ms, rowptr, col, W, sptr, sidx, sval, inst_next, off_next);
 
   // ---- initial labels, level map ----
   int32_t* minid = flag;  // reuse
@@ -719,10 +1144,6 @@ bool aggregate(Solver& S, const Level& L, const int32_t* P, Level& next, const s
          (const int32_t*)minid, N, next_labels);
   if (node_of0)
     launch(c, k_compose, dim3(gsz(S.N0)), dim3(256), 0, (const int32_t*)S.R, (const int32_t*)newid, S.N0, node_of0);
-  int32_t* d_mx = c.ws->get<int32_t>("ag_mx", 1);
-  check_cuda(cudaMemsetAsync(d_mx, 0, sizeof(int32_t), c.stream), "memset");
-  launch(c, k_max_deg, dim3(gsz(Np)), dim3(256), 0, (const int64_t*)rowptr, Np, d_mx);
-  next.max_deg = *static_cast<const int32_t*>(readback(c, d_mx, sizeof(int32_t)));
   if (checksum) *checksum = (int64_t)level_checksum(S, next);
   return true;
 }

@@ -511,7 +511,8 @@ void run_leiden(Ctx& c, const SupraGraph& G, const std::vector<InstParams>& jobs
         break;
       }
       tw[2] = wall();
-      const bool settled = B > 1 ? freeze_settled(S, cur, lab) == 0 : count_distinct(S, lab, cur.d.N) == cur.d.N;
+      const bool settled = B > 1 ? freeze_settled(S, cur, lab) == 0
+                                  : (mo.communities >= 0 ? mo.communities : count_communities(S, cur.d.N)) == cur.d.N;
       tw[3] = wall();
       if (c.trace)
         fprintf(stderr, "[mslice steps] it=%d lvl=%d prepare_ms=%.3f local_move_ms=%.3f count_ms=%.3f\n", it, lvl,

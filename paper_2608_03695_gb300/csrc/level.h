@@ -143,7 +143,10 @@ struct Level {
   int64_t nnz = 0;       // stored entries
   int64_t nnz_eff = 0;   // entries that are edges for this omega
   int64_t ns = 0;        // snapshot-strength entries
-  int32_t max_deg = 0;
+  // nodes per degree tier when the aggregation that made the level found them
+  // (the tiers themselves are then in the solver's tier array)
+  bool tiers_known = false;
+  int32_t tier_cnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 };
 
 }  // namespace mslice

@@ -632,7 +632,7 @@ struct ResidentIn {
   long long max_listed = 0;
 };
 struct ResidentOut {
-  int64_t rounds = 0, moves = 0, last_moved = 0, last_listed = 0;
+  int64_t rounds = 0, moves = 0, last_moved = 0, last_listed = 0, communities = 0;
   ull used = 0;
   unsigned status = 0;
 };

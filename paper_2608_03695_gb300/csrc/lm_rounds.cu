@@ -30,6 +30,7 @@ struct ResidentCtl {
   int32_t empties[2][64];  // moves to empty communities per sub-round
   // results
   long long rounds, moves, last_moved, last_listed;
+  ull communities;  // non-empty at the end
 };
 
 struct ResidentArgs {
@@ -184,6 +185,13 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
     ++r;
     if (moved == 0 || r >= a.r_end || listed > a.max_listed || (a.sig_used && *a.sig_used) || *a.status) break;
   }
+  {
+    int n = 0;
+    for (int64_t v = (int64_t)blockIdx.x * RT + threadIdx.x; v < a.g.N; v += (int64_t)gridDim.x * RT)
+      n += a.size[v] > 0;
+    n = warp_sum(n);
+    if (lane == 0 && n) atomicAdd(&a.ctl->communities, (ull)n);
+  }
   if (blockIdx.x == 0) {
     if (a.inst_moved) {
       const int p = (r - 1) & 1;
@@ -261,12 +269,12 @@ void resident_rounds(Solver& S, const Level& L, int32_t* labels, int it, int lvl
   else
     launch_rounds(c, lm_policy<false>(S, L, labels, trk), a, grid);
   char* h = static_cast<char*>(c.pinned);
-  check_cuda(cudaMemcpyAsync(h, &a.ctl->rounds, 4 * sizeof(long long), cudaMemcpyDeviceToHost, c.stream), "copy");
-  check_cuda(cudaMemcpyAsync(h + 32, S.sig_used, sizeof(ull), cudaMemcpyDeviceToHost, c.stream), "copy");
-  check_cuda(cudaMemcpyAsync(h + 40, c.d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream), "copy");
+  check_cuda(cudaMemcpyAsync(h, &a.ctl->rounds, 5 * sizeof(long long), cudaMemcpyDeviceToHost, c.stream), "copy");
+  check_cuda(cudaMemcpyAsync(h + 40, S.sig_used, sizeof(ull), cudaMemcpyDeviceToHost, c.stream), "copy");
+  check_cuda(cudaMemcpyAsync(h + 48, c.d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream), "copy");
   sync(c);
   struct {
-    long long rounds, moves, last_moved, last_listed;
+    long long rounds, moves, last_moved, last_listed, communities;
     ull used;
     unsigned status;
   } rb;
@@ -275,6 +283,7 @@ void resident_rounds(Solver& S, const Level& L, int32_t* labels, int it, int lvl
   out.moves = rb.moves;
   out.last_moved = rb.last_moved;
   out.last_listed = rb.last_listed;
+  out.communities = rb.communities;
   out.used = rb.used;
   out.status = rb.status;
 }

@@ -226,6 +226,14 @@ __global__ void k_sigma_insert(LevelDev g, const int32_t* labels, SigStore h, in
   }
 }
 
+__global__ void k_count_sizes(const int32_t* size, int64_t N, ull* out) {
+  int n = 0;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x)
+    n += size[v] > 0;
+  n = warp_sum(n);
+  if ((threadIdx.x & 31) == 0 && n) atomicAdd(out, (ull)n);
+}
+
 // Round start (one block) of a tracked round: its tracking state, budgets and
 // counters, and the other parity's accumulators cleared for the round after.
 __global__ void __launch_bounds__(512) k_round_begin(TrackView trk, int32_t* state_prev, int32_t Tn, int first,
@@ -365,6 +373,15 @@ void prepare_level(Solver& S, const Level& L) {
   Ctx& c = *S.c;
   const int32_t N = L.d.N;
   configure_stores(S, N);
+  if (L.tiers_known) {
+    int32_t off = 0;
+    for (int t = 0; t < NTIERS; ++t) {
+      S.tier_cnt[t] = L.tier_cnt[t];
+      S.tier_off[t] = off;
+      off += L.tier_cnt[t];
+    }
+    return;
+  }
   int32_t* cnt = S.cursors;  // reused: tier counts
   check_cuda(cudaMemsetAsync(cnt, 0, NTIERS * sizeof(int32_t), c.stream), "memset");
   int64_t* gsize = reinterpret_cast<int64_t*>(c.ws->get<int64_t>("s_gsize", (size_t)(N > 0 ? N : 1)));
@@ -568,6 +585,15 @@ void bucket(Solver& S, const Level& L, uint64_t tag, int it, int lvl, int r, con
   bucket_tracked(S, L, tag, it, lvl, r, active, TrackView{});
 }
 
+int64_t count_communities(Solver& S, int64_t N) {
+  Ctx& c = *S.c;
+  if (N == 0) return 0;
+  ull* d = c.ws->get<ull>("cd_tot", 1);
+  check_cuda(cudaMemsetAsync(d, 0, sizeof(ull), c.stream), "memset");
+  launch(c, k_count_sizes, dim3(std::min(grid_for(N, 1024), fixed_grid(4))), dim3(256), 0, (const int32_t*)S.size, N, d);
+  return (int64_t)*static_cast<const ull*>(readback(c, d, sizeof(ull)));
+}
+
 // The tracking state of a level (see track.cuh).  Margins live in a
 // refinement array, which is only read after local moving.  Their unit is set
 // so that a node of average strength has about 2^20 of them.
@@ -710,6 +736,7 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
       if (ro.rounds < 1) fail(MSLICE_ECUDA, "resident rounds ran no round");
       moved = ro.last_moved;
       listed = ro.last_listed;
+      out.communities = ro.communities;
       rebuild = !S.sig.d && ro.used > 0;
       if (moved == 0) break;
       if (r >= max_rounds) out.capped = true;
@@ -720,6 +747,7 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
       autotune_cuts(S, L, it, r, active, [&](const TierSegs& sg) { decide(sg, TrackView{}); });
     S.lm_rounds++;
     S.lm_edges += L.nnz_eff;
+    out.communities = -1;
     const bool prof = c.profile && lvl == 0;
     const size_t spans = prof ? c.prof_spans->size() : 0;
     if (prof) c.prof_bytes += 12 * L.nnz_eff + 40 * (int64_t)N;

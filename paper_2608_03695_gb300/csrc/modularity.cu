@@ -201,11 +201,6 @@ __global__ void k_canon(const int32_t* x, const int32_t* first, const int32_t* r
     out[v] = rank[first[x[v]]] - (inst ? rank[inst_off[inst[v]]] : 0);
 }
 
-__global__ void k_mark(const int32_t* x, int64_t N, int32_t* flag) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x)
-    flag[x[v]] = 1;
-}
-
 __global__ void k_checksum(LevelDev g, ull* out) {
   ull h = 0;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < g.N; v += (int64_t)gridDim.x * blockDim.x) {
@@ -277,17 +272,6 @@ void canonicalise(Solver& S, const int32_t* x, int32_t* out, int64_t N) {
   const SupraGraph& G = *S.G0;
   launch(c, k_canon, dim3(gsz(N)), dim3(256), 0, x, (const int32_t*)first, (const int32_t*)rank, N,
          (const int32_t*)G.inst0, (const int32_t*)G.inst_off0, out);
-}
-
-int64_t count_distinct(Solver& S, const int32_t* x, int64_t N) {
-  Ctx& c = *S.c;
-  if (N == 0) return 0;
-  int32_t* flag = S.freelist;
-  check_cuda(cudaMemsetAsync(flag, 0, N * sizeof(int32_t), c.stream), "memset");
-  launch(c, k_mark, dim3(gsz(N)), dim3(256), 0, x, N, flag);
-  int32_t* d_tot = c.ws->get<int32_t>("cd_tot", 1);
-  scan_excl(c, flag, S.tmp32a, N, d_tot);
-  return *static_cast<const int32_t*>(readback(c, d_tot, sizeof(int32_t)));
 }
 
 uint64_t level_checksum(Solver& S, const Level& L) {

@@ -156,6 +156,7 @@ void setup_tracking(Solver& S);
 struct MoveOut {
   int64_t rounds = 0, moves = 0;
   bool capped = false;  // stopped at max_rounds while nodes were still moving
+  int64_t communities = -1;  // non-empty communities at the end (-1: not counted)
 };
 // Local moving of `labels` (N entries, values in [0, N)) at level lvl.
 MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, int max_rounds);
@@ -163,8 +164,9 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
 // Refinement of the local-moving partition P; result in S.R.
 void refine(Solver& S, const Level& L, const int32_t* P, int it, int lvl);
 
-// Number of distinct values in x[0, N) (values in [0, N)).
-int64_t count_distinct(Solver& S, const int32_t* x, int64_t N);
+// Non-empty communities of the level after local_move (from the community
+// sizes it keeps).
+int64_t count_communities(Solver& S, int64_t N);
 
 // Aggregation; returns false when the refined partition has N communities.
 bool aggregate(Solver& S, const Level& L, const int32_t* P, Level& next, const std::string& slot,
