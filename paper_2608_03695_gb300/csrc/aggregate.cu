@@ -533,7 +533,8 @@ __global__ void k_contract_compact(int32_t Np, const int64_t* eoff, const int32_
 
 __global__ void k_min_init(const int32_t* P, const int32_t* R, const int32_t* newid, int32_t N, int32_t* minid) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x)
-    atomicMin(&minid[P[v]], newid[R[v]]);
+    // (looked up first: one atomic a node serialised on large communities)
+    if (newid[R[v]] < __ldcg(&minid[P[v]])) atomicMin(&minid[P[v]], newid[R[v]]);
 }
 
 __global__ void k_next_labels(const int32_t* P, const int32_t* R, const int32_t* newid, const int32_t* minid,
@@ -668,7 +669,7 @@ __global__ void __launch_bounds__(RT, 1) k_aggregate(AggArgs a) {
     int64_t b, e;
     slice_range(a.g, (int32_t)v, b, e);
     if (e > b) atomicAdd(&a.scnt[x], (int32_t)(e - b));
-    atomicMin(&a.minid[a.P[v]], x);
+    if (x < __ldcg(&a.minid[a.P[v]])) atomicMin(&a.minid[a.P[v]], x);
     if (a.inst_next) {
       const int32_t i = a.g.inst[v];
       a.inst_next[x] = i;

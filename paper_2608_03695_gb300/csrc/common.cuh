@@ -118,12 +118,19 @@ __device__ __forceinline__ uint64_t hash_next(uint64_t i, uint64_t base, uint64_
   return (i + 1 == base + size) ? base : i + 1;
 }
 
-// Counts a freshly taken slot against its region (rebuild trigger).
+// Counts a freshly taken slot against its region (rebuild trigger).  Threads of
+// a warp that take slots of the same region together count them with one
+// atomic: the nodes of a level's first table share a few regions, and one atomic
+// each (1.6 M on 16 words) took 0.5 ms where the inserts need 0.1.
 __device__ __forceinline__ void hash_took_slot(const HashView& h, ull key, uint64_t size) {
   if (!h.used) return;
+  const uint32_t s = (uint32_t)key;
+  const unsigned peers = __match_any_sync(__activemask(), s);
+  if ((threadIdx.x & 31) != __ffs(peers) - 1) return;
+  const ull n = (ull)__popc(peers);
   // count the region once, when its taken slots pass half of it
-  const ull taken = atomicAdd(&h.region_used[(uint32_t)key], 1ull) + 1;
-  if (2 * taken > size && 2 * (taken - 1) <= size) atomicAdd(h.used, 1ull);
+  const ull taken = atomicAdd(&h.region_used[s], n) + n;
+  if (2 * taken > size && 2 * (taken - n) <= size) atomicAdd(h.used, 1ull);
 }
 
 __device__ __forceinline__ void hash_add(const HashView& h, ull key, long long delta) {

@@ -193,16 +193,17 @@ __global__ void k_hash_clear(HashView h) {
   }
 }
 
-// Aggregated levels: one warp per node, the lanes sharing its list.
-__global__ void k_sigma_insert_warp(LevelDev g, const int32_t* labels, SigStore h, int32_t* size) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = (((int64_t)blockIdx.x * blockDim.x) >> 5) + (threadIdx.x >> 5); v < g.N; v += warps) {
+// Aggregated levels: G lanes per node, sharing its list.
+template <int G>
+__global__ void k_sigma_insert_group(LevelDev g, const int32_t* labels, SigStore h, int32_t* size) {
+  const int lane = threadIdx.x % G;
+  const int64_t groups = (int64_t)gridDim.x * blockDim.x / G;
+  for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G; v < g.N; v += groups) {
     const int32_t c = labels[v];
     if (size && lane == 0) atomicAdd(&size[c], 1);
     int64_t b, e;
     slice_range(g, (int32_t)v, b, e);
-    for (int64_t j = b + lane; j < e; j += 32) {
+    for (int64_t j = b + lane; j < e; j += G) {
       int32_t s;
       long long k;
       slice_entry(g, (int32_t)v, j, s, k);
@@ -547,8 +548,12 @@ static void rebuild_sigma(Solver& S, const Level& L, const int32_t* labels, bool
   if (N > 0)
     if (L.d.is0)
       launch(c, k_sigma_insert, dim3(grid_for(N, 256)), dim3(256), 0, L.d, labels, S.sig, sizes ? S.size : nullptr);
+    else if (L.ns < 4 * (int64_t)N)  // (lists of one or two entries mostly)
+      launch(c, k_sigma_insert_group<4>, dim3(fixed_grid(8)), dim3(256), 0, L.d, labels, S.sig,
+             sizes ? S.size : nullptr);
     else
-      launch(c, k_sigma_insert_warp, dim3(fixed_grid(8)), dim3(256), 0, L.d, labels, S.sig, sizes ? S.size : nullptr);
+      launch(c, k_sigma_insert_group<32>, dim3(fixed_grid(8)), dim3(256), 0, L.d, labels, S.sig,
+             sizes ? S.size : nullptr);
 }
 
 void sigma_rebuild(Solver& S, const Level& L, const int32_t* labels) { rebuild_sigma(S, L, labels, false); }
