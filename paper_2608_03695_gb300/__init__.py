@@ -536,23 +536,10 @@ def mslice_build(snaps, omega=(1, 1), stream=None, device_ptrs=False, host_tenso
     tensors (``device_ptrs=True``).  ``coupling``: "ordinal" (adjacent
     snapshots) or "categorical" (every pair of snapshots)."""
     T = len(snaps)
-    arr = (Csr * max(T, 1))()
-    keep = []
-    for s, sn in enumerate(snaps):
-        if device_ptrs or host_tensors:
-            ip, ix, w = sn.indptr, sn.indices, sn.weights
-            n = ip.numel() - 1
-        else:
-            ip = np.ascontiguousarray(sn.indptr, dtype=np.int64)
-            ix = np.ascontiguousarray(sn.indices, dtype=np.int32)
-            w = np.ascontiguousarray(sn.weights, dtype=np.int32)
-            n = len(ip) - 1
-        keep += [ip, ix, w]
-        arr[s] = Csr(n, _ptr(ip).value, _ptr(ix).value if _ptr(ix) is not None else None,
-                     _ptr(w).value if _ptr(w) is not None else None)
+    arr, keep = _csr_array(snaps, device_ptrs, host_tensors)
     h = C.c_void_p()
     st = C.c_void_p(stream) if stream is not None else None
-    _check(lib().mslice_build_ex(C.cast(arr, C.c_void_p), T, _COUPLINGS[coupling], omega[0], omega[1],
+    _check(lib().mslice_build_ex(_ptr(arr), T, _COUPLINGS[coupling], omega[0], omega[1],
                                  MSLICE_DEVICE_PTRS if device_ptrs else 0, st, C.byref(h)), "mslice_build_ex")
     return Handle(h, keep)
 
@@ -560,23 +547,46 @@ def mslice_build(snaps, omega=(1, 1), stream=None, device_ptrs=False, host_tenso
 build_graph = mslice_build
 
 
+_I64, _I32 = np.dtype(np.int64), np.dtype(np.int32)
+
+
+def _flat(a, dtype):
+    """`a` itself when it is such a contiguous array already."""
+    if type(a) is np.ndarray and a.dtype == dtype and a.flags.c_contiguous:
+        return a
+    return np.ascontiguousarray(a, dtype=dtype)
+
+
+def _address(a):
+    """Address of an array's data: through the buffer protocol, a quarter of the
+    time of ``a.ctypes.data``, where that works (not read-only, not empty)."""
+    try:
+        return C.addressof(C.c_char.from_buffer(a))
+    except (TypeError, ValueError, BufferError):
+        return a.ctypes.data
+
+
+def _tensor_address(a):
+    return 0 if a is None else a.data_ptr()
+
+
 def _csr_array(snaps, device_ptrs=False, host_tensors=False):
-    T = len(snaps)
-    arr = (Csr * max(T, 1))()
-    keep = []
-    for s, sn in enumerate(snaps):
-        if device_ptrs or host_tensors:
+    """The snapshots as an array of ``mslice_csr`` (four words each: n and three
+    addresses) and the arrays that it points into.  Filled as one integer array:
+    a ctypes structure and three pointer objects per snapshot took 9 us, 66 ms
+    of a sequence of 7,375 snapshots (now under 3 us)."""
+    keep, rows = [], []
+    if device_ptrs or host_tensors:
+        for sn in snaps:
             ip, ix, w = sn.indptr, sn.indices, sn.weights
-            n = ip.numel() - 1
-        else:
-            ip = np.ascontiguousarray(sn.indptr, dtype=np.int64)
-            ix = np.ascontiguousarray(sn.indices, dtype=np.int32)
-            w = np.ascontiguousarray(sn.weights, dtype=np.int32)
-            n = len(ip) - 1
-        keep += [ip, ix, w]
-        arr[s] = Csr(n, _ptr(ip).value, _ptr(ix).value if _ptr(ix) is not None else None,
-                     _ptr(w).value if _ptr(w) is not None else None)
-    return arr, keep
+            keep += [ip, ix, w]
+            rows.append((ip.numel() - 1, _tensor_address(ip), _tensor_address(ix), _tensor_address(w)))
+    else:
+        for sn in snaps:
+            ip, ix, w = _flat(sn.indptr, _I64), _flat(sn.indices, _I32), _flat(sn.weights, _I32)
+            keep += [ip, ix, w]
+            rows.append((len(ip) - 1, _address(ip), _address(ix), _address(w)))
+    return np.array(rows or [(0, 0, 0, 0)], dtype=np.int64), keep
 
 
 def mslice_leiden_windowed(snaps, W, stride, gamma=(1, 1), omega=(1, 1), null="multislice", n_iterations=2, K=4,
@@ -601,7 +611,7 @@ def mslice_leiden_windowed(snaps, W, stride, gamma=(1, 1), omega=(1, 1), null="m
     nw = C.c_int32(0)
     st = Stats()
     s = C.c_void_p(stream) if stream is not None else None
-    _check(lib().mslice_leiden_windowed(C.cast(arr, C.c_void_p), T, W, stride, C.byref(o), s, _ptr(labels),
+    _check(lib().mslice_leiden_windowed(_ptr(arr), T, W, stride, C.byref(o), s, _ptr(labels),
                                         _ptr(Qw), cap, C.byref(nw), C.byref(st)), "mslice_leiden_windowed")
     del keep
     return labels[: n * T].copy(), [float(x) for x in Qw[: nw.value]], _stats_dict(st)
