@@ -61,7 +61,41 @@ __device__ __forceinline__ int32_t coupling_flag(int32_t coupling, int32_t T, in
 // The searches bound the pass (about four dependent lookups each, a few rows
 // away in L2); checking and copying apart, with a search per entry and a scan
 // for the row pointers, took 1.6 ms for 31 M entries.
+// Rows of more than BUILD_LONG entries are taken by the whole warp: with 8 lanes
+// a row of 1,400 entries alone took as long as the rest of the pass.
 constexpr int BUILD_LANES = 8;
+constexpr int64_t BUILD_LONG = 64;
+
+// Entries gl, gl + step, ... of row i of a snapshot (entries [a, b)): checked and
+// written at out.
+__device__ __forceinline__ void build_entries(const int64_t* ip, const int32_t* ix, const int32_t* wt, int32_t n,
+                                              int32_t i, int64_t a, int64_t b, int2* out, int32_t off, int gl, int step,
+                                              long long& ksum, int& above, bool& bad) {
+  for (int64_t e = a + gl; e < b; e += step) {
+    const int32_t j = ix[e];
+    const int32_t w = wt[e];
+    out[e - a] = make_int2(j + off, w);
+    ksum += w;
+    if (j < 0 || j >= n || j == i || w < 1) {
+      bad = true;
+      continue;
+    }
+    if (e > a && ix[e - 1] >= j) bad = true;
+    above += j > i ? 1 : -1;
+    if (j < i) continue;
+    // binary search for i in row j
+    int64_t x = ip[j], y = ip[j + 1];
+    const int64_t end = y;
+    while (x < y) {
+      const int64_t mid = (x + y) >> 1;
+      if (ix[mid] < i)
+        x = mid + 1;
+      else
+        y = mid;
+    }
+    if (x >= end || ix[x] != i || wt[x] != w) bad = true;
+  }
+}
 
 __global__ void k_build_rows(SliceTable st, int32_t T, int64_t n, int32_t coupling, const int64_t* first,
                              int64_t* rowptr, int2* adj, int64_t* k, ull* balance, unsigned* status) {
@@ -69,58 +103,55 @@ __global__ void k_build_rows(SliceTable st, int32_t T, int64_t n, int32_t coupli
   const int lane = threadIdx.x & 31, gl = lane % BUILD_LANES;
   const unsigned gmask = ((1u << BUILD_LANES) - 1u) << (lane - gl);
   const int64_t groups = (int64_t)gridDim.x * blockDim.x / BUILD_LANES;
-  long long above = 0;
+  const int32_t n32 = (int32_t)n;
+  long long above_sum = 0;
   bool bad = false;
-  for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / BUILD_LANES; v < total; v += groups) {
-    const int32_t s = (int32_t)(v / n);
-    const int64_t i = v - (int64_t)s * n;
+  // (warp-uniform loop)
+  for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / BUILD_LANES; v0 < total; v0 += groups) {
+    const int64_t v = v0 + lane / BUILD_LANES;
+    const bool ok = v < total;
+    const int32_t s = ok ? (int32_t)v / n32 : 0, i = ok ? (int32_t)v - s * n32 : 0;
     const int64_t* ip = st.indptr[s];
-    const int32_t* ix = st.indices[s];
-    const int32_t* wt = st.weights[s];
-    const int64_t a = ip[i], b = ip[i + 1];
+    const int64_t a = ok ? ip[i] : 0, b = ok ? ip[i + 1] : 0;
     int32_t lo, hi;
     coupled_range(coupling, T, s, lo, hi);
     int64_t out = first[s] + a + i * (int64_t)(hi - lo - 1);
-    if (gl == 0) rowptr[v] = out;
-    for (int32_t r = lo + gl; r < s; r += BUILD_LANES)
-      adj[out + (r - lo)] = make_int2((int32_t)((int64_t)r * n + i), coupling_flag(coupling, T, s, r));
-    out += s - lo;
-    const int32_t off = (int32_t)((int64_t)s * n);
+    const int32_t off = s * n32;
     long long ksum = 0;
-    for (int64_t e = a + gl; e < b; e += BUILD_LANES) {
-      const int32_t j = ix[e];
-      const int32_t w = wt[e];
-      adj[out + (e - a)] = make_int2(j + off, w);
-      ksum += w;
-      if (j < 0 || j >= n || j == i || w < 1) {
-        bad = true;
-        continue;
-      }
-      if (e > a && ix[e - 1] >= j) bad = true;
-      above += j > i ? 1 : -1;
-      if (j < i) continue;
-      // binary search for i in row j
-      int64_t x = ip[j], y = ip[j + 1];
-      const int64_t end = y;
-      while (x < y) {
-        const int64_t mid = (x + y) >> 1;
-        if (ix[mid] < i)
-          x = mid + 1;
-        else
-          y = mid;
-      }
-      if (x >= end || ix[x] != i || wt[x] != w) bad = true;
+    int above = 0;
+    if (ok) {
+      if (gl == 0) rowptr[v] = out;
+      for (int32_t r = lo + gl; r < s; r += BUILD_LANES)
+        adj[out + (r - lo)] = make_int2(r * n32 + i, coupling_flag(coupling, T, s, r));
+      out += s - lo;
+      for (int32_t r = s + 1 + gl; r < hi; r += BUILD_LANES)
+        adj[out + (b - a) + (r - s - 1)] = make_int2(r * n32 + i, coupling_flag(coupling, T, s, r));
+      if (b - a <= BUILD_LONG)
+        build_entries(ip, st.indices[s], st.weights[s], n32, i, a, b, adj + out, off, gl, BUILD_LANES, ksum, above,
+                      bad);
+    }
+    unsigned wide = __ballot_sync(0xffffffffu, gl == 0 && b - a > BUILD_LONG);
+    while (wide) {
+      const int src = __ffs(wide) - 1;
+      wide &= wide - 1;
+      const int32_t ss = __shfl_sync(0xffffffffu, s, src), is = __shfl_sync(0xffffffffu, i, src);
+      const int64_t as = __shfl_sync(0xffffffffu, a, src), bs = __shfl_sync(0xffffffffu, b, src),
+                    os = __shfl_sync(0xffffffffu, out, src);
+      long long kw = 0;
+      build_entries(st.indptr[ss], st.indices[ss], st.weights[ss], n32, is, as, bs, adj + os, ss * n32, lane, 32, kw,
+                    above, bad);
+      kw = warp_sum(kw);
+      if (lane == src) ksum = kw;  // (the others of the group hold 0)
     }
 #pragma unroll
     for (int m = BUILD_LANES / 2; m >= 1; m >>= 1) ksum += __shfl_xor_sync(gmask, ksum, m);
-    for (int32_t r = s + 1 + gl; r < hi; r += BUILD_LANES)
-      adj[out + (b - a) + (r - s - 1)] = make_int2((int32_t)((int64_t)r * n + i), coupling_flag(coupling, T, s, r));
-    if (gl == 0) k[v] = ksum;
+    if (ok && gl == 0) k[v] = ksum;
+    above_sum += above;
   }
-  above = warp_sum(above);
+  above_sum = warp_sum(above_sum);
   const bool any = __any_sync(0xffffffffu, bad);
   if (lane == 0) {
-    if (above) atomicAdd(balance, (ull)above);
+    if (above_sum) atomicAdd(balance, (ull)above_sum);
     if (any) atomicOr(status, ERR_BAD_INPUT);
   }
 }

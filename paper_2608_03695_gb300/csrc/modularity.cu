@@ -31,41 +31,68 @@ namespace mslice {
 
 namespace {
 
-// I and J of every instance (IJ: 2 words per instance).  A warp's rows ascend,
-// and so do their instances: sums go out when the instance changes and at the
-// end (one atomic a row on B words took 1.5 ms of a batch of 36, N = 1.5 M).
-__global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  ull I = 0, J = 0;
-  int32_t cur = 0;  // instance the sums belong to
-  auto flush = [&] {
-    I = warp_sum(I);
-    J = warp_sum(J);
-    if (lane == 0) {
-      if (I) atomicAdd(&IJ[2 * cur], I);
-      if (J) atomicAdd(&IJ[2 * cur + 1], J);
+// I and J of every instance (IJ: 2 words per instance): 8 lanes a row, the whole
+// warp for a row of more than 64 entries.  A warp's rows ascend, and so do their
+// instances: sums go out when the instance changes and at the end (one atomic a
+// row on B words took 1.5 ms of a batch of 36, N = 1.5 M).
+__device__ __forceinline__ void ij_row(const LevelDev& g, const int32_t* labels, int32_t c, int64_t b, int64_t e,
+                                       int t, int nt, ull& I, ull& J) {
+  for (int64_t q = b + t; q < e; q += nt) {
+    const int2 x = g.adj0[q];
+    if (labels[x.x] == c) {
+      if (x.y > 0)
+        I += (ull)x.y;
+      else
+        J += g.cw ? (ull)g.cw[-x.y - 1] : 1ull;  // weighted by the pair's numerator with a table
     }
+  }
+}
+
+__global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B) {
+  constexpr int G = 8;
+  constexpr int64_t LONG = 64;
+  const int lane = threadIdx.x & 31, gl = lane % G;
+  const int64_t groups = (int64_t)gridDim.x * blockDim.x / G;
+  ull I = 0, J = 0;
+  int32_t cur = 0;  // instance the lane's sums belong to
+  auto flush = [&] {
+    if (I) atomicAdd(&IJ[2 * cur], I);
+    if (J) atomicAdd(&IJ[2 * cur + 1], J);
     I = J = 0;
   };
-  for (int64_t v = (((int64_t)blockIdx.x * blockDim.x) >> 5) + (threadIdx.x >> 5); v < g.N; v += warps) {
-    const int32_t c = labels[v];
-    const int32_t inst = B > 1 ? node_inst(g, (int32_t)v) : 0;
+  for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G; v0 < g.N; v0 += groups) {
+    const int64_t v = v0 + lane / G;
+    const bool ok = v < g.N;
+    const int64_t b = ok ? g.rowptr[v] : 0, e = ok ? g.rowptr[v + 1] : 0;
+    const int32_t c = ok ? labels[v] : 0;
+    const int32_t inst = ok && B > 1 ? node_inst(g, (int32_t)v) : cur;
     if (inst != cur) {
       flush();
       cur = inst;
     }
-    for (int64_t e = g.rowptr[v] + lane; e < g.rowptr[v + 1]; e += 32) {
-      const int2 x = g.adj0[e];
-      if (labels[x.x] == c) {
-        if (x.y > 0)
-          I += (ull)x.y;
-        else
-          J += g.cw ? (ull)g.cw[-x.y - 1] : 1ull;  // weighted by the pair's numerator with a table
+    if (e - b <= LONG) ij_row(g, labels, c, b, e, gl, G, I, J);
+    unsigned wide = __ballot_sync(0xffffffffu, gl == 0 && e - b > LONG);
+    while (wide) {
+      const int src = __ffs(wide) - 1;
+      wide &= wide - 1;
+      ull Iw = 0, Jw = 0;
+      ij_row(g, labels, __shfl_sync(0xffffffffu, c, src), __shfl_sync(0xffffffffu, b, src),
+             __shfl_sync(0xffffffffu, e, src), lane, 32, Iw, Jw);
+      Iw = warp_sum(Iw);
+      Jw = warp_sum(Jw);
+      if (lane == src) {
+        I += Iw;
+        J += Jw;
       }
     }
   }
-  flush();
+  if (B == 1) {
+    I = warp_sum(I);
+    J = warp_sum(J);
+    if (lane == 0) flush();
+  } else {
+    flush();
+  }
 }
 
 // S_s += Sigma_{c,s}^2 over the table; per-block partial sums in shared
@@ -250,7 +277,7 @@ void modularity(Solver& S, const int32_t* labels0, double* Q) {
   }
   check_cuda(cudaMemcpyAsync(dqi, qi.data(), B * sizeof(QInst), cudaMemcpyHostToDevice, c.stream), "copy");
   check_cuda(cudaMemsetAsync(acc, 0, (2 * (size_t)B + 2 * (size_t)Tn) * sizeof(ull), c.stream), "memset");
-  if (G.N > 0) launch(c, k_IJ, dim3(gsz(G.N * 32)), dim3(256), 0, g, labels0, acc, B);
+  if (G.N > 0) launch(c, k_IJ, dim3(gsz(G.N * 8)), dim3(256), 0, g, labels0, acc, B);
   const size_t smem = Tn <= 1024 ? 2 * (size_t)Tn * sizeof(ull) : 0;
   const int64_t span = S.sig.d ? S.sig.rows * S.sig.T : (int64_t)S.sig.h.cap;
   launch(c, k_S, dim3(gsz(span)), dim3(256), smem, S.sig, Tn, acc + 2 * B);

@@ -30,6 +30,8 @@ __device__ __forceinline__ u128 lam_k_x(const u128* lam, int32_t s, long long k,
 // node (G = 32 at aggregated levels, whose long (snapshot, strength) lists
 // the lanes share; fewer at level 0, whose rows are short and whose nodes
 // hold one snapshot each, so a warp takes several nodes at once).
+constexpr int64_t REF_LONG_ROW = 64;  // longer rows are summed by the whole warp
+
 template <int G>
 __device__ __forceinline__ void ref_init(const LevelDev& g, const int32_t* P, const SigStore& sig, const u128* lam,
                                          int32_t* R, int32_t* sizeR, long long* Wc, long long* Wout, uint8_t* elig,
@@ -46,12 +48,32 @@ __device__ __forceinline__ void ref_init(const LevelDev& g, const int32_t* P, co
     const int32_t C = ok ? P[v] : 0;
     const Omega om = ok ? node_omega(g, (int32_t)v) : Omega{1, 1};
     long long w = 0;
-    if (ok)
-      for (int64_t e = g.rowptr[v] + gl; e < g.rowptr[v + 1]; e += G) {
+    const int64_t rb = ok ? g.rowptr[v] : 0, re = ok ? g.rowptr[v + 1] : 0;
+    const bool wide_row = G < 32 && re - rb > REF_LONG_ROW;
+    if (!wide_row)
+      for (int64_t e = rb + gl; e < re; e += G) {
         int32_t u;
         long long W;
         if (edge_at(g, e, u, W, om) && P[u] == C) w += W;
       }
+    if constexpr (G < 32) {
+      unsigned wide = __ballot_sync(0xffffffffu, gl == 0 && wide_row);
+      while (wide) {
+        const int src = __ffs(wide) - 1;
+        wide &= wide - 1;
+        const int64_t bs = __shfl_sync(0xffffffffu, rb, src), es = __shfl_sync(0xffffffffu, re, src);
+        const int32_t Cs = __shfl_sync(0xffffffffu, C, src);
+        const Omega os{__shfl_sync(0xffffffffu, om.on, src), __shfl_sync(0xffffffffu, om.od, src)};
+        long long ww = 0;
+        for (int64_t e = bs + lane; e < es; e += 32) {
+          int32_t u;
+          long long W;
+          if (edge_at(g, e, u, W, os) && P[u] == Cs) ww += W;
+        }
+        ww = warp_sum(ww);
+        if (lane == src) w = ww;
+      }
+    }
 #pragma unroll
     for (int m = G / 2; m >= 1; m >>= 1) w += __shfl_xor_sync(gmask, w, m);
     // a long (snapshot, strength) list is shared by the lanes of the group;
