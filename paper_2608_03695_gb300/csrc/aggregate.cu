@@ -82,7 +82,7 @@ __global__ void k_contract_tier(int32_t Np, const long long* dsum, const int32_t
   }
 }
 
-// Insert-or-add into a table of `cap` (a power of two) slots.
+// Insert-or-add into a shared table of `cap` (a power of two) slots.
 __device__ __forceinline__ int64_t ctab_add(int32_t* hk, long long* hv, int64_t cap, int32_t key, long long w,
                                             bool& fresh) {
   const uint64_t mask = (uint64_t)cap - 1;
@@ -91,7 +91,7 @@ __device__ __forceinline__ int64_t ctab_add(int32_t* hk, long long* hv, int64_t 
   for (uint64_t p = 0; p <= mask; ++p) {
     const int32_t prev = atomicCAS(&hk[i], -1, key);
     if (prev == -1 || prev == key) {
-      atomicAdd((ull*)&hv[i], (ull)w);
+      shared_add64(&hv[i], w);
       fresh = prev == -1;
       return (int64_t)i;
     }
@@ -377,7 +377,7 @@ __device__ __forceinline__ bool stab_add(int32_t* K, long long* V, uint16_t* L, 
   for (int p = 0; p < BI_PROBES; ++p) {
     const int32_t prev = atomicCAS(&K[i], -1, key);
     if (prev == -1 || prev == key) {
-      atomicAdd((ull*)&V[i], (ull)w);
+      shared_add64(&V[i], w);
       if (prev == -1) L[atomicAdd(n, 1)] = (uint16_t)i;
       return true;
     }
@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(RT, 1) k_aggregate(AggArgs a) {
           int32_t sl;
           long long k;
           slice_entry(a.g, v, q, sl, k);
-          atomicAdd((ull*)&hv[sl], (ull)k);  // (strengths are positive)
+          shared_add64(&hv[sl], k);  // (strengths are positive)
         }
       }
       __syncthreads();

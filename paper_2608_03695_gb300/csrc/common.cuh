@@ -118,6 +118,17 @@ __device__ __forceinline__ uint64_t hash_next(uint64_t i, uint64_t base, uint64_
   return (i + 1 == base + size) ? base : i + 1;
 }
 
+// 64-bit add to shared memory as 32-bit adds: the low word's carry goes to the
+// high word with the high half.  (Shared memory adds 32-bit words in place; a
+// 64-bit atomicAdd is a compare-and-swap loop, which serialises on the slot that
+// most of a node's entries share.)  Sums are complete after the next barrier.
+__device__ __forceinline__ void shared_add64(long long* p, long long x) {
+  unsigned* w = reinterpret_cast<unsigned*>(p);
+  const unsigned lo = (unsigned)x, old = atomicAdd(w, lo);
+  const unsigned hi = (unsigned)((ull)x >> 32) + (old + lo < old ? 1u : 0u);
+  if (hi) atomicAdd(w + 1, hi);
+}
+
 // Counts a freshly taken slot against its region (rebuild trigger).  Threads of
 // a warp that take slots of the same region together count them with one
 // atomic: the nodes of a level's first table share a few regions, and one atomic

@@ -193,7 +193,7 @@ __device__ __forceinline__ int table_add_slot(int32_t* hk, long long* hv, int bi
   for (uint32_t p = 0; p <= mask; ++p) {
     const int32_t prev = atomicCAS(&hk[i], -1, key);
     if (prev == -1 || prev == key) {
-      atomicAdd((ull*)&hv[i], (ull)w);
+      shared_add64(&hv[i], w);
       fresh = prev == -1;
       return (int)i;
     }
