@@ -233,36 +233,95 @@ __device__ __forceinline__ void track_moved(const TrackView& trk, int32_t s, lon
   if (old + k > trk.B[s]) trk.state[TRACK_PAST] = 1;
 }
 
-// A mover's warp takes the move off the margins of the mover's neighbours; a
-// settled one that has to decide after all joins the list of its class when
-// that is still to come in this round (it decides in the next one otherwise:
-// its class has been decided, from the state before this move).
-__device__ __forceinline__ void track_push(const TrackView& trk, const LevelDev& g, const int32_t* labels,
-                                           const BucketLists& bl, int q, int32_t v, int32_t from, int32_t to,
-                                           int64_t rb, int64_t re, int lane) {
-  const Omega om = node_omega(g, v);
-  for (int64_t e = rb + lane; e < re; e += 32) {
-    int32_t u;
-    long long w;
-    if (!edge_at(g, e, u, w, om)) continue;
-    // (the label of a neighbour that moves in this sub-round may be read before
-    // or after its move: that neighbour has to decide either way)
-    const long long d = track_drop(trk, labels[u], from, to, w);
-    if (*(volatile long long*)&trk.slack[u] < 0) continue;
-    const long long old = (long long)atomicAdd((ull*)&trk.slack[u], (ull)(-d));
-    if (old >= 0 && old < d) {
-      const int sg = bl.seg[u];
-      if ((sg & SEG_SETTLED) && sg != SEG_FROZEN) {
-        const int sgu = sg & ~(int)SEG_SETTLED;
-        if (sgu / NTIERS > q) bucket_append(bl, sgu, u);
-      }
+// One neighbour u of a mover (from, to) over weight w; see track_push.
+__device__ __forceinline__ void track_push_one(const TrackView& trk, const BucketLists& bl, int q, int32_t u,
+                                               long long d, long long slack) {
+  if (slack < 0) return;
+  const long long old = (long long)atomicAdd((ull*)&trk.slack[u], (ull)(-d));
+  if (old >= 0 && old < d) {
+    const int sg = bl.seg[u];
+    if ((sg & SEG_SETTLED) && sg != SEG_FROZEN) {
+      const int sgu = sg & ~(int)SEG_SETTLED;
+      if (sgu / NTIERS > q) bucket_append(bl, sgu, u);
     }
   }
 }
 
-__device__ __forceinline__ bool seg_item(const TierSegs& sg, int64_t idx, int32_t& v) {
+// A warp takes its movers' moves off the margins of their neighbours; a settled
+// one that has to decide after all joins the list of its class when that is still
+// to come in this round (it decides in the next one otherwise: its class has been
+// decided, from the state before this move).  (The label of a neighbour that moves
+// in this sub-round may be read before or after its move: that neighbour has to
+// decide either way.)  The movers' rows are dealt to the lanes as one sequence,
+// four entries a lane at a time, so that the loads of four neighbours are in
+// flight: mover by mover, a warp with a few hubs held the sub-round for 0.3 ms.
+// All lanes of the warp call it; a lane without a mover has no entries.
+__device__ __forceinline__ void track_push(const TrackView& trk, const LevelDev& g, const int32_t* labels,
+                                           const BucketLists& bl, int q, int32_t v, int32_t from, int32_t to,
+                                           int64_t rb, int64_t re, int lane) {
+  constexpr int U = 4;
+  const Omega om = re > rb ? node_omega(g, v) : Omega{g.on, g.od};
+  if (__any_sync(0xffffffffu, re - rb > (1 << 25))) {  // (their sum must fit 32 bits)
+    for (int src = 0; src < 32; ++src) {
+      const int32_t f = __shfl_sync(0xffffffffu, from, src), t = __shfl_sync(0xffffffffu, to, src);
+      const int64_t b = __shfl_sync(0xffffffffu, rb, src), e = __shfl_sync(0xffffffffu, re, src);
+      const Omega os{__shfl_sync(0xffffffffu, om.on, src), __shfl_sync(0xffffffffu, om.od, src)};
+      for (int64_t x = b + lane; x < e; x += 32) {
+        int32_t u;
+        long long w;
+        if (edge_at(g, x, u, w, os))
+          track_push_one(trk, bl, q, u, track_drop(trk, labels[u], f, t, w), *(volatile long long*)&trk.slack[u]);
+      }
+    }
+    return;
+  }
+  int incl = (int)(re - rb);
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += y;
+  }
+  const int total = __shfl_sync(0xffffffffu, incl, 31);
+  for (int i0 = 0; i0 < total; i0 += 32 * U) {
+    int32_t us[U], fs[U], ts[U], cs[U];
+    long long ws[U], sl[U];
+    bool ok[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int i = i0 + 32 * k + lane;
+      int m = 0;  // the mover whose entry i is: the lanes before it hold at most i
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1)
+        if (__shfl_sync(0xffffffffu, incl, m + d - 1) <= i) m += d;
+      m = min(m, 31);
+      const int before = __shfl_sync(0xffffffffu, incl, m > 0 ? m - 1 : 0);
+      fs[k] = __shfl_sync(0xffffffffu, from, m);
+      ts[k] = __shfl_sync(0xffffffffu, to, m);
+      const int64_t b = __shfl_sync(0xffffffffu, rb, m);
+      Omega os = om;
+      if (g.od_i) {
+        os.on = __shfl_sync(0xffffffffu, om.on, m);
+        os.od = __shfl_sync(0xffffffffu, om.od, m);
+      }
+      ok[k] = i < total && edge_at(g, b + (i - (m > 0 ? before : 0)), us[k], ws[k], os);
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (ok[k]) {
+        cs[k] = labels[us[k]];
+        sl[k] = *(volatile long long*)&trk.slack[us[k]];
+      }
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (ok[k]) track_push_one(trk, bl, q, us[k], track_drop(trk, cs[k], fs[k], ts[k], ws[k]), sl[k]);
+  }
+}
+
+// Node idx of the lists of tiers [t0, t1), and their length.
+__device__ __forceinline__ bool seg_item(const TierSegs& sg, int t0, int t1, int64_t idx, int32_t& v) {
 #pragma unroll
   for (int t = 0; t < NTIERS; ++t) {
+    if (t < t0 || t >= t1) continue;
     const int cnt = *sg.count[t];
     if (idx < cnt) {
       v = sg.list[t][idx];
@@ -273,10 +332,11 @@ __device__ __forceinline__ bool seg_item(const TierSegs& sg, int64_t idx, int32_
   return false;
 }
 
-__device__ __forceinline__ int seg_total(const TierSegs& sg) {
+__device__ __forceinline__ int seg_total(const TierSegs& sg, int t0, int t1) {
   int t = 0;
 #pragma unroll
-  for (int i = 0; i < NTIERS; ++i) t += *sg.count[i];
+  for (int i = 0; i < NTIERS; ++i)
+    if (i >= t0 && i < t1) t += *sg.count[i];
   return t;
 }
 
@@ -287,76 +347,78 @@ __device__ __forceinline__ int seg_total(const TierSegs& sg) {
 __device__ __forceinline__ void lm_apply(const LevelDev& g, const TierSegs& sg, int32_t* labels, int32_t* size,
                                          const SigStore& sig, int32_t* target, ull* moved, int32_t* empties,
                                          int32_t* inst_moved, const TrackView& trk, const BucketLists& bl, int q) {
-  const int total = seg_total(sg);
   const bool track = track_mode(trk) != TRACK_OFF;
   const int lane = threadIdx.x & 31;
-  // List items a warp takes at a time: 32, but a tracked round deals a short
-  // list out to all warps, as a warp pushes its movers one after another.
-  const int warps = gridDim.x * (blockDim.x >> 5);
-  const int take = track ? min(32, (total + warps - 1) / warps) : 32;
+  const int warps = gridDim.x * (blockDim.x >> 5), warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   int local = 0, local_empty = 0;
-  for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * take; base < total;
-       base += (int64_t)warps * take) {
-    const int64_t idx = base + lane;
-    int32_t v = 0, t = NO_MOVE, a = 0;
-    int64_t b = 0, e = 0, rb = 0, re = 0;
-    if (lane < take && idx < total && seg_item(sg, idx, v)) t = target[v];
+  // A warp takes 32 list items at a time.  A tracked round walks its movers'
+  // rows as well: there the tiers come one after another, heaviest first, fewer
+  // items at a time, and a short list is dealt out to all warps.
+  int used = 0;  // claims of the tiers before: the next tiers' start with other warps
+  for (int part = 0; part < (track ? 3 : 1); ++part) {
+    const int t0 = !track ? 0 : part == 0 ? 3 : part == 1 ? 2 : 0;
+    const int t1 = !track || part == 0 ? NTIERS : part == 1 ? 3 : 2;
+    const int total = seg_total(sg, t0, t1);
+    const int most = !track || part == 2 ? 32 : part == 1 ? 4 : 1;
+    const int take = track ? max(1, min(most, (total + warps - 1) / warps)) : 32;
+    const int first = (warp + warps - used % warps) % warps;
+    used += (total + take - 1) / take;
+    for (int64_t base = (int64_t)first * take; base < total; base += (int64_t)warps * take) {
+      const int64_t idx = base + lane;
+      int32_t v = 0, t = NO_MOVE, a = 0;
+      int64_t b = 0, e = 0, rb = 0, re = 0;
+      if (lane < take && idx < total && seg_item(sg, t0, t1, idx, v)) t = target[v];
 #if MSLICE_CHECKED
-    if (t != NO_MOVE && (t >= g.N || (t < 0 && t != TO_EMPTY))) {
-      atomicOr(g.chk, ERR_BOUNDS);
-      t = NO_MOVE;
-    }
+      if (t != NO_MOVE && (t >= g.N || (t < 0 && t != TO_EMPTY))) {
+        atomicOr(g.chk, ERR_BOUNDS);
+        t = NO_MOVE;
+      }
 #endif
-    if (t != NO_MOVE) {
-      if (inst_moved) inst_moved[node_inst(g, v)] = 1;
-      a = labels[v];
-      atomicSub(&size[a], 1);
-      slice_range(g, v, b, e);
-      if (g.is0 && e > b) {
-        const int32_t s = node_slice0(g, v);
-        const long long k = g.k0[v];
-        ss_add(sig, a, s, -k);
-        if (t >= 0) ss_add(sig, t, s, k);
-      }
-      if (track) {
-        rb = g.rowptr[v];
-        re = g.rowptr[v + 1];
-        trk.slack[v] = TRACK_DEAD;
-      }
-    }
-    if (track) {
-      const unsigned mv = __ballot_sync(0xffffffffu, t != NO_MOVE);
-      if (mv && g.is0) {
-        const int32_t s = t != NO_MOVE ? node_slice0(g, v) : -1;
-        const long long k = t != NO_MOVE ? g.k0[v] : 0;
-        const int32_t s0 = __shfl_sync(0xffffffffu, s, __ffs(mv) - 1);
-        const long long k0 = warp_sum(s == s0 ? k : 0ll);
-        if (lane == 0) track_moved(trk, s0, k0);
-        if (t != NO_MOVE && s != s0) track_moved(trk, s, k);
-      } else if (t != NO_MOVE) {
-        for (int64_t j = b; j < e; ++j) {
-          int32_t s;
-          long long k;
-          slice_entry(g, v, j, s, k);
-          track_moved(trk, s, k);
+      if (t != NO_MOVE) {
+        if (inst_moved) inst_moved[node_inst(g, v)] = 1;
+        a = labels[v];
+        atomicSub(&size[a], 1);
+        slice_range(g, v, b, e);
+        if (g.is0 && e > b) {
+          const int32_t s = node_slice0(g, v);
+          const long long k = g.k0[v];
+          ss_add(sig, a, s, -k);
+          if (t >= 0) ss_add(sig, t, s, k);
+        }
+        if (track) {
+          rb = g.rowptr[v];
+          re = g.rowptr[v + 1];
+          trk.slack[v] = TRACK_DEAD;
         }
       }
-      for (unsigned m = mv; m; m &= m - 1) {
-        const int src = __ffs(m) - 1;
-        const int32_t vs = __shfl_sync(0xffffffffu, v, src), as = __shfl_sync(0xffffffffu, a, src),
-                      ts = __shfl_sync(0xffffffffu, t, src);
-        const int64_t rbs = __shfl_sync(0xffffffffu, rb, src), res = __shfl_sync(0xffffffffu, re, src);
-        track_push(trk, g, labels, bl, q, vs, as, ts, rbs, res, lane);
+      if (track) {
+        const unsigned mv = __ballot_sync(0xffffffffu, t != NO_MOVE);
+        if (mv && g.is0) {
+          const int32_t s = t != NO_MOVE ? node_slice0(g, v) : -1;
+          const long long k = t != NO_MOVE ? g.k0[v] : 0;
+          const int32_t s0 = __shfl_sync(0xffffffffu, s, __ffs(mv) - 1);
+          const long long k0 = warp_sum(s == s0 ? k : 0ll);
+          if (lane == 0) track_moved(trk, s0, k0);
+          if (t != NO_MOVE && s != s0) track_moved(trk, s, k);
+        } else if (t != NO_MOVE) {
+          for (int64_t j = b; j < e; ++j) {
+            int32_t s;
+            long long k;
+            slice_entry(g, v, j, s, k);
+            track_moved(trk, s, k);
+          }
+        }
+        if (mv) track_push(trk, g, labels, bl, q, v, a, t, rb, re, lane);
       }
-    }
-    if (!g.is0) move_slices(g, sig, v, a, t, b, e, lane);
-    if (t >= 0) {
-      atomicAdd(&size[t], 1);
-      labels[v] = t;
-      target[v] = NO_MOVE;
-      local++;
-    } else if (t == TO_EMPTY) {
-      local_empty++;
+      if (!g.is0) move_slices(g, sig, v, a, t, b, e, lane);
+      if (t >= 0) {
+        atomicAdd(&size[t], 1);
+        labels[v] = t;
+        target[v] = NO_MOVE;
+        local++;
+      } else if (t == TO_EMPTY) {
+        local_empty++;
+      }
     }
   }
   local = warp_sum(local);
@@ -397,25 +459,44 @@ __device__ __forceinline__ T block_scan_excl(T x, T* sm, T& total) {
   return r;
 }
 
-// A pruned round whose movement has passed a budget lets the settled nodes of
-// class q that the passed slices concern rejoin its lists (see track.cuh).
+// A pruned round whose movement has passed a budget: the settled nodes of class q
+// (the next one) whose margin does not cover what their slices have moved past
+// their budgets rejoin its lists (see track.cuh).  Four nodes a thread at a time,
+// and a node's margin is read only when a slice of it has passed its budget.
 __device__ __forceinline__ void track_rescan(const TrackView& trk, const LevelDev& g, const BucketLists& bl, int q) {
-  if (track_mode(trk) == TRACK_PRUNE && trk.state[TRACK_PAST]) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < g.N; v += (int64_t)gridDim.x * blockDim.x) {
-      const int sg = bl.seg[v];
-      if (!(sg & SEG_SETTLED) || sg == SEG_FROZEN) continue;
-      const int sgv = sg & ~(int)SEG_SETTLED;
-      if (sgv / NTIERS != q || trk.slack[v] < 0) continue;
-      int64_t b, e;
-      slice_range(g, (int32_t)v, b, e);
-      bool past = false;
-      for (int64_t j = b; j < e && !past; ++j) {
-        int32_t s;
-        long long k;
-        slice_entry(g, (int32_t)v, j, s, k);
-        past = trk.E[s] > trk.B[s];
+  constexpr int U = 4;
+  if (track_mode(trk) != TRACK_PRUNE || !trk.state[TRACK_PAST]) return;
+  const int64_t threads = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v0 < g.N; v0 += U * threads) {
+    int sgs[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) sgs[k] = v0 + k * threads < g.N ? bl.seg[v0 + k * threads] : SEG_FROZEN;
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      if (!(sgs[k] & SEG_SETTLED) || sgs[k] == SEG_FROZEN) continue;
+      const int sgv = sgs[k] & ~(int)SEG_SETTLED;
+      if (sgv / NTIERS != q) continue;
+      const int32_t v = (int32_t)(v0 + k * threads);
+      double x = 0;
+      if (g.is0) {
+        const int32_t s = node_slice0(g, v);
+        const long long over = trk.E[s] - trk.B[s];
+        if (over > 0) x = (double)trk.lam[s] * (double)g.k0[v] * (double)over;
+      } else {
+        int64_t b, e;
+        slice_range(g, v, b, e);
+        for (int64_t j = b; j < e; ++j) {
+          int32_t s;
+          long long kk;
+          slice_entry(g, v, j, s, kk);
+          const long long over = trk.E[s] - trk.B[s];
+          if (over > 0) x += (double)trk.lam[s] * (double)kk * (double)over;
+        }
       }
-      if (past) bucket_append(bl, sgv, (int32_t)v);
+      if (x <= 0) continue;
+      const long long m = trk.slack[v];
+      if (m >= 0 && m < track_cost(x * (double)null_scale(g, node_omega(g, v)) * trk.scale, 0.0))
+        bucket_append(bl, sgv, v);
     }
   }
 }

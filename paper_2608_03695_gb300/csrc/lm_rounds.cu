@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
       int s = prev_moved && !prev_moved[node_inst(a.g, v)]
                   ? (int)SEG_FROZEN
                   : bucket_seg(a.g, a.tier, a.seed, 0, a.it, a.lvl, (uint64_t)r, a.K, a.active, v);
-      if (prune && s < nseg && track_settled(trk, a.g, v)) {
+      if (prune && s < nseg && track_settled(trk, a.g, v, trk.slack[v], a.g.is0 ? a.g.k0[v] : 0)) {
         s |= SEG_SETTLED;
         ++settled;
       }

@@ -99,16 +99,34 @@ __global__ void __launch_bounds__(BUCKET_THREADS)
   for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
     for (int i = threadIdx.x; i < nseg; i += BUCKET_THREADS) cnt[i] = 0;
     __syncthreads();
-    for (int k = 0; k < BUCKET_ITEMS; ++k) {
-      const int64_t v = ch * BUCKET_CHUNK + (int64_t)k * BUCKET_THREADS + threadIdx.x;
-      if (v >= g.N) break;
-      int sg = bucket_seg(g, tier, seed, tag, it, lvl, r, K, active, v);
-      if (prune && sg < nseg && track_settled(trk, g, (int32_t)v)) {
-        sg |= SEG_SETTLED;
-        ++settled;
+    constexpr int U = 4;  // nodes whose margins are loaded together
+    for (int k0 = 0; k0 < BUCKET_ITEMS; k0 += U) {
+      const int64_t v0 = ch * BUCKET_CHUNK + (int64_t)k0 * BUCKET_THREADS + threadIdx.x;
+      if (v0 >= g.N) break;
+      long long ms[U] = {};
+      int64_t ks[U] = {};
+      if (prune) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t v = v0 + (int64_t)u * BUCKET_THREADS;
+          if (v < g.N) {
+            ms[u] = trk.slack[v];
+            if (g.is0) ks[u] = g.k0[v];
+          }
+        }
       }
-      seg[v] = (uint16_t)sg;
-      if (sg < nseg) atomicAdd(&cnt[sg], 1);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t v = v0 + (int64_t)u * BUCKET_THREADS;
+        if (v >= g.N) break;
+        int sg = bucket_seg(g, tier, seed, tag, it, lvl, r, K, active, v);
+        if (prune && sg < nseg && track_settled(trk, g, (int32_t)v, ms[u], ks[u])) {
+          sg |= SEG_SETTLED;
+          ++settled;
+        }
+        seg[v] = (uint16_t)sg;
+        if (sg < nseg) atomicAdd(&cnt[sg], 1);
+      }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < nseg; i += BUCKET_THREADS) counts[(int64_t)i * nchunks + ch] = cnt[i];

@@ -54,10 +54,14 @@ __global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B) {
   const int lane = threadIdx.x & 31, gl = lane % G;
   const int64_t groups = (int64_t)gridDim.x * blockDim.x / G;
   ull I = 0, J = 0;
-  int32_t cur = 0;  // instance the lane's sums belong to
+  int32_t cur = 0;  // instance the warp's sums belong to
   auto flush = [&] {
-    if (I) atomicAdd(&IJ[2 * cur], I);
-    if (J) atomicAdd(&IJ[2 * cur + 1], J);
+    I = warp_sum(I);
+    J = warp_sum(J);
+    if (lane == 0) {
+      if (I) atomicAdd(&IJ[2 * cur], I);
+      if (J) atomicAdd(&IJ[2 * cur + 1], J);
+    }
     I = J = 0;
   };
   for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G; v0 < g.N; v0 += groups) {
@@ -65,10 +69,12 @@ __global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B) {
     const bool ok = v < g.N;
     const int64_t b = ok ? g.rowptr[v] : 0, e = ok ? g.rowptr[v + 1] : 0;
     const int32_t c = ok ? labels[v] : 0;
-    const int32_t inst = ok && B > 1 ? node_inst(g, (int32_t)v) : cur;
-    if (inst != cur) {
+    const int32_t inst = B > 1 ? node_inst(g, (int32_t)(ok ? v : v0)) : 0;
+    const int32_t first = __shfl_sync(0xffffffffu, inst, 0);
+    const bool alike = __all_sync(0xffffffffu, inst == first);
+    if (first != cur || !alike) {
       flush();
-      cur = inst;
+      cur = first;
     }
     if (e - b <= LONG) ij_row(g, labels, c, b, e, gl, G, I, J);
     unsigned wide = __ballot_sync(0xffffffffu, gl == 0 && e - b > LONG);
@@ -85,14 +91,13 @@ __global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B) {
         J += Jw;
       }
     }
+    if (!alike) {  // rows of several instances: each lane's sums go out alone
+      if (I) atomicAdd(&IJ[2 * inst], I);
+      if (J) atomicAdd(&IJ[2 * inst + 1], J);
+      I = J = 0;
+    }
   }
-  if (B == 1) {
-    I = warp_sum(I);
-    J = warp_sum(J);
-    if (lane == 0) flush();
-  } else {
-    flush();
-  }
+  flush();
 }
 
 // S_s += Sigma_{c,s}^2 over the table; per-block partial sums in shared

@@ -20,10 +20,10 @@
 // is capped below one weight unit, so that any neighbour's move ends it.
 //
 // E_s is charged ahead: a margin is kept net of a budget B_s of movement for
-// the whole round, so the lists are made once, at the round's start.  Movement
-// past a budget (the flag) makes the settled nodes of that slice rejoin the
-// lists of the classes still to come (track_rescan); a margin that a push
-// takes below 0 makes its node rejoin at once.
+// the whole round, so the lists are made once, at the round's start.  After
+// movement past a budget (the flag), settled nodes whose margin does not cover
+// the excess rejoin the lists before their class decides (track_rescan); a margin
+// that a push takes below 0 makes its node rejoin at once.
 //
 // Modes of a round (device word, so that device-driven rounds need no host):
 //   OFF     most nodes move: nothing is recorded, every node decides
@@ -146,20 +146,27 @@ __device__ __forceinline__ void track_budgets(const TrackView& t, int32_t mode, 
 
 // Round start: charges the node's margin with the last round's movement and the
 // change of the budgets, and says whether the node is settled for the round.
-__device__ __forceinline__ bool track_settled(const TrackView& t, const LevelDev& g, int32_t v) {
-  long long m = t.slack[v];
+// (m: its margin; k0: its strength at level 0, both loaded ahead)
+__device__ __forceinline__ bool track_settled(const TrackView& t, const LevelDev& g, int32_t v, long long m,
+                                              int64_t k0) {
   if (m < 0) return false;
-  int64_t b, e;
-  slice_range(g, v, b, e);  // (at most TRACK_MAX_SLICES: longer lists are recorded dead)
   double x = 0;
-  for (int64_t j = b; j < e; ++j) {
-    int32_t s;
-    long long k;
-    slice_entry(g, v, j, s, k);
-    // (a budget that shrinks is not credited: the cap of a node alone in its
-    // community has to hold)
+  // (a budget that shrinks is not credited: the cap of a node alone in its
+  // community has to hold)
+  if (g.is0) {
+    const int32_t s = node_slice0(g, v);
     const long long grown = t.Ep[s] + track_budget(t, s) - t.Bp[s];
-    if (grown > 0) x += (double)t.lam[s] * (double)k * (double)grown;
+    if (grown > 0) x = (double)t.lam[s] * (double)k0 * (double)grown;
+  } else {
+    int64_t b, e;
+    slice_range(g, v, b, e);  // (at most TRACK_MAX_SLICES: longer lists are recorded dead)
+    for (int64_t j = b; j < e; ++j) {
+      int32_t s;
+      long long k;
+      slice_entry(g, v, j, s, k);
+      const long long grown = t.Ep[s] + track_budget(t, s) - t.Bp[s];
+      if (grown > 0) x += (double)t.lam[s] * (double)k * (double)grown;
+    }
   }
   if (x > 0) {
     m -= track_cost(x * (double)null_scale(g, node_omega(g, v)) * t.scale, 0.0);
