@@ -29,7 +29,7 @@ __global__ void k_present(const int32_t* sizeR, int32_t N, int32_t* flag) {
 constexpr int CW_BITS = 9;        // warp tier: rows with at most 256 entries / snapshot entries
 constexpr int CW_WARPS = 8;
 constexpr int CB_BITS = 13;       // block tier: at most 4096
-constexpr int CB_THREADS = 256;
+constexpr int CB_THREADS = 512;
 constexpr int CW_MAX = 1 << (CW_BITS - 1), CB_MAX = 1 << (CB_BITS - 1);
 
 // Per node: its new id; per new node: members, stored entries and snapshot

@@ -344,10 +344,13 @@ __device__ __forceinline__ int seg_total(const TierSegs& sg, int t0, int t1) {
 // resets each applied decision.  Moves to an empty community only leave here
 // (their label is assigned by lm_empty).  Tracked rounds also lower the margins
 // of the movers' neighbours.
+// TRACK = false leaves the tracking out (its registers cost an untracked round's
+// pass a third of its time).
+template <bool TRACK>
 __device__ __forceinline__ void lm_apply(const LevelDev& g, const TierSegs& sg, int32_t* labels, int32_t* size,
                                          const SigStore& sig, int32_t* target, ull* moved, int32_t* empties,
                                          int32_t* inst_moved, const TrackView& trk, const BucketLists& bl, int q) {
-  const bool track = track_mode(trk) != TRACK_OFF;
+  const bool track = TRACK && track_mode(trk) != TRACK_OFF;
   const int lane = threadIdx.x & 31;
   const int warps = gridDim.x * (blockDim.x >> 5), warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   int local = 0, local_empty = 0;
@@ -626,7 +629,7 @@ struct TrackState {
   int32_t mode, pause, next_pause, moved, pause_moved;
 };
 
-__device__ __forceinline__ TrackState track_next(const int32_t* prev, bool first, int32_t mode_init, long long moved,
+__host__ __device__ __forceinline__ TrackState track_next(const int32_t* prev, bool first, int32_t mode_init, long long moved,
                                                  long long listed) {
   TrackState s{mode_init, 0, TRACK_FIRST_PAUSE, 0, 0};
   if (first) return s;
@@ -640,7 +643,7 @@ __device__ __forceinline__ TrackState track_next(const int32_t* prev, bool first
   s.moved = (int32_t)moved;
   if (before == TRACK_PRUNE && listed > 3 * settled) {
     s.pause = s.next_pause;
-    s.next_pause = min(2 * s.next_pause, 1 << 20);
+    s.next_pause = s.next_pause < (1 << 19) ? 2 * s.next_pause : 1 << 20;
     s.pause_moved = (int32_t)moved;
   }
   if (s.pause > 0) {
@@ -714,6 +717,7 @@ struct ResidentIn {
 };
 struct ResidentOut {
   int64_t rounds = 0, moves = 0, last_moved = 0, last_listed = 0, communities = 0;
+  int32_t state[TRACK_WORDS] = {};  // of the last round
   ull used = 0;
   unsigned status = 0;
 };

@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
                                             &ncand[w * 4 + gi], gl, 0xffu << (gi * 8));
           });
       resident_bar();
-      lm_apply(a.g, sg, a.labels, a.size, a.sig, a.target, &a.ctl->moved[p], &a.ctl->empties[p][q],
+      lm_apply<true>(a.g, sg, a.labels, a.size, a.sig, a.target, &a.ctl->moved[p], &a.ctl->empties[p][q],
                a.inst_moved ? a.inst_moved + p * a.B : nullptr, trk, bl, q);
       resident_bar();
       const bool past = mode == TRACK_PRUNE && trk.state[TRACK_PAST];
@@ -272,6 +272,8 @@ void resident_rounds(Solver& S, const Level& L, int32_t* labels, int it, int lvl
   check_cuda(cudaMemcpyAsync(h, &a.ctl->rounds, 5 * sizeof(long long), cudaMemcpyDeviceToHost, c.stream), "copy");
   check_cuda(cudaMemcpyAsync(h + 40, S.sig_used, sizeof(ull), cudaMemcpyDeviceToHost, c.stream), "copy");
   check_cuda(cudaMemcpyAsync(h + 48, c.d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream), "copy");
+  if (trk.state)
+    check_cuda(cudaMemcpyAsync(h + 64, trk.state, 2 * sizeof(out.state), cudaMemcpyDeviceToHost, c.stream), "copy");
   sync(c);
   struct {
     long long rounds, moves, last_moved, last_listed, communities;
@@ -284,6 +286,8 @@ void resident_rounds(Solver& S, const Level& L, int32_t* labels, int it, int lvl
   out.last_moved = rb.last_moved;
   out.last_listed = rb.last_listed;
   out.communities = rb.communities;
+  if (trk.state && rb.rounds > 0)
+    std::memcpy(out.state, h + 64 + ((in.r + rb.rounds - 1) & 1) * sizeof(out.state), sizeof(out.state));
   out.used = rb.used;
   out.status = rb.status;
 }

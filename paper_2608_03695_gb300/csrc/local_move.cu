@@ -281,9 +281,10 @@ __global__ void k_round_freeze(int32_t* lm_active, int32_t* inst_moved, int32_t 
   }
 }
 
+template <bool TRACK>
 __global__ void k_lm_apply(LevelDev g, TierSegs sg, int32_t* labels, int32_t* size, SigStore sig, int32_t* target,
                            int32_t* counters, int32_t* inst_moved, TrackView trk, BucketLists bl, int q) {
-  lm_apply(g, sg, labels, size, sig, target, (ull*)counters, &counters[2], inst_moved, trk, bl, q);
+  lm_apply<TRACK>(g, sg, labels, size, sig, target, (ull*)counters, &counters[2], inst_moved, trk, bl, q);
 }
 
 // The rest of a host-driven sub-round (one cooperative launch; it returns at
@@ -735,6 +736,7 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
   const long long few = RESIDENT_MAX_WORK / (L.nnz / N + RESIDENT_NODE_WORK);
   long long moved = 0, listed = N;  // of the last round
   bool first_round = true, rebuild = false;
+  int32_t state[TRACK_WORDS] = {};  // tracking words of the last round
   int r = 0;
   while (r < max_rounds) {
     if (rebuild) rebuild_sigma(S, L, labels, false);
@@ -760,6 +762,7 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
       moved = ro.last_moved;
       listed = ro.last_listed;
       out.communities = ro.communities;
+      std::memcpy(state, ro.state, sizeof(state));
       rebuild = !S.sig.d && ro.used > 0;
       if (moved == 0) break;
       if (r >= max_rounds) out.capped = true;
@@ -778,6 +781,8 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
     // empty communities; its moves, the table fill, the status word, the list
     // lengths and the tracking mode go to the pinned buffer.
     const TrackView tr = track_at(trk, S.Tn, r);
+    // (the mode k_round_begin comes to, from the same words)
+    const bool tracked = tr.state && track_next(state, first_round, mode_init, moved, listed).mode != TRACK_OFF;
     const BucketLists bl{S.lists, (int64_t)S.N0, S.cursors, tier_offsets(S), S.bseg};
     if (tr.state)
       launch(c, k_round_begin, dim3(1), dim3(512), 0, tr, track_at(trk, S.Tn, r + 1).state, S.Tn, (int)first_round,
@@ -798,7 +803,7 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
       } else {
         decide(sg, tr);
       }
-      launch(c, k_lm_apply, dim3(fixed_grid(4)), dim3(APPLY_THREADS), 0, L.d, sg, labels, S.size, S.sig, S.target,
+      launch(c, tracked ? k_lm_apply<true> : k_lm_apply<false>, dim3(fixed_grid(4)), dim3(APPLY_THREADS), 0, L.d, sg, labels, S.size, S.sig, S.target,
              S.counters, batch ? S.inst_moved : nullptr, tr, bl, q);
       launch_coop(c, k_empty_pass, dim3(S.empty_grid), dim3(EMPTY_THREADS), 0, L.d, S.B, S.target, labels, S.size,
                   S.sig, S.counters, S.empty_blk, S.freelist, S.tmp32b, S.inst_cnt, tr, bl, q + 1);
@@ -810,16 +815,16 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
       int64_t moved;
       ull used;
       unsigned status;
-      int32_t mode;
-    } rb{0, 0, 0, TRACK_OFF};
+      int32_t pad_;
+      int32_t state[TRACK_WORDS];
+    } rb{};
     std::memcpy(h, &rb, sizeof(rb));
     check_cuda(cudaMemcpyAsync(h, S.counters, sizeof(int64_t), cudaMemcpyDeviceToHost, c.stream), "copy");
     check_cuda(cudaMemcpyAsync(h + 8, S.sig_used, sizeof(ull), cudaMemcpyDeviceToHost, c.stream), "copy");
     check_cuda(cudaMemcpyAsync(h + 16, c.d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream), "copy");
     if (tr.state) {
-      check_cuda(cudaMemcpyAsync(h + 20, tr.state + TRACK_MODE, sizeof(int32_t), cudaMemcpyDeviceToHost, c.stream),
-                 "copy");
-      check_cuda(cudaMemcpyAsync(h + 24, S.cursors, nseg * sizeof(int32_t), cudaMemcpyDeviceToHost, c.stream), "copy");
+      check_cuda(cudaMemcpyAsync(h + 24, tr.state, sizeof(rb.state), cudaMemcpyDeviceToHost, c.stream), "copy");
+      check_cuda(cudaMemcpyAsync(h + sizeof(rb), S.cursors, nseg * sizeof(int32_t), cudaMemcpyDeviceToHost, c.stream), "copy");
     }
     sync(c);
     std::memcpy(&rb, h, sizeof(rb));
@@ -828,11 +833,12 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
     moved = rb.moved;
     listed = N;
     if (tr.state) {
-      const int32_t* cur = reinterpret_cast<const int32_t*>(h + 24);
+      std::memcpy(state, rb.state, sizeof(state));
+      const int32_t* cur = reinterpret_cast<const int32_t*>(h + sizeof(rb));
       listed = 0;
       for (int i = 0; i < nseg; ++i) listed += cur[i];
     }
-    if (prof && rb.mode == TRACK_PRUNE) {
+    if (prof && tr.state && rb.state[TRACK_MODE] == TRACK_PRUNE) {
       // the decision timing covers the rounds in which every node decides
       for (size_t k = spans; k < c.prof_spans->size(); ++k) {
         cudaEventDestroy((*c.prof_spans)[k].first);
