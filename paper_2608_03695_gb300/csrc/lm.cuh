@@ -705,12 +705,18 @@ inline TrackView track_at(const TrackView& trk, int32_t Tn, int r) {
 constexpr int64_t RESIDENT_MAX_WORK = (int64_t)1 << 22, RESIDENT_NODE_WORK = 16;
 constexpr int64_t RESIDENT_REFINE_WORK = (int64_t)1 << 21;
 
+// Bytes behind the list lengths for a resident launch's control words.
+constexpr size_t RESIDENT_CTL_BYTES = 1024;
+// Words of a dense table up to which a resident launch builds it itself.
+constexpr int64_t RESIDENT_BUILD_MAX = (int64_t)1 << 20;
+
 // Rounds in one launch (lm_rounds.cu): from round r, up to r_end, while nodes
 // move, no hash region needs a rebuild and no round lists more than max_listed
 // nodes.  Synchronises.
 struct ResidentIn {
   int r = 0, r_end = 0;
   bool first = false;        // r is the level's first round
+  bool build = false;        // sizes and (dense) Sigma are to be built first
   int32_t mode_init = 0;
   long long prev_moved = 0, prev_listed = 0;
   long long max_listed = 0;

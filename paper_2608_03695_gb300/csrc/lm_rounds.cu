@@ -15,6 +15,7 @@
 // lengths, move counts and tracking words of the other parity are cleared by
 // block 0 between the round's first and second barrier, when every block has
 // read what it needs of them.
+#include <cstddef>
 #include <cstring>
 
 #include "../../include/mslice.h"
@@ -31,7 +32,11 @@ struct ResidentCtl {
   // results
   long long rounds, moves, last_moved, last_listed;
   ull communities;  // non-empty at the end
+  ull used;         // the hash's rebuild flag
+  unsigned status;
+  int32_t state[TRACK_WORDS];
 };
+static_assert(sizeof(ResidentCtl) <= RESIDENT_CTL_BYTES, "room behind the list lengths");
 
 struct ResidentArgs {
   LevelDev g;
@@ -59,6 +64,7 @@ struct ResidentArgs {
   const int64_t* goff;
   unsigned* status;
   const ull* sig_used;           // nullptr: dense tables
+  int32_t build;                 // sizes and (dense) Sigma are to be built first
   int32_t *blk, *freelist, *mrank, *icnt;
   ResidentCtl* ctl;
 };
@@ -83,6 +89,27 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
   }
   for (int i = threadIdx.x; i < RW * 4; i += RT) ncand[i] = 0;
   if (threadIdx.x == 0) block_ncand = 0;
+  if (a.build) {
+    // community sizes and Sigma of the labels: five launches less a level
+    const int64_t tid = (int64_t)blockIdx.x * RT + threadIdx.x, threads = (int64_t)gridDim.x * RT;
+    for (int64_t i = tid; i < a.g.N; i += threads) a.size[i] = 0;
+    for (int64_t i = tid; i < a.sig.rows * a.sig.T; i += threads) a.sig.d[i] = 0;
+    resident_bar();
+    if (a.g.is0) {
+      for (int64_t v = tid; v < a.g.N; v += threads) {
+        const int32_t c = a.labels[v];
+        atomicAdd(&a.size[c], 1);
+        if (a.g.k0[v] > 0) ss_add(a.sig, c, node_slice0(a.g, (int32_t)v), a.g.k0[v]);
+      }
+    } else {
+      for (int64_t v = tid >> 3; v < a.g.N; v += threads >> 3) {
+        const int32_t c = a.labels[v];
+        if ((lane & 7) == 0) atomicAdd(&a.size[c], 1);
+        for (int64_t j = a.g.sptr[v] + (lane & 7); j < a.g.sptr[v + 1]; j += 8) ss_add(a.sig, c, a.g.sidx[j], a.g.sval[j]);
+      }
+    }
+    // (complete at the barrier after the first round's lists)
+  }
   const int nseg = a.K * NTIERS;
   long long moved = a.prev_moved, listed = a.prev_listed, moves = 0;
   int32_t r = a.r0;
@@ -205,6 +232,10 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
       a.ctl->moves = moves;
       a.ctl->last_moved = moved;
       a.ctl->last_listed = listed;
+      a.ctl->used = a.sig_used ? *a.sig_used : 0;
+      a.ctl->status = *a.status;
+      if (a.trk.state)
+        for (int i = 0; i < TRACK_WORDS; ++i) a.ctl->state[i] = a.trk.state[((r - 1) & 1) * TRACK_WORDS + i];
     }
   }
 }
@@ -260,36 +291,27 @@ void resident_rounds(Solver& S, const Level& L, int32_t* labels, int it, int lvl
   a.freelist = S.freelist;
   a.mrank = S.tmp32b;
   a.icnt = S.inst_cnt;
-  a.ctl = reinterpret_cast<ResidentCtl*>(c.ws->get_bytes("s_resident", sizeof(ResidentCtl)));
-  check_cuda(cudaMemsetAsync(a.ctl, 0, sizeof(ResidentCtl), c.stream), "memset");
-  check_cuda(cudaMemsetAsync(S.cursors, 0, 2 * (size_t)S.p.K * NTIERS * sizeof(int32_t), c.stream), "memset");
+  // (the control words lie behind the two sets of list lengths: one clear)
+  const size_t lengths = (2 * (size_t)S.p.K * NTIERS * sizeof(int32_t) + 15) & ~(size_t)15;
+  a.ctl = reinterpret_cast<ResidentCtl*>(reinterpret_cast<char*>(S.cursors) + lengths);
+  a.build = in.build ? 1 : 0;
+  check_cuda(cudaMemsetAsync(S.cursors, 0, lengths + sizeof(ResidentCtl), c.stream), "memset");
   const unsigned grid = resident_grid(L.d.N, (int64_t)S.tier_cnt[3] + S.tier_cnt[4], S.p.K, S.sms);
   if (S.sig.d)
     launch_rounds(c, lm_policy<true>(S, L, labels, trk), a, grid);
   else
     launch_rounds(c, lm_policy<false>(S, L, labels, trk), a, grid);
-  char* h = static_cast<char*>(c.pinned);
-  check_cuda(cudaMemcpyAsync(h, &a.ctl->rounds, 5 * sizeof(long long), cudaMemcpyDeviceToHost, c.stream), "copy");
-  check_cuda(cudaMemcpyAsync(h + 40, S.sig_used, sizeof(ull), cudaMemcpyDeviceToHost, c.stream), "copy");
-  check_cuda(cudaMemcpyAsync(h + 48, c.d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream), "copy");
-  if (trk.state)
-    check_cuda(cudaMemcpyAsync(h + 64, trk.state, 2 * sizeof(out.state), cudaMemcpyDeviceToHost, c.stream), "copy");
-  sync(c);
-  struct {
-    long long rounds, moves, last_moved, last_listed, communities;
-    ull used;
-    unsigned status;
-  } rb;
-  std::memcpy(&rb, h, sizeof(rb));
-  out.rounds = rb.rounds;
-  out.moves = rb.moves;
-  out.last_moved = rb.last_moved;
-  out.last_listed = rb.last_listed;
-  out.communities = rb.communities;
-  if (trk.state && rb.rounds > 0)
-    std::memcpy(out.state, h + 64 + ((in.r + rb.rounds - 1) & 1) * sizeof(out.state), sizeof(out.state));
-  out.used = rb.used;
-  out.status = rb.status;
+  ResidentCtl h;
+  const size_t at = offsetof(ResidentCtl, rounds);
+  std::memcpy(&h.rounds, readback(c, &a.ctl->rounds, sizeof(ResidentCtl) - at), sizeof(ResidentCtl) - at);
+  out.rounds = h.rounds;
+  out.moves = h.moves;
+  out.last_moved = h.last_moved;
+  out.last_listed = h.last_listed;
+  out.communities = (int64_t)h.communities;
+  out.used = h.used;
+  out.status = h.status;
+  std::memcpy(out.state, h.state, sizeof(out.state));
 }
 
 }  // namespace mslice

@@ -359,7 +359,7 @@ void solver_alloc(Solver& S) {
   S.bseg = c.ws->get<uint16_t>("s_bseg", N);
   S.bcounts = c.ws->get<int32_t>("s_bcounts", (size_t)S.p.K * NTIERS * ((N + BUCKET_CHUNK - 1) / BUCKET_CHUNK));
   S.lists = c.ws->get<int32_t>("s_lists", (size_t)N * S.p.K);
-  S.cursors = c.ws->get<int32_t>("s_cursors", 2 * NTIERS * S.p.K + NTIERS);
+  S.cursors = c.ws->get<int32_t>("s_cursors", 2 * NTIERS * S.p.K + NTIERS + 4 + RESIDENT_CTL_BYTES / sizeof(int32_t));
   S.counters = c.ws->get<int32_t>("s_counters", 8);
   S.sig_used = c.ws->get<ull>("s_sig_used", 1);
   S.goff = c.ws->get<int64_t>("s_goff", N + 1);
@@ -695,15 +695,24 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
     }
     return out;
   }
+  const bool tuning = S.p.autotune && lvl == 0;
+  // Rounds are resident (lm_rounds.cu) while they have at most
+  // RESIDENT_MAX_WORK to decide, by the level's average degree:
+  // every round of a level that small, and the others once a pruned round has
+  // listed few enough nodes.  Not while the level-0 decisions are being timed
+  // or the tier cuts tuned.
+  const bool may_reside = !tuning && !(c.profile && lvl == 0);
+  const long long few = RESIDENT_MAX_WORK / (L.nnz / N + RESIDENT_NODE_WORK);
   // community sizes and Sigma of the level's initial labels (refinement
-  // reads Sigma even when no round runs)
-  rebuild_sigma(S, L, labels, true);
+  // reads Sigma even when no round runs), unless the first resident launch
+  // builds them
+  bool build = max_rounds > 0 && may_reside && N <= few && S.sig.d && S.sig.rows * S.sig.T <= RESIDENT_BUILD_MAX;
+  if (!build) rebuild_sigma(S, L, labels, true);
   if (max_rounds <= 0) return out;
   // Margins are recorded once few nodes move: from the level's first round,
   // except where the level starts from singletons (its first rounds move most
   // nodes), and not on a level whose tier cuts are still being tuned.
   // (MSLICE_TRACK_MIN_ENTRIES: tracks every level of that many entries)
-  const bool tuning = S.p.autotune && lvl == 0;
   const char* track_min = std::getenv("MSLICE_TRACK_MIN_ENTRIES");
   const bool worth = track_min ? L.nnz >= std::atoll(track_min)
                                : L.nnz >= TRACK_MIN_ENTRIES && L.nnz >= TRACK_MIN_DEGREE * (int64_t)N &&
@@ -727,13 +736,6 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
     else
       decide_all(c, lm_policy<false>(S, L, labels, t), sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
   };
-  // Rounds are resident (lm_rounds.cu) while they have at most
-  // RESIDENT_MAX_WORK to decide, by the level's average degree:
-  // every round of a level that small, and the others once a pruned round has
-  // listed few enough nodes.  Not while the level-0 decisions are being timed
-  // or the tier cuts tuned.
-  const bool may_reside = !tuning && !(c.profile && lvl == 0);
-  const long long few = RESIDENT_MAX_WORK / (L.nnz / N + RESIDENT_NODE_WORK);
   long long moved = 0, listed = N;  // of the last round
   bool first_round = true, rebuild = false;
   int32_t state[TRACK_WORDS] = {};  // tracking words of the last round
@@ -745,6 +747,8 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
       in.r = r;
       in.r_end = max_rounds;
       in.first = first_round;
+      in.build = build;
+      build = false;
       in.mode_init = mode_init;
       in.prev_moved = moved;
       in.prev_listed = listed;

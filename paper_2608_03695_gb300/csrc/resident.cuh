@@ -72,8 +72,10 @@ __device__ __forceinline__ TierSegs resident_segs(int32_t* lists, int64_t row_st
 }
 
 // The nodes of one class, dealt out by tier: a block per node of tiers 4 and 3,
-// a warp per node of tier 2, 8 lanes per node of tiers 1 and 0 (the last blocks
-// take the first of the short ones).
+// a warp per node of tier 2, 8 lanes per node of tiers 1 and 0.  The last blocks
+// take the first of tier 2, and the low tiers start with the warps after those:
+// a node is a chain of dependent loads of 5-15 us, so two in one warp while
+// others idle double the sub-round.
 template <class ByBlock, class ByWarp, class ByEight>
 __device__ __forceinline__ void resident_deal(const TierSegs& sg, ByBlock&& by_block, ByWarp&& by_warp,
                                               ByEight&& by_eight) {
@@ -91,8 +93,8 @@ __device__ __forceinline__ void resident_deal(const TierSegs& sg, ByBlock&& by_b
   const int n2 = *sg.count[2];
   for (int i = gw; i < n2; i += warps) by_warp(sg.list[2][i]);
   const int n0 = *sg.count[0], n = n0 + *sg.count[1];
-  const int gi = lane >> 3;
-  for (int i = gw * 4 + gi; i < n; i += warps * 4) by_eight(i < n0 ? sg.list[0][i] : sg.list[1][i - n0], gi, lane & 7);
+  const int gi = lane >> 3, g0 = (gw + warps - n2 % warps) % warps;
+  for (int i = g0 * 4 + gi; i < n; i += warps * 4) by_eight(i < n0 ? sg.list[0][i] : sg.list[1][i - n0], gi, lane & 7);
   __syncwarp();
 }
 
