@@ -992,7 +992,7 @@ bool aggregate(Solver& S, const Level& L, const int32_t* P, Level& next, const s
                int32_t* next_labels, int32_t* node_of0, int64_t* checksum) {
   Ctx& c = *S.c;
   const int32_t N = L.d.N;
-  if (L.nnz + RESIDENT_NODE_WORK * (int64_t)N <= RESIDENT_AGGREGATE_WORK) {
+  if (L.nnz + RESIDENT_NODE_WORK * (int64_t)N <= resident_work(RESIDENT_AGGREGATE_WORK)) {
     const Resident r = aggregate_resident(S, L, P, next, slot, next_labels, node_of0);
     if (r == Resident::SAME) return false;
     if (r == Resident::DONE) {

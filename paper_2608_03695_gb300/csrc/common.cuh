@@ -261,6 +261,12 @@ __device__ __forceinline__ Slot hash_first(const HashView& h, ull key) {
   return h.slots[hash_home(key, base, size)];
 }
 
+// The same with the key's region at hand.
+__device__ __forceinline__ Slot hash_first_at(const HashView& h, ull key, uint64_t base, uint64_t size) {
+  if (h.narrow) return widen(slots8(h)[hash_home8((uint32_t)(key >> 32), base, size)]);
+  return h.slots[hash_home(key, base, size)];
+}
+
 // Region holding slot i (binary search over the offsets).
 __device__ __forceinline__ int32_t hash_region_of(const HashView& h, uint64_t i) {
   int32_t lo = 0, hi = h.nregions - 1;

@@ -78,6 +78,8 @@ __device__ __forceinline__ int32_t node_slice0(const LevelDev& g, int32_t v) {
 // A coupling entry weighs on (uniform omega) or its pair's numerator in the
 // coupling table, and is absent when that is 0.  (om: the omega of the row's
 // instance.)
+// (L0: level 0 is known at compile time.)
+template <bool L0 = false>
 __device__ __forceinline__ bool edge_at(const LevelDev& g, int64_t e, int32_t& u, long long& W, const Omega& om) {
 #if MSLICE_CHECKED
   if (e < 0 || e >= g.rowptr[g.N]) {
@@ -94,7 +96,7 @@ __device__ __forceinline__ bool edge_at(const LevelDev& g, int64_t e, int32_t& u
     return false;
   }
 #endif
-  if (g.is0) {
+  if (L0 || g.is0) {
     const int2 x = __ldcs(&g.adj0[e]);
     u = x.x;
     if (x.y <= 0) {

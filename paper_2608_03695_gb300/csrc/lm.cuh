@@ -3,6 +3,9 @@
 // a sub-round's decisions, the moves to empty communities and the round's
 // tracking state.  The rules are stated in local_move.cu.
 #pragma once
+#include <algorithm>
+#include <cstdlib>
+
 #include "decide.cuh"
 #include "solver.h"
 #include "track.cuh"
@@ -74,7 +77,11 @@ __device__ __forceinline__ u128 null_sum_part(const LevelDev& g, const u128* lam
   return acc;
 }
 
-template <bool DENSE>
+// L0: a level-0 policy for hashed tables.  Its nodes hold one (snapshot, strength)
+// entry each, so the code that walks lists is left out and the snapshot's hash
+// region is looked up once per node instead of once per candidate; the group
+// kernels, capped at 64 registers, spill 52 bytes instead of 116.
+template <bool DENSE, bool L0 = false>
 struct LMPolicy {
   static constexpr int MIN_BLOCKS = DENSE ? MSLICE_DENSE_MIN_BLOCKS : MSLICE_GROUP_MIN_BLOCKS;
   LevelDev g;
@@ -96,6 +103,7 @@ struct LMPolicy {
     long long k;
     Omega om;
     u128 A;
+    uint64_t base, size;  // L0: the snapshot's hash region
   };
 
   __device__ bool begin(int32_t) const { return true; }
@@ -103,7 +111,7 @@ struct LMPolicy {
     VCtx c;
     c.a = labels[v];
     c.size_a = size[c.a];
-    c.single = g.is0 != 0;
+    c.single = L0 || g.is0 != 0;
     c.s = 0;
     c.k = 0;
     c.A = 0;
@@ -111,6 +119,7 @@ struct LMPolicy {
     if (c.single) {
       c.k = g.k0[v];
       c.s = node_slice0(g, v);
+      if constexpr (L0) hash_region(sig.h, pack_cs(0, c.s), c.base, c.size);
       if (c.k > 0) c.A = (u128)(ull)null_scale(g, c.om) * lam[c.s] * (u128)(ull)c.k;
     }
     return c;
@@ -118,7 +127,7 @@ struct LMPolicy {
   __device__ void skip(int32_t v) const { target[v] = NO_MOVE; }
   __device__ bool edge(int32_t, const VCtx& vc, int64_t e, int32_t& key, long long& w) const {
     int32_t u;
-    if (!edge_at(g, e, u, w, vc.om)) return false;
+    if (!edge_at<L0>(g, e, u, w, vc.om)) return false;
     key = labels[u];
     return true;
   }
@@ -128,25 +137,30 @@ struct LMPolicy {
     return (((i128)W) << P_BITS) - (i128)((u128)(ull)null_scale(g, vc.om) * ns);
   }
   __device__ Probe probe(int32_t, const VCtx& vc, int32_t c) const {
-    if (vc.single && vc.k > 0) return sst_first<DENSE>(sig, c, vc.s);
+    if (vc.single && vc.k > 0) {
+      if constexpr (L0)
+        return hash_first_at(sig.h, pack_cs(c, vc.s), vc.base, vc.size);
+      else
+        return sst_first<DENSE>(sig, c, vc.s);
+    }
     return Slot{EMPTY_KEY, 0};
   }
   __device__ Cand cand(int32_t v, const VCtx& vc, int32_t c, long long W, const Probe& pr) const {
-    if (vc.single) {
+    if (L0 || vc.single) {
       const long long x = vc.k > 0 ? sst_resolve<DENSE>(sig, c, vc.s, pr) : 0;
       return Cand{(((i128)W) << P_BITS) - (i128)(vc.A * (u128)(ull)x), c};
     }
     return Cand{key_of(v, vc, c, W, false), c};
   }
   __device__ i128 own(int32_t v, const VCtx& vc, long long Wown) const {
-    if (vc.single) {
+    if (L0 || vc.single) {
       const long long x = vc.k > 0 ? sst_get<DENSE>(sig, vc.a, vc.s) - vc.k : 0;
       return (((i128)Wown) << P_BITS) - (i128)(vc.A * (u128)(ull)x);
     }
     return key_of(v, vc, vc.a, Wown, true);
   }
   // slice-parallel scoring (block tiers, aggregated levels)
-  __device__ int64_t slice_count(int32_t v) const { return g.is0 ? 0 : g.sptr[v + 1] - g.sptr[v]; }
+  __device__ int64_t slice_count(int32_t v) const { return L0 || g.is0 ? 0 : g.sptr[v + 1] - g.sptr[v]; }
   __device__ bool own_walks_slices() const { return true; }
   __device__ u128 null_part(int32_t v, const VCtx&, int32_t c, bool self, int t, int nt) const {
     return null_sum_part<DENSE>(g, lam, sig, v, c, self, t, nt);
@@ -169,7 +183,7 @@ struct LMPolicy {
     }
     target[v] = t;
     if (t == NO_MOVE && track_mode(trk) != TRACK_OFF)
-      track_record(trk, g, vc.om, v, vc.size_a == 1, has, Ga, best.G);
+      track_record<L0>(trk, g, vc.om, v, vc.size_a == 1, has, Ga, best.G);
   }
 };
 
@@ -613,16 +627,18 @@ __device__ __forceinline__ void lm_empty(const LevelDev& g, int32_t B, int32_t* 
 // The tracking state of a round from that of the round before (prev) and what
 // that round did.
 //   - Tracking starts when the movement, going on as in the last two rounds,
-//     is expected to stay under a twelfth of the nodes, and stops past a
+//     is expected to stay under a sixteenth of the nodes, and stops past a
 //     quarter: the movers' pushes and the drift of the null sums would leave
 //     few nodes settled for what they cost.
 //   - Pruning that leaves three nodes in four in the lists is given up until
 //     the movement has fallen to a quarter, or for a number of rounds that
 //     doubles each time (communities can swap nodes for dozens of rounds).
 //   - Levels with fewer entries, or with short rows (the decisions cost little
-//     more than the tracking) or long strength lists, are not tracked.
+//     more than the tracking), are not tracked, unless strength lists of two or
+//     more entries a node make their decisions dear (TRACK_MIN_LOOKUPS).
 constexpr int64_t TRACK_MIN_ENTRIES = 1 << 20, TRACK_MIN_DEGREE = 8;
-constexpr double TRACK_START = 1.0 / 12, TRACK_STOP = 1.0 / 4;
+constexpr int64_t TRACK_MIN_LOOKUPS = 1 << 21;
+constexpr double TRACK_START = 1.0 / 16, TRACK_STOP = 1.0 / 4;
 constexpr int TRACK_FIRST_PAUSE = 8;
 
 struct TrackState {
@@ -667,9 +683,9 @@ __device__ __forceinline__ void track_store(int32_t* state, const TrackState& s)
   state[TRACK_PAUSE_MOVED] = s.pause_moved;
 }
 
-template <bool DENSE>
-inline LMPolicy<DENSE> lm_policy(const Solver& S, const Level& L, const int32_t* labels, const TrackView& trk) {
-  LMPolicy<DENSE> pol;
+template <bool DENSE, bool L0 = false>
+inline LMPolicy<DENSE, L0> lm_policy(const Solver& S, const Level& L, const int32_t* labels, const TrackView& trk) {
+  LMPolicy<DENSE, L0> pol;
   pol.g = L.d;
   pol.labels = labels;
   pol.size = S.size;
@@ -704,6 +720,12 @@ inline TrackView track_at(const TrackView& trk, int32_t Tn, int r) {
 // which rounds are resident, and the same for a level's refinement.
 constexpr int64_t RESIDENT_MAX_WORK = (int64_t)1 << 22, RESIDENT_NODE_WORK = 16;
 constexpr int64_t RESIDENT_REFINE_WORK = (int64_t)1 << 21;
+
+// The bound in force: MSLICE_RESIDENT_MAX_WORK lowers it (0: nothing is resident).
+inline int64_t resident_work(int64_t bound) {
+  const char* e = std::getenv("MSLICE_RESIDENT_MAX_WORK");
+  return e ? std::min<int64_t>(bound, std::atoll(e)) : bound;
+}
 
 // Bytes behind the list lengths for a resident launch's control words.
 constexpr size_t RESIDENT_CTL_BYTES = 1024;

@@ -702,7 +702,7 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
   // listed few enough nodes.  Not while the level-0 decisions are being timed
   // or the tier cuts tuned.
   const bool may_reside = !tuning && !(c.profile && lvl == 0);
-  const long long few = RESIDENT_MAX_WORK / (L.nnz / N + RESIDENT_NODE_WORK);
+  const long long few = resident_work(RESIDENT_MAX_WORK) / (L.nnz / N + RESIDENT_NODE_WORK);
   // community sizes and Sigma of the level's initial labels (refinement
   // reads Sigma even when no round runs), unless the first resident launch
   // builds them
@@ -715,8 +715,9 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
   // (MSLICE_TRACK_MIN_ENTRIES: tracks every level of that many entries)
   const char* track_min = std::getenv("MSLICE_TRACK_MIN_ENTRIES");
   const bool worth = track_min ? L.nnz >= std::atoll(track_min)
-                               : L.nnz >= TRACK_MIN_ENTRIES && L.nnz >= TRACK_MIN_DEGREE * (int64_t)N &&
-                                     L.ns <= 4 * (int64_t)N;
+                               : (L.nnz >= TRACK_MIN_ENTRIES && L.nnz >= TRACK_MIN_DEGREE * (int64_t)N &&
+                                  L.ns <= 4 * (int64_t)N) ||
+                                     (L.ns >= 2 * (int64_t)N && L.nnz + L.nnz / N * L.ns >= TRACK_MIN_LOOKUPS);
   const TrackView trk = !worth || tuning ? TrackView{} : track_view(S, L);
   const int32_t mode_init = lvl == 0 && it == 0 && !S.warm ? TRACK_OFF : TRACK_RECORD;
   if (trk.state)
@@ -733,6 +734,8 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
   auto decide = [&](const TierSegs& sg, const TrackView& t) {
     if (S.sig.d)
       decide_all(c, lm_policy<true>(S, L, labels, t), sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
+    else if (L.d.is0)
+      decide_all(c, lm_policy<false, true>(S, L, labels, t), sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
     else
       decide_all(c, lm_policy<false>(S, L, labels, t), sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
   };

@@ -1106,7 +1106,7 @@ static void refine_impl(Solver& S, const Level& L, const int32_t* P, int it, int
   if (N == 0) return;
   clear_store(S, S.kr);
   long long* PR = c.ws->get<long long>("ref_PR", N);
-  const bool resident = L.nnz + RESIDENT_NODE_WORK * (int64_t)N <= RESIDENT_REFINE_WORK;
+  const bool resident = L.nnz + RESIDENT_NODE_WORK * (int64_t)N <= resident_work(RESIDENT_REFINE_WORK);
   if (!resident) {
     if (L.d.is0)
       launch(c, k_ref_init<8>, dim3(fixed_grid(8)), dim3(256), 0, L.d, P, S.sig, (const u128*)S.lam, S.R, S.sizeR,

@@ -88,8 +88,16 @@ __device__ __forceinline__ long long track_cost(double xp, double xn) {
 
 // Margin cost of what is left of the budgets (B_s - E_s; a credit past them)
 // for node v; false when the node's list is too long to be tracked.
+template <bool L0>
 __device__ __forceinline__ bool track_budget_cost(const TrackView& t, const LevelDev& g, const Omega& om, int32_t v,
                                                   long long& cost) {
+  if constexpr (L0) {
+    const int32_t s = node_slice0(g, v);
+    const double x = (double)t.lam[s] * (double)g.k0[v] * (double)(t.B[s] - t.E[s]) *
+                     ((double)null_scale(g, om) * t.scale);
+    cost = track_cost(x > 0 ? x : 0, x < 0 ? -x : 0);
+    return true;
+  }
   int64_t b, e;
   slice_range(g, v, b, e);
   if (e - b > TRACK_MAX_SLICES) return false;
@@ -109,6 +117,7 @@ __device__ __forceinline__ bool track_budget_cost(const TrackView& t, const Leve
 
 // Margin of a node that decided to stay: Ga its key of staying, Gb its best
 // other candidate's key when has.
+template <bool L0>
 __device__ __forceinline__ void track_record(const TrackView& t, const LevelDev& g, const Omega& om, int32_t v,
                                              bool alone, bool has, const i128& Ga, const i128& Gb) {
   // (alone without a candidate: a node without edges)
@@ -118,7 +127,7 @@ __device__ __forceinline__ void track_record(const TrackView& t, const LevelDev&
     const i128 u = M >> (P_BITS - t.F);
     m = u > (i128)TRACK_CAP ? TRACK_CAP : (long long)u;
     long long cost;
-    if (track_budget_cost(t, g, om, v, cost)) {
+    if (track_budget_cost<L0>(t, g, om, v, cost)) {
       const long long cap = !alone ? TRACK_CAP : t.F > 0 ? (1ll << t.F) - 1 : 0;
       m -= cost;
       m = m < cap ? m : cap;

@@ -3,7 +3,8 @@
 The library tracks settled nodes on large levels; here every level of small
 graphs is tracked (MSLICE_TRACK_MIN_ENTRIES=0), so that pushes, budgets and
 rejoining nodes occur next to tie-breaks, singletons and moves to empty
-communities.  Every result must be the oracle's: labels bit-exact, counters
+communities.  Small levels run inside one launch per phase; with
+MSLICE_RESIDENT_MAX_WORK=0 the same graphs take the large levels' kernels.  Every result must be the oracle's: labels bit-exact, counters
 equal, Q within 1e-12 relative.
 """
 import numpy as np
@@ -49,10 +50,13 @@ def same(g, o):
         assert g[2][k] == o[2][k], k
 
 
+@pytest.mark.parametrize("resident", [None, "0"])
 @pytest.mark.parametrize("dense", [None, "0"])
 @pytest.mark.parametrize("null", ["multislice", "global", "cpm"])
 @pytest.mark.parametrize("kind", ["planted", "powerlaw", "contact", "random"])
-def test_tracked_solves(kind, null, dense, monkeypatch):
+def test_tracked_solves(kind, null, dense, resident, monkeypatch):
+    if resident is not None:
+        monkeypatch.setenv("MSLICE_RESIDENT_MAX_WORK", resident)
     if dense is not None:
         monkeypatch.setenv("MSLICE_DENSE_LIMIT", dense)
     for seed in range(4):
@@ -69,9 +73,12 @@ def test_tracked_solves(kind, null, dense, monkeypatch):
         same(g, oracle.leiden(snaps, gamma, omega, null=null, coupling=coupling, **kw))
 
 
+@pytest.mark.parametrize("resident", [None, "0"])
 @pytest.mark.parametrize("shift", [8, 16, 24])
-def test_tracked_heavy_weights(shift):
+def test_tracked_heavy_weights(shift, resident, monkeypatch):
     """Margins in units coarser than a weight unit, and pushes past the largest."""
+    if resident is not None:
+        monkeypatch.setenv("MSLICE_RESIDENT_MAX_WORK", resident)
     snaps = graph(2, "powerlaw")
     for s in snaps:
         s.weights = (s.weights.astype(np.int64) << shift).astype(np.int32)
@@ -80,8 +87,25 @@ def test_tracked_heavy_weights(shift):
     same(g, oracle.leiden(snaps, (1, 1), (1 << shift, 3)))
 
 
-def test_tracked_batch():
+@pytest.mark.parametrize("theta", [None, (1, 100)])
+def test_untracked_large_level_kernels(theta, monkeypatch):
+    """The large levels' kernels without tracking, greedy and randomised."""
+    monkeypatch.delenv("MSLICE_TRACK_MIN_ENTRIES")
+    monkeypatch.setenv("MSLICE_RESIDENT_MAX_WORK", "0")
+    for kind in ("planted", "powerlaw", "contact", "random"):
+        for dense in ("4194304", "0"):
+            monkeypatch.setenv("MSLICE_DENSE_LIMIT", dense)
+            snaps = graph(1, kind)
+            with pkg.mslice_build(snaps) as h:
+                g = h.mslice_leiden(theta=theta)
+            same(g, oracle.leiden(snaps, theta=theta))
+
+
+@pytest.mark.parametrize("resident", [None, "0"])
+def test_tracked_batch(resident, monkeypatch):
     """Instances of very different movement in one batch, alone and together."""
+    if resident is not None:
+        monkeypatch.setenv("MSLICE_RESIDENT_MAX_WORK", resident)
     cases = [(graph(s, k), gm, om) for s, k in ((0, "planted"), (3, "planted"), (1, "powerlaw"), (2, "contact"))
              for gm, om in (((1, 1), (1, 1)), ((3, 2), (10, 1)))]
     handles = [pkg.mslice_build(c[0]) for c in cases]
