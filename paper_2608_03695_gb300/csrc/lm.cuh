@@ -77,9 +77,9 @@ __device__ __forceinline__ u128 null_sum_part(const LevelDev& g, const u128* lam
   return acc;
 }
 
-// L0: a level-0 policy for hashed tables.  Its nodes hold one (snapshot, strength)
-// entry each, so the code that walks lists is left out and the snapshot's hash
-// region is looked up once per node instead of once per candidate; the group
+// L0: a level-0 policy.  Its nodes hold one (snapshot, strength)
+// entry each, so the code that walks lists is left out and (hashed tables) the
+// snapshot's region is looked up once per node instead of once per candidate; the group
 // kernels, capped at 64 registers, spill 52 bytes instead of 116.
 template <bool DENSE, bool L0 = false>
 struct LMPolicy {
@@ -119,7 +119,7 @@ struct LMPolicy {
     if (c.single) {
       c.k = g.k0[v];
       c.s = node_slice0(g, v);
-      if constexpr (L0) hash_region(sig.h, pack_cs(0, c.s), c.base, c.size);
+      if constexpr (L0 && !DENSE) hash_region(sig.h, pack_cs(0, c.s), c.base, c.size);
       if (c.k > 0) c.A = (u128)(ull)null_scale(g, c.om) * lam[c.s] * (u128)(ull)c.k;
     }
     return c;
@@ -138,7 +138,7 @@ struct LMPolicy {
   }
   __device__ Probe probe(int32_t, const VCtx& vc, int32_t c) const {
     if (vc.single && vc.k > 0) {
-      if constexpr (L0)
+      if constexpr (L0 && !DENSE)
         return hash_first_at(sig.h, pack_cs(c, vc.s), vc.base, vc.size);
       else
         return sst_first<DENSE>(sig, c, vc.s);

@@ -732,7 +732,9 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
   const int32_t* active = batch ? S.lm_active : S.inst_active;
   const int nseg = S.p.K * NTIERS;
   auto decide = [&](const TierSegs& sg, const TrackView& t) {
-    if (S.sig.d)
+    if (S.sig.d && L.d.is0)
+      decide_all(c, lm_policy<true, true>(S, L, labels, t), sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
+    else if (S.sig.d)
       decide_all(c, lm_policy<true>(S, L, labels, t), sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
     else if (L.d.is0)
       decide_all(c, lm_policy<false, true>(S, L, labels, t), sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);

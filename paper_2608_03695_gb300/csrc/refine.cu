@@ -160,7 +160,8 @@ __global__ void k_wc(LevelDev g, const int32_t* sizeR, const long long* Wout, co
   ref_wc(g, sizeR, Wout, rhs, elig, cls, wc, desc);
 }
 
-template <bool DENSE>
+// L0: a level-0 policy (see LMPolicy).
+template <bool DENSE, bool L0 = false>
 struct RefPolicy {
   static constexpr int MIN_BLOCKS = DENSE ? MSLICE_DENSE_MIN_BLOCKS : MSLICE_GROUP_MIN_BLOCKS;
   LevelDev g;
@@ -190,12 +191,13 @@ struct RefPolicy {
     long long k;
     Omega om;
     u128 A;
+    uint64_t base, size;  // L0: the snapshot's hash region
   };
 
   __device__ bool begin(int32_t v) const { return sizeR[R[v]] == 1 && elig[v]; }
   __device__ VCtx vctx(int32_t v) const {
     VCtx c;
-    c.single = g.is0 != 0;
+    c.single = L0 || g.is0 != 0;
     c.s = 0;
     c.k = 0;
     c.A = 0;
@@ -204,6 +206,7 @@ struct RefPolicy {
     if (c.single) {
       c.k = g.k0[v];
       c.s = node_slice0(g, v);
+      if constexpr (L0 && !DENSE) hash_region(kr.h, pack_cs(0, c.s), c.base, c.size);
       if (c.k > 0) c.A = (u128)(ull)null_scale(g, c.om) * lam[c.s] * (u128)(ull)c.k;
     }
     return c;
@@ -211,7 +214,7 @@ struct RefPolicy {
   __device__ void skip(int32_t v) const { target[v] = NO_MOVE; }
   __device__ bool edge(int32_t v, const VCtx& vc, int64_t e, int32_t& key, long long& w) const {
     int32_t u;
-    if (!edge_at(g, e, u, w, vc.om)) return false;
+    if (!edge_at<L0>(g, e, u, w, vc.om)) return false;
     const unsigned long long pr = (unsigned long long)PR[u];  // (P[u], R[u]) in one load
     if ((int32_t)(pr >> 32) != vc.Pv) return false;
     key = (int32_t)(uint32_t)pr;
@@ -225,7 +228,13 @@ struct RefPolicy {
     p.size = (int32_t)(uint32_t)d;
     p.cls = (uint8_t)(d >> 32);
     p.wc = (uint8_t)(d >> 40);
-    p.first = (vc.single && vc.k > 0) ? sst_first<DENSE>(kr, X, vc.s) : Slot{EMPTY_KEY, 0};
+    p.first = Slot{EMPTY_KEY, 0};
+    if (vc.single && vc.k > 0) {
+      if constexpr (L0 && !DENSE)
+        p.first = hash_first_at(kr.h, pack_cs(X, vc.s), vc.base, vc.size);
+      else
+        p.first = sst_first<DENSE>(kr, X, vc.s);
+    }
     return p;
   }
   // A singleton sub-community's label is its node, so cls[X] is the class of
@@ -234,7 +243,7 @@ struct RefPolicy {
     if (p.size == 1 && p.cls == q) return Cand{0, INT32_MAX};
     if (!p.wc) return Cand{0, INT32_MAX};
     i128 G;
-    if (vc.single) {
+    if (L0 || vc.single) {
       const long long x = vc.k > 0 ? sst_resolve<DENSE>(kr, X, vc.s, p.first) : 0;
       G = (((i128)W) << P_BITS) - (i128)(vc.A * (u128)(ull)x);
     } else {
@@ -253,7 +262,7 @@ struct RefPolicy {
     return Cand{G, X};
   }
   // slice-parallel scoring (block tiers, aggregated levels); own() is 0
-  __device__ int64_t slice_count(int32_t v) const { return g.is0 ? 0 : g.sptr[v + 1] - g.sptr[v]; }
+  __device__ int64_t slice_count(int32_t v) const { return L0 || g.is0 ? 0 : g.sptr[v + 1] - g.sptr[v]; }
   __device__ bool own_walks_slices() const { return false; }
   __device__ u128 null_part(int32_t v, const VCtx&, int32_t X, bool, int t, int nt) const {
     return null_sum_part<DENSE>(g, lam, kr, v, X, false, t, nt);
@@ -281,7 +290,7 @@ struct RefPolicy {
     const Probe p = probe(v, vc, X);
     if (p.size == 1 && p.cls == q) return false;
     if (!p.wc) return false;
-    if (vc.single) {
+    if (L0 || vc.single) {
       const long long x = vc.k > 0 ? sst_resolve<DENSE>(kr, X, vc.s, p.first) : 0;
       G = (((i128)W) << P_BITS) - (i128)(vc.A * (u128)(ull)x);
     } else {
@@ -1131,6 +1140,7 @@ static void refine_impl(Solver& S, const Level& L, const int32_t* P, int it, int
   pol.target = S.target;
   pol.Wsel = S.Wsel;
   pol.cls = S.cls;
+  pol.q = 0;
   const RandParams rp{S.p.seed, (uint64_t)it, (uint64_t)lvl, S.rdiv, (ull)S.p.theta_den};
   if (resident) {
     RefArgs a{};
@@ -1177,6 +1187,11 @@ static void refine_impl(Solver& S, const Level& L, const int32_t* P, int it, int
                 pol, a);
     return;
   }
+  const auto level0 = [](const RefPolicy<DENSE>& p) {
+    return RefPolicy<DENSE, true>{p.g,  p.P,   p.R,   p.desc, p.PR,     p.sizeR, p.elig,
+                                  p.wc, p.cls, p.kr,  p.lam,  p.target, p.Wsel,  p.q};
+  };
+  RefPolicy<DENSE, true> pol0 = level0(pol);
   launch(c, k_classes, dim3(fixed_grid(8)), dim3(256), 0, L.d, S.p.seed, (uint64_t)it, (uint64_t)lvl, S.p.K, S.cls);
   for (int q = 0; q < S.p.K; ++q) {
     // well-connectedness of every sub-community at the sub-round start
@@ -1192,7 +1207,12 @@ static void refine_impl(Solver& S, const Level& L, const int32_t* P, int it, int
     if (S.p.theta_num > 0) {
       random_all<DENSE>(S, pol, sg, rp);
     } else {
-      decide_all(c, pol, sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
+      if (L.d.is0) {
+        pol0.q = q;
+        decide_all(c, pol0, sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
+      } else {
+        decide_all(c, pol, sg, S.tier_cnt, S.gkeys, S.gvals, S.goff);
+      }
     }
     launch(c, k_ref_apply<8, 0, 2>, dim3(fixed_grid(8)), dim3(256), 0, L.d, sg, P, (const int32_t*)S.target,
            (const long long*)S.Wc, (const long long*)S.Wsel, S.R, S.sizeR, S.Wout, S.kr, PR);
