@@ -183,8 +183,7 @@ typedef struct {
                                 nodes still moving (the synchronous schedule cycling), part of ms_local_move */
   int64_t capped_levels;     /* number of those levels */
   int64_t capped_rounds;     /* their local-moving rounds */
-  int64_t host_launches;     /* launch calls the host made for this call (kernels launched one by one, and
-                                graph launches, each counting once however many kernels the graph runs) */
+  int64_t host_launches;     /* launch calls the host made for this call */
 } mslice_stats;
 
 /* Defaults above; stop_level = -1. */

@@ -61,11 +61,10 @@ struct StreamFan {
 struct Ctx {
   cudaStream_t stream = nullptr;
   StreamFan* fan = nullptr;      // nullptr: tiers run one after another
-  bool capturing = false;        // launches are being captured into a graph
   Workspace* ws = nullptr;
   unsigned* d_status = nullptr;  // device error bits
   int64_t launches = 0;
-  int64_t host_launches = 0;     // launch calls the host made (a graph launch counts once)
+  int64_t host_launches = 0;     // launch calls the host made
   bool profile = false;          // event-time the decision kernels
   // MSLICE_TRACE: every launch is bracketed by CUDA events (per-kernel table
   // printed at the end of a solve)
@@ -85,7 +84,7 @@ inline void launch(Ctx& c, void (*k)(KArgs...), dim3 grid, dim3 block, size_t sm
   if (c.trace) trace_begin(c, (const void*)k, &e0);
   k<<<grid, block, smem, c.stream>>>(std::forward<Args>(args)...);
   c.launches++;
-  if (!c.capturing) c.host_launches++;
+  c.host_launches++;
   check_cuda(cudaGetLastError(), "kernel launch");
   if (c.trace) trace_end(c, (const void*)k, e0);
 }
@@ -114,10 +113,7 @@ inline void launch_coop(Ctx& c, void (*k)(KArgs...), dim3 grid, dim3 block, size
   void* argv[] = {(void*)&args...};
   cudaEvent_t e0 = nullptr;
   if (c.trace) trace_begin(c, (const void*)k, &e0);
-  if (c.capturing) {
-    // ordered as a whole by the graph's launch
-    check_cuda(cudaLaunchCooperativeKernel((const void*)k, grid, block, argv, smem, c.stream), "cooperative launch");
-  } else {
+  {
     CoopOrder order(c.stream);
     check_cuda(cudaLaunchCooperativeKernel((const void*)k, grid, block, argv, smem, c.stream), "cooperative launch");
     c.host_launches++;
@@ -155,15 +151,10 @@ void check_status(Ctx& c, const char* where);
 
 // ---- primitives (primitives.cu) ----
 // out[i] = sum_{j<i} in[j] (int64 accumulation); *d_total (device, nullable)
-// receives the full sum.  in and out may alias.  With `cond` (device,
-// nullable) the kernels do nothing when *cond == 0, so a scan can sit in a
-// stream behind work whose outcome decides whether it is needed.
-void scan_excl(Ctx& c, const int32_t* in, int64_t* out, int64_t n, int64_t* d_total,
-               const int32_t* cond = nullptr);
-void scan_excl(Ctx& c, const int64_t* in, int64_t* out, int64_t n, int64_t* d_total,
-               const int32_t* cond = nullptr);
-void scan_excl(Ctx& c, const int32_t* in, int32_t* out, int64_t n, int32_t* d_total,
-               const int32_t* cond = nullptr);
+// receives the full sum.  in and out may alias.
+void scan_excl(Ctx& c, const int32_t* in, int64_t* out, int64_t n, int64_t* d_total);
+void scan_excl(Ctx& c, const int64_t* in, int64_t* out, int64_t n, int64_t* d_total);
+void scan_excl(Ctx& c, const int32_t* in, int32_t* out, int64_t n, int32_t* d_total);
 
 void fill_i32(Ctx& c, int32_t* p, int32_t v, int64_t n);
 void fill_i64(Ctx& c, int64_t* p, int64_t v, int64_t n);

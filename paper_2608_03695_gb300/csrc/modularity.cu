@@ -20,8 +20,8 @@
 // FP64 order: I + omega*J, divided by 2mu; S' divided by the product
 // 2M'*2M' (each converted first); times gamma; subtracted.
 //
-// Also: canonical relabelling (first occurrence order), distinct counting
-// and the order-free level checksum used by the step-level tests.
+// Also: canonical relabelling (first occurrence order) and the order-free
+// level checksum used by the step-level tests.
 #include <cstring>
 #include <vector>
 

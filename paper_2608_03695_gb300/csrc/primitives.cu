@@ -42,8 +42,7 @@ __device__ __forceinline__ T block_excl_scan(T x, T* sm, T& total) {
 }
 
 template <class In, class Acc>
-__global__ void k_tile_reduce(const In* in, int64_t n, Acc* bsum, const int32_t* cond) {
-  if (cond && *cond == 0) return;
+__global__ void k_tile_reduce(const In* in, int64_t n, Acc* bsum) {
   __shared__ Acc sm[33];
   const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
   Acc t = 0;
@@ -58,8 +57,7 @@ __global__ void k_tile_reduce(const In* in, int64_t n, Acc* bsum, const int32_t*
 }
 
 template <class In, class Out, class Acc>
-__global__ void k_tile_scan(const In* in, Out* out, int64_t n, const Acc* boff, Out* d_total, const int32_t* cond) {
-  if (cond && *cond == 0) return;
+__global__ void k_tile_scan(const In* in, Out* out, int64_t n, const Acc* boff, Out* d_total) {
   __shared__ Acc sm[33];
   const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
   Acc v[SCAN_ITEMS];
@@ -83,21 +81,20 @@ __global__ void k_tile_scan(const In* in, Out* out, int64_t n, const Acc* boff, 
 }
 
 template <class In, class Out, class Acc>
-void scan_impl(Ctx& c, const In* in, Out* out, int64_t n, Out* d_total, int depth, const int32_t* cond) {
+void scan_impl(Ctx& c, const In* in, Out* out, int64_t n, Out* d_total, int depth) {
   if (n <= 0) {
     if (d_total) check_cuda(cudaMemsetAsync(d_total, 0, sizeof(Out), c.stream), "memset");
     return;
   }
   const unsigned nb = grid_for(n, SCAN_TILE);
   if (nb == 1) {
-    launch(c, k_tile_scan<In, Out, Acc>, dim3(1), dim3(SCAN_THREADS), 0, in, out, n, (const Acc*)nullptr, d_total,
-           cond);
+    launch(c, k_tile_scan<In, Out, Acc>, dim3(1), dim3(SCAN_THREADS), 0, in, out, n, (const Acc*)nullptr, d_total);
     return;
   }
   Acc* bsum = c.ws->get<Acc>("scan_bsum" + std::to_string(depth), nb);
-  launch(c, k_tile_reduce<In, Acc>, dim3(nb), dim3(SCAN_THREADS), 0, in, n, bsum, cond);
-  scan_impl<Acc, Acc, Acc>(c, bsum, bsum, (int64_t)nb, (Acc*)nullptr, depth + 1, cond);
-  launch(c, k_tile_scan<In, Out, Acc>, dim3(nb), dim3(SCAN_THREADS), 0, in, out, n, (const Acc*)bsum, d_total, cond);
+  launch(c, k_tile_reduce<In, Acc>, dim3(nb), dim3(SCAN_THREADS), 0, in, n, bsum);
+  scan_impl<Acc, Acc, Acc>(c, bsum, bsum, (int64_t)nb, (Acc*)nullptr, depth + 1);
+  launch(c, k_tile_scan<In, Out, Acc>, dim3(nb), dim3(SCAN_THREADS), 0, in, out, n, (const Acc*)bsum, d_total);
 }
 
 __global__ void k_fill_i32(int32_t* p, int32_t v, int64_t n) {
@@ -121,14 +118,14 @@ unsigned grid_stride(int64_t n) {
 
 }  // namespace
 
-void scan_excl(Ctx& c, const int32_t* in, int64_t* out, int64_t n, int64_t* d_total, const int32_t* cond) {
-  scan_impl<int32_t, int64_t, long long>(c, in, out, n, d_total, 0, cond);
+void scan_excl(Ctx& c, const int32_t* in, int64_t* out, int64_t n, int64_t* d_total) {
+  scan_impl<int32_t, int64_t, long long>(c, in, out, n, d_total, 0);
 }
-void scan_excl(Ctx& c, const int64_t* in, int64_t* out, int64_t n, int64_t* d_total, const int32_t* cond) {
-  scan_impl<int64_t, int64_t, long long>(c, in, out, n, d_total, 0, cond);
+void scan_excl(Ctx& c, const int64_t* in, int64_t* out, int64_t n, int64_t* d_total) {
+  scan_impl<int64_t, int64_t, long long>(c, in, out, n, d_total, 0);
 }
-void scan_excl(Ctx& c, const int32_t* in, int32_t* out, int64_t n, int32_t* d_total, const int32_t* cond) {
-  scan_impl<int32_t, int32_t, long long>(c, in, out, n, d_total, 0, cond);
+void scan_excl(Ctx& c, const int32_t* in, int32_t* out, int64_t n, int32_t* d_total) {
+  scan_impl<int32_t, int32_t, long long>(c, in, out, n, d_total, 0);
 }
 
 void fill_i32(Ctx& c, int32_t* p, int32_t v, int64_t n) {
