@@ -640,7 +640,7 @@ __device__ __forceinline__ void lm_empty(const LevelDev& g, int32_t B, int32_t* 
 // movement (T = 64, n = 100,000), hence the sixteenth of the expected movement.
 // Levels of 2^22, 2^20 and 2^18 entries as the least to track: within 1% of one
 // another; tracking every level of 2^16 nodes: 0.85x on a long contact sequence
-// and 0.89x on n = 400 graphs, whose pushes cost more than their decisions. With
+// and 0.89x on n = 1,000 graphs, whose pushes cost more than their decisions. With
 // the strength-list rule the contact sequence went from 162 to 150 ms.
 constexpr int64_t TRACK_MIN_ENTRIES = 1 << 20, TRACK_MIN_DEGREE = 8;
 constexpr int64_t TRACK_MIN_LOOKUPS = 1 << 21;
