@@ -973,7 +973,7 @@ static Resident aggregate_resident(Solver& S, const Level& L, const int32_t* P, 
   check_cuda(cudaFuncSetAttribute(k_aggregate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TIER4_SMEM_BYTES),
              "resident aggregation's shared memory");
   const int64_t want = std::max<int64_t>((L.nnz + 4095) / 4096, (N + RT - 1) / RT);
-  launch_coop(c, k_aggregate, dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(want, S.sms))), dim3(RT),
+  launch_coop(c, k_aggregate, dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(want, coop_share(S.sms)))), dim3(RT),
               TIER4_SMEM_BYTES, a);
   AggCtl h;
   std::memcpy(&h, readback(c, a.ctl, sizeof(AggCtl)), sizeof(AggCtl));

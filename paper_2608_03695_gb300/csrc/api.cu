@@ -8,6 +8,7 @@
 #include <cstring>
 #include <atomic>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <functional>
 #include <new>
@@ -16,6 +17,7 @@
 #include <vector>
 
 #include "../../include/mslice.h"
+#include "coop_budget.h"
 #include "solver.h"
 
 namespace mslice {
@@ -119,23 +121,67 @@ size_t Workspace::bytes_held() const {
 }
 
 namespace {
-std::mutex g_coop_mu;
-cudaEvent_t g_coop_ev[64] = {};
+constexpr int COOP_DEVICES = 64;
+struct CoopDevice {
+  std::mutex mu;
+  std::unique_ptr<CoopBudget> budget;
+  std::vector<cudaEvent_t> ev;  // by the budget's event numbers
+  std::atomic<int> solves{0};
+};
+
+int coop_device() {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < COOP_DEVICES ? dev : 0;
+}
+
+CoopDevice& coop_state(int dev) {
+  static CoopDevice* all = new CoopDevice[COOP_DEVICES];  // (outlives every thread that launches)
+  return all[dev];
+}
+
+// Whether an event has passed; an error that is pending stays pending.
+bool event_done(cudaEvent_t e) {
+  if (!e || cudaPeekAtLastError() != cudaSuccess) return false;
+  const cudaError_t r = cudaEventQuery(e);
+  if (r == cudaErrorNotReady) cudaGetLastError();
+  return r == cudaSuccess;
+}
 }  // namespace
 
-CoopOrder::CoopOrder(cudaStream_t s) : s_(s) {
-  g_coop_mu.lock();
-  if (cudaGetDevice(&dev_) != cudaSuccess || dev_ < 0 || dev_ >= 64) dev_ = 0;
-  if (!g_coop_ev[dev_]) {
-    if (cudaEventCreateWithFlags(&g_coop_ev[dev_], cudaEventDisableTiming) != cudaSuccess) g_coop_ev[dev_] = nullptr;
-  } else {
-    cudaStreamWaitEvent(s_, g_coop_ev[dev_], 0);
+CoopOrder::CoopOrder(cudaStream_t s, unsigned blocks) : s_(s) {
+  const int dev = coop_device();
+  CoopDevice& d = coop_state(dev);
+  lock_ = std::unique_lock<std::mutex>(d.mu);
+  if (!d.budget) {
+    int sms = 0;
+    check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "attribute");
+    d.budget = std::make_unique<CoopBudget>(sms);
   }
+  std::vector<int> wait;
+  const int e = d.budget->take((int)std::min(blocks, 1u << 30), (uintptr_t)s,
+                               [&](int x) { return event_done(d.ev[x]); }, wait);
+  if ((int)d.ev.size() <= e) d.ev.resize(e + 1, nullptr);
+  try {
+    for (int x : wait)
+      if (d.ev[x]) check_cuda(cudaStreamWaitEvent(s_, d.ev[x], 0), "stream wait");
+    if (!d.ev[e]) check_cuda(cudaEventCreateWithFlags(&d.ev[e], cudaEventDisableTiming), "event");
+  } catch (...) {
+    cudaDeviceSynchronize();  // the units are this grid's now: nothing may still run on them
+    throw;
+  }
+  end_ = d.ev[e];
 }
 
 CoopOrder::~CoopOrder() {
-  if (g_coop_ev[dev_]) cudaEventRecord(g_coop_ev[dev_], s_);
-  g_coop_mu.unlock();
+  if (cudaEventRecord(end_, s_) != cudaSuccess) cudaStreamSynchronize(s_);
+}
+
+SolveScope::SolveScope() : dev_(coop_device()) { coop_state(dev_).solves++; }
+SolveScope::~SolveScope() { coop_state(dev_).solves--; }
+
+int32_t coop_share(int32_t sms) {
+  const int n = coop_state(coop_device()).solves.load();
+  return std::max(1, sms / std::max(1, std::min(n, COOP_MAX_SHARES)));
 }
 
 void StreamFan::create() {

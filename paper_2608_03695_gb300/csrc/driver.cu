@@ -416,6 +416,7 @@ void set_instances(Ctx& c, Solver& S, const std::vector<InstParams>& jobs) {
 void run_leiden(Ctx& c, const SupraGraph& G, const std::vector<InstParams>& jobs, const SolveParams& p,
                 int stop_level, int stop_stage, int stop_rounds, const int32_t* init, int32_t* out, Solver& S,
                 RunOut& ro) {
+  const SolveScope solving;
   PhaseClock clock(c);
   cudaEvent_t t_all = clock.begin();
   const int32_t B = G.B;

@@ -6,6 +6,7 @@
 
 #include <cstdint>
 #include <map>
+#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
@@ -89,23 +90,40 @@ inline void launch(Ctx& c, void (*k)(KArgs...), dim3 grid, dim3 block, size_t sm
   if (c.trace) trace_end(c, (const void*)k, e0);
 }
 
-// Orders cooperative launches device-wide: a kernel with grid-wide barriers
-// starts only after the previous one (from any stream or thread of the
-// process) has finished, so two such grids never hold part of the SMs each
-// while waiting for the rest.  Every other kernel of the library runs to
-// completion without waiting on other blocks, so a cooperative grid always
-// becomes fully resident.
+// Orders cooperative launches device-wide, by any stream or thread of the
+// process: the grids that may run together never have more blocks than the
+// device has SMs (see coop_budget.h).
 class CoopOrder {
  public:
-  explicit CoopOrder(cudaStream_t s);  // waits for the previous cooperative kernel
-  ~CoopOrder();                        // marks this stream's point as the new one
+  CoopOrder(cudaStream_t s, unsigned blocks);  // waits for the grids whose SMs this one takes over
+  ~CoopOrder();                                // marks the stream's point as this grid's end
   CoopOrder(const CoopOrder&) = delete;
   CoopOrder& operator=(const CoopOrder&) = delete;
 
  private:
   cudaStream_t s_;
+  cudaEvent_t end_ = nullptr;
+  std::unique_lock<std::mutex> lock_;
+};
+
+// A solve in progress on the current device.  Solves of several threads share
+// the SMs: coop_share(sms) is the part of them that a cooperative grid launched
+// now should keep to, so that the others' grids can run beside it.
+class SolveScope {
+ public:
+  SolveScope();
+  ~SolveScope();
+  SolveScope(const SolveScope&) = delete;
+  SolveScope& operator=(const SolveScope&) = delete;
+
+ private:
   int dev_ = 0;
 };
+// (At most COOP_MAX_SHARES parts; beyond that grids wait for one another.  Solves
+// per second of 4 and 8 threads, planted n = 20,000, T = 3: 157 and 116; at most 4
+// parts 157 and 97, 16 parts 157 and 118; whole-device grids in turn 67 and 67.)
+constexpr int COOP_MAX_SHARES = 8;
+int32_t coop_share(int32_t sms);
 
 // Cooperative launch (grid-wide barriers); the grid must be co-resident.
 template <class... KArgs, class... Args>
@@ -114,7 +132,7 @@ inline void launch_coop(Ctx& c, void (*k)(KArgs...), dim3 grid, dim3 block, size
   cudaEvent_t e0 = nullptr;
   if (c.trace) trace_begin(c, (const void*)k, &e0);
   {
-    CoopOrder order(c.stream);
+    CoopOrder order(c.stream, grid.x);
     check_cuda(cudaLaunchCooperativeKernel((const void*)k, grid, block, argv, smem, c.stream), "cooperative launch");
     c.host_launches++;
   }

@@ -296,7 +296,7 @@ void resident_rounds(Solver& S, const Level& L, int32_t* labels, int it, int lvl
   a.ctl = reinterpret_cast<ResidentCtl*>(reinterpret_cast<char*>(S.cursors) + lengths);
   a.build = in.build ? 1 : 0;
   check_cuda(cudaMemsetAsync(S.cursors, 0, lengths + sizeof(ResidentCtl), c.stream), "memset");
-  const unsigned grid = resident_grid(L.d.N, (int64_t)S.tier_cnt[3] + S.tier_cnt[4], S.p.K, S.sms);
+  const unsigned grid = resident_grid(L.d.N, (int64_t)S.tier_cnt[3] + S.tier_cnt[4], S.p.K, coop_share(S.sms));
   if (S.sig.d)
     launch_rounds(c, lm_policy<true>(S, L, labels, trk), a, grid);
   else

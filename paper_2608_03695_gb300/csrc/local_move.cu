@@ -814,7 +814,9 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
       }
       launch(c, tracked ? k_lm_apply<true> : k_lm_apply<false>, dim3(fixed_grid(4)), dim3(APPLY_THREADS), 0, L.d, sg, labels, S.size, S.sig, S.target,
              S.counters, batch ? S.inst_moved : nullptr, tr, bl, q);
-      launch_coop(c, k_empty_pass, dim3(S.empty_grid), dim3(EMPTY_THREADS), 0, L.d, S.B, S.target, labels, S.size,
+      // (all of the co-resident grid, unless other solves share the SMs)
+      const int32_t share = coop_share(S.sms);
+      launch_coop(c, k_empty_pass, dim3(share < S.sms ? std::min(share, S.empty_grid) : S.empty_grid), dim3(EMPTY_THREADS), 0, L.d, S.B, S.target, labels, S.size,
                   S.sig, S.counters, S.empty_blk, S.freelist, S.tmp32b, S.inst_cnt, tr, bl, q + 1);
     }
     if (batch)

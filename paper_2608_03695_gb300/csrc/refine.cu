@@ -1183,7 +1183,7 @@ static void refine_impl(Solver& S, const Level& L, const int32_t* P, int it, int
     const auto k = random ? k_refine<DENSE, true> : k_refine<DENSE, false>;
     check_cuda(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
                "resident refinement's shared memory");
-    launch_coop(c, k, dim3(resident_grid(N, (int64_t)S.tier_cnt[3] + S.tier_cnt[4], S.p.K, S.sms)), dim3(RT), bytes,
+    launch_coop(c, k, dim3(resident_grid(N, (int64_t)S.tier_cnt[3] + S.tier_cnt[4], S.p.K, coop_share(S.sms))), dim3(RT), bytes,
                 pol, a);
     return;
   }
