@@ -259,8 +259,10 @@ void* readback(Ctx& c, const void* dptr, size_t bytes) {
   return c.pinned;
 }
 
-void check_status(Ctx& c, const char* where) {
-  const unsigned st = *static_cast<const unsigned*>(readback(c, c.d_status, sizeof(unsigned)));
+void check_status(Ctx& c, const char* where, unsigned* info) {
+  const unsigned* w = static_cast<const unsigned*>(readback(c, c.d_status, 2 * sizeof(unsigned)));
+  const unsigned st = w[0];
+  if (info) *info = w[1];
   if (st == 0) return;
   check_cuda(cudaMemsetAsync(c.d_status, 0, sizeof(unsigned), c.stream), "memset");
   if (st & ERR_BAD_INPUT) fail(MSLICE_EINVAL, std::string(where) + ": malformed input");

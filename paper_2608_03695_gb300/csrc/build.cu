@@ -13,6 +13,7 @@
 #include "../../include/mslice.h"
 
 #include <algorithm>
+#include <numeric>
 
 namespace mslice {
 
@@ -24,7 +25,8 @@ struct SliceTable {
   const int32_t* const* weights;
 };
 
-// indptr of every snapshot: starts at 0, non-decreasing, ends at nnz_s.
+// indptr of every snapshot: starts at 0, non-decreasing, ends at nnz_s.  status[1]:
+// some row is a hub's.
 __global__ void k_check_indptr(SliceTable st, const int64_t* nnz, int32_t T, int64_t n, unsigned* status) {
   const int64_t total = n * (int64_t)T;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < total; v += (int64_t)gridDim.x * blockDim.x) {
@@ -35,6 +37,7 @@ __global__ void k_check_indptr(SliceTable st, const int64_t* nnz, int32_t T, int
     if (i == 0 && a != 0) bad = true;
     if (i == n - 1 && b != nnz[s]) bad = true;
     if (bad) atomicOr(status, ERR_BAD_INPUT);
+    if (b - a > HUB_ROW) status[1] = 1;
   }
 }
 
@@ -49,7 +52,7 @@ __device__ __forceinline__ int32_t coupling_flag(int32_t coupling, int32_t T, in
   return coupling == 0 ? -((s < r ? s : r) + 1) : -(s * T + r + 1);
 }
 
-// Rows: BUILD_LANES lanes per supra-row check the snapshot row and write the
+// Rows: G lanes per supra-row check the snapshot row and write the
 // supra-row in the same pass: rowptr (in closed form: first[s] entries come
 // before snapshot s, and every row of a snapshot has the same coupling entries),
 // the shifted entries, the coupling flags and k_v = sum of the row's weights.
@@ -61,17 +64,29 @@ __device__ __forceinline__ int32_t coupling_flag(int32_t coupling, int32_t T, in
 // The searches bound the pass (about four dependent lookups each, a few rows
 // away in L2); checking and copying apart, with a search per entry and a scan
 // for the row pointers, took 1.6 ms for 31 M entries.
-// Rows of more than BUILD_LONG entries are taken by the whole warp: with 8 lanes
-// a row of 1,400 entries alone took as long as the rest of the pass.
-constexpr int BUILD_LANES = 8;
+// G = 8, where rows are short and there are more of them than warps: with a warp
+// each, most lanes of a warp have no entry.  Rows of more than BUILD_LONG entries
+// are then taken by the whole warp (with 8 lanes a row of 1,400 entries alone took
+// as long as the rest of the pass), and rows of more than HUB_ROW by blocks of
+// their own (k_build_hubs): a warp takes the long ones of its four rows one after
+// another, and where hubs are neighbours in node order that alone was the pass.
+// G = 32 (a warp a row), where the rows are long on average or there are warps for
+// all of them.
+// Builds, four long rows a warp in turn -> now (a warp a row before that): hubs of
+// 100,000, 60,000, 20,000 and 40 of 3,000 (N = 300,000) 12.0 -> 0.77 ms (6.9); 12
+// hubs of 6,000 (N = 60,000) 1.60 -> 0.58 (0.88); one snapshot of 1,500 nodes,
+// every second pair linked, 0.77 -> 0.60 (0.61).  Hubs from 512 entries on: 3%
+// slower on a power-law graph of n = 100,000 (rows up to 1,400, 2,560 of them).
 constexpr int64_t BUILD_LONG = 64;
+constexpr int BUILD_HUB_PARTS = 8;                // blocks that share a hub's row
+constexpr int64_t BUILD_WARPS = 152 * (2048 / 32);  // resident at a time
 
-// Entries gl, gl + step, ... of row i of a snapshot (entries [a, b)): checked and
-// written at out.
+// Entries from + gl, from + gl + step, ... (up to `to`) of row i of a snapshot
+// (entries from a on): checked and written at out.
 __device__ __forceinline__ void build_entries(const int64_t* ip, const int32_t* ix, const int32_t* wt, int32_t n,
-                                              int32_t i, int64_t a, int64_t b, int2* out, int32_t off, int gl, int step,
-                                              long long& ksum, int& above, bool& bad) {
-  for (int64_t e = a + gl; e < b; e += step) {
+                                              int32_t i, int64_t a, int64_t from, int64_t to, int2* out, int32_t off,
+                                              int gl, int step, long long& ksum, int& above, bool& bad) {
+  for (int64_t e = from + gl; e < to; e += step) {
     const int32_t j = ix[e];
     const int32_t w = wt[e];
     out[e - a] = make_int2(j + off, w);
@@ -97,22 +112,38 @@ __device__ __forceinline__ void build_entries(const int64_t* ip, const int32_t* 
   }
 }
 
+// What the rows' passes found (per warp): entries above less those below the
+// diagonal, and anything malformed.
+__device__ __forceinline__ void build_verdict(long long above, bool bad, ull* balance, unsigned* status) {
+  above = warp_sum(above);
+  const bool any = __any_sync(0xffffffffu, bad);
+  if ((threadIdx.x & 31) == 0) {
+    if (above) atomicAdd(balance, (ull)above);
+    if (any) atomicOr(status, ERR_BAD_INPUT);
+  }
+}
+
+// hubs: room for every row of more than HUB_ROW entries, hubs' number at
+// *nhubs; nullptr: those rows are taken here too.
+template <int G>
 __global__ void k_build_rows(SliceTable st, int32_t T, int64_t n, int32_t coupling, const int64_t* first,
-                             int64_t* rowptr, int2* adj, int64_t* k, ull* balance, unsigned* status) {
+                             int64_t* rowptr, int2* adj, int64_t* k, int32_t* hubs, ull* nhubs, ull* balance,
+                             unsigned* status) {
   const int64_t total = n * (int64_t)T;
-  const int lane = threadIdx.x & 31, gl = lane % BUILD_LANES;
-  const unsigned gmask = ((1u << BUILD_LANES) - 1u) << (lane - gl);
-  const int64_t groups = (int64_t)gridDim.x * blockDim.x / BUILD_LANES;
+  const int lane = threadIdx.x & 31, gl = lane % G;
+  const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (lane - gl);
+  const int64_t groups = (int64_t)gridDim.x * blockDim.x / G;
   const int32_t n32 = (int32_t)n;
   long long above_sum = 0;
   bool bad = false;
   // (warp-uniform loop)
-  for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / BUILD_LANES; v0 < total; v0 += groups) {
-    const int64_t v = v0 + lane / BUILD_LANES;
+  for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / G; v0 < total; v0 += groups) {
+    const int64_t v = v0 + lane / G;
     const bool ok = v < total;
     const int32_t s = ok ? (int32_t)v / n32 : 0, i = ok ? (int32_t)v - s * n32 : 0;
     const int64_t* ip = st.indptr[s];
     const int64_t a = ok ? ip[i] : 0, b = ok ? ip[i + 1] : 0;
+    const bool hub = hubs && b - a > HUB_ROW;
     int32_t lo, hi;
     coupled_range(coupling, T, s, lo, hi);
     int64_t out = first[s] + a + i * (int64_t)(hi - lo - 1);
@@ -120,40 +151,65 @@ __global__ void k_build_rows(SliceTable st, int32_t T, int64_t n, int32_t coupli
     long long ksum = 0;
     int above = 0;
     if (ok) {
-      if (gl == 0) rowptr[v] = out;
-      for (int32_t r = lo + gl; r < s; r += BUILD_LANES)
+      if (gl == 0) {
+        rowptr[v] = out;
+        if (hub) hubs[atomicAdd(nhubs, 1ull)] = (int32_t)v;
+      }
+      for (int32_t r = lo + gl; r < s; r += G)
         adj[out + (r - lo)] = make_int2(r * n32 + i, coupling_flag(coupling, T, s, r));
       out += s - lo;
-      for (int32_t r = s + 1 + gl; r < hi; r += BUILD_LANES)
+      for (int32_t r = s + 1 + gl; r < hi; r += G)
         adj[out + (b - a) + (r - s - 1)] = make_int2(r * n32 + i, coupling_flag(coupling, T, s, r));
-      if (b - a <= BUILD_LONG)
-        build_entries(ip, st.indices[s], st.weights[s], n32, i, a, b, adj + out, off, gl, BUILD_LANES, ksum, above,
-                      bad);
+      if (!hub && (G == 32 || b - a <= BUILD_LONG))
+        build_entries(ip, st.indices[s], st.weights[s], n32, i, a, a, b, adj + out, off, gl, G, ksum, above, bad);
     }
-    unsigned wide = __ballot_sync(0xffffffffu, gl == 0 && b - a > BUILD_LONG);
-    while (wide) {
-      const int src = __ffs(wide) - 1;
-      wide &= wide - 1;
-      const int32_t ss = __shfl_sync(0xffffffffu, s, src), is = __shfl_sync(0xffffffffu, i, src);
-      const int64_t as = __shfl_sync(0xffffffffu, a, src), bs = __shfl_sync(0xffffffffu, b, src),
-                    os = __shfl_sync(0xffffffffu, out, src);
-      long long kw = 0;
-      build_entries(st.indptr[ss], st.indices[ss], st.weights[ss], n32, is, as, bs, adj + os, ss * n32, lane, 32, kw,
-                    above, bad);
-      kw = warp_sum(kw);
-      if (lane == src) ksum = kw;  // (the others of the group hold 0)
+    if constexpr (G < 32) {
+      unsigned wide = __ballot_sync(0xffffffffu, gl == 0 && !hub && b - a > BUILD_LONG);
+      while (wide) {
+        const int src = __ffs(wide) - 1;
+        wide &= wide - 1;
+        const int32_t ss = __shfl_sync(0xffffffffu, s, src), is = __shfl_sync(0xffffffffu, i, src);
+        const int64_t as = __shfl_sync(0xffffffffu, a, src), bs = __shfl_sync(0xffffffffu, b, src),
+                      os = __shfl_sync(0xffffffffu, out, src);
+        long long kw = 0;
+        build_entries(st.indptr[ss], st.indices[ss], st.weights[ss], n32, is, as, as, bs, adj + os, ss * n32, lane, 32,
+                      kw, above, bad);
+        kw = warp_sum(kw);
+        if (lane == src) ksum = kw;  // (the others of the group hold 0)
+      }
     }
 #pragma unroll
-    for (int m = BUILD_LANES / 2; m >= 1; m >>= 1) ksum += __shfl_xor_sync(gmask, ksum, m);
-    if (ok && gl == 0) k[v] = ksum;
+    for (int m = G / 2; m >= 1; m >>= 1) ksum += __shfl_xor_sync(gmask, ksum, m);
+    if (ok && gl == 0) k[v] = ksum;  // (0 so far for a hub)
     above_sum += above;
   }
-  above_sum = warp_sum(above_sum);
-  const bool any = __any_sync(0xffffffffu, bad);
-  if (lane == 0) {
-    if (above_sum) atomicAdd(balance, (ull)above_sum);
-    if (any) atomicOr(status, ERR_BAD_INPUT);
+  build_verdict(above_sum, bad, balance, status);
+}
+
+// The snapshot rows of the hubs: blocks (x, 0 .. BUILD_HUB_PARTS - 1) share one.
+__global__ void __launch_bounds__(256)
+    k_build_hubs(SliceTable st, int32_t T, int64_t n, int32_t coupling, const int64_t* rowptr, int2* adj, int64_t* k,
+                 const int32_t* hubs, const ull* nhubs, ull* balance, unsigned* status) {
+  const int32_t n32 = (int32_t)n;
+  const int64_t count = (int64_t)*nhubs;
+  long long above_sum = 0;
+  bool bad = false;
+  for (int64_t h = blockIdx.x; h < count; h += gridDim.x) {
+    const int32_t v = hubs[h], s = v / n32, i = v - s * n32;
+    const int64_t a = st.indptr[s][i], b = st.indptr[s][i + 1];
+    const int64_t part = (b - a + gridDim.y - 1) / gridDim.y;
+    const int64_t from = min(b, a + blockIdx.y * part), to = min(b, from + part);
+    int32_t lo, hi;
+    coupled_range(coupling, T, s, lo, hi);
+    long long ksum = 0;
+    int above = 0;
+    build_entries(st.indptr[s], st.indices[s], st.weights[s], n32, i, a, from, to, adj + rowptr[v] + (s - lo), s * n32,
+                  threadIdx.x, blockDim.x, ksum, above, bad);
+    ksum = warp_sum(ksum);
+    if ((threadIdx.x & 31) == 0 && ksum) atomicAdd((ull*)&k[v], (ull)ksum);
+    above_sum += above;
   }
+  build_verdict(above_sum, bad, balance, status);
 }
 
 // 2m_s = sum of k_v over the rows of snapshot s: blockIdx.y is the snapshot,
@@ -233,10 +289,13 @@ void build_supra(Ctx& c, const std::vector<const int64_t*>& indptr, const std::v
   check_cuda(cudaMemcpyAsync(d_wt, weights.data(), T * sizeof(void*), cudaMemcpyHostToDevice, c.stream), "copy");
   check_cuda(cudaMemcpyAsync(d_nnz, nnz.data(), T * sizeof(int64_t), cudaMemcpyHostToDevice, c.stream), "copy");
   SliceTable st{d_ip, d_ix, d_wt};
-  check_cuda(cudaMemsetAsync(c.d_status, 0, sizeof(unsigned), c.stream), "memset");
+  check_cuda(cudaMemsetAsync(c.d_status, 0, 2 * sizeof(unsigned), c.stream), "memset");
+  g.hubs = false;
   if (g.N > 0) {
+    unsigned hubs = 0;
     launch(c, k_check_indptr, dim3(gs(g.N, 256)), dim3(256), 0, st, (const int64_t*)d_nnz, T, n, c.d_status);
-    check_status(c, "snapshot row pointers");
+    check_status(c, "snapshot row pointers", &hubs);
+    g.hubs = hubs != 0;
   }
   // entries before every snapshot, and in all
   std::vector<int64_t> first(T + 1, 0);
@@ -255,10 +314,21 @@ void build_supra(Ctx& c, const std::vector<const int64_t*>& indptr, const std::v
   g.two_m = static_cast<int64_t*>(g.mem.get_bytes("two_m", T * sizeof(int64_t)));
   check_cuda(cudaMemsetAsync(g.two_m, 0, T * sizeof(int64_t), c.stream), "memset");
   if (g.N > 0) {
-    ull* balance = c.ws->get<ull>("b_balance", 1);
-    check_cuda(cudaMemsetAsync(balance, 0, sizeof(ull), c.stream), "memset");
-    launch(c, k_build_rows, dim3(gs(g.N * BUILD_LANES, 256)), dim3(256), 0, st, T, n, coupling,
-           (const int64_t*)d_first, g.rowptr, g.adj, g.k, balance, c.d_status);
+    ull* balance = c.ws->get<ull>("b_balance", 2);
+    ull* nhubs = balance + 1;
+    check_cuda(cudaMemsetAsync(balance, 0, 2 * sizeof(ull), c.stream), "memset");
+    const int64_t entries = std::accumulate(nnz.begin(), nnz.end(), (int64_t)0);
+    const bool all_warps = g.N <= BUILD_WARPS;
+    int32_t* hubs = g.hubs && !all_warps ? c.ws->get<int32_t>("b_hubs", entries / HUB_ROW + 1) : nullptr;
+    if (all_warps || entries > BUILD_LONG * g.N)
+      launch(c, k_build_rows<32>, dim3(gs(g.N * 32, 256)), dim3(256), 0, st, T, n, coupling, (const int64_t*)d_first,
+             g.rowptr, g.adj, g.k, hubs, nhubs, balance, c.d_status);
+    else
+      launch(c, k_build_rows<8>, dim3(gs(g.N * 8, 256)), dim3(256), 0, st, T, n, coupling, (const int64_t*)d_first,
+             g.rowptr, g.adj, g.k, hubs, nhubs, balance, c.d_status);
+    if (hubs)
+      launch(c, k_build_hubs, dim3(76, BUILD_HUB_PARTS), dim3(256), 0, st, T, n, coupling, (const int64_t*)g.rowptr,
+             g.adj, g.k, (const int32_t*)hubs, (const ull*)nhubs, balance, c.d_status);
     unsigned gx = (unsigned)std::min<int64_t>((n + 255) / 256, 64);
     launch(c, k_slice_mass, dim3(gx, T), dim3(256), 0, (const int64_t*)g.k, n, (ull*)g.two_m);
     const bool mirrored = *static_cast<const ull*>(readback(c, balance, sizeof(ull))) == 0;
@@ -285,16 +355,19 @@ void concat_instances(Ctx& c, const std::vector<const SupraGraph*>& parts, Supra
   out.inst.assign(B, InstInfo{});
   int64_t N = 0, nnz = 0, nnz_intra = 0, ncw = 0;
   int32_t T = 0;
+  bool hubs = false;
   for (int32_t i = 0; i < B; ++i) {
     out.inst[i] = InstInfo{parts[i]->n, N, parts[i]->T, T, parts[i]->coupling, ncw};
     N += parts[i]->N;
     nnz += parts[i]->nnz;
     nnz_intra += parts[i]->nnz_intra;
+    hubs = hubs || parts[i]->hubs;
     T += parts[i]->T;
     ncw += parts[i]->ncw;
   }
   if (ncw >= INT32_MAX) fail(MSLICE_EINVAL, "the batch's coupling tables need fewer than 2^31 slots");
   out.ncw = ncw;
+  out.hubs = hubs;
   out.coupling = -1;  // per instance
   out.N = N;
   out.T = T;

@@ -22,6 +22,10 @@ inline int64_t coupling_slots(int32_t coupling, int32_t T) {
   return coupling == 0 ? (T > 1 ? T - 1 : 0) : (int64_t)T * T;
 }
 
+// Rows of more entries than this are shared by several blocks where a pass takes
+// rows by lanes or warps.
+constexpr int64_t HUB_ROW = 2048;
+
 // Directed coupling entries of an instance.
 inline int64_t coupling_entries(int32_t coupling, int64_t n, int32_t T) {
   if (T < 2) return 0;
@@ -33,6 +37,7 @@ struct SupraGraph {
   int64_t n = 0, N = 0; // n: nodes per snapshot of a single instance
   int64_t nnz = 0;        // stored entries (intra both directions + coupling flags)
   int64_t nnz_intra = 0;  // intra-snapshot entries
+  bool hubs = false;      // some snapshot row has more than HUB_ROW entries
   int32_t coupling = 0;   // single graph: its coupling pattern (batches: per instance)
   int64_t ncw = 0;        // slots of omega^(sr) numerators over all instances
   int64_t* rowptr = nullptr;  // N+1

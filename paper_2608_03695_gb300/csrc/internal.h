@@ -63,7 +63,7 @@ struct Ctx {
   cudaStream_t stream = nullptr;
   StreamFan* fan = nullptr;      // nullptr: tiers run one after another
   Workspace* ws = nullptr;
-  unsigned* d_status = nullptr;  // device error bits
+  unsigned* d_status = nullptr;  // device error bits; a second word for what a build finds out
   int64_t launches = 0;
   int64_t host_launches = 0;     // launch calls the host made
   bool profile = false;          // event-time the decision kernels
@@ -165,7 +165,7 @@ constexpr size_t PINNED_BYTES = 4096;
 void* readback(Ctx& c, const void* dptr, size_t bytes);
 void sync(Ctx& c);
 // Synchronises and throws if the device status word holds an error bit.
-void check_status(Ctx& c, const char* where);
+void check_status(Ctx& c, const char* where, unsigned* info = nullptr);
 
 // ---- primitives (primitives.cu) ----
 // out[i] = sum_{j<i} in[j] (int64 accumulation); *d_total (device, nullable)

@@ -31,10 +31,19 @@ namespace mslice {
 
 namespace {
 
-// I and J of every instance (IJ: 2 words per instance): 8 lanes a row, the whole
-// warp for a row of more than 64 entries.  A warp's rows ascend, and so do their
+// I and J of every instance (IJ: 2 words per instance): G lanes a row, as in
+// k_build_rows: 8 where rows are short and there are more of them than warps, with
+// the whole warp for a row of more than IJ_LONG entries and blocks of their own
+// (k_IJ_hubs) for rows of more than HUB_ROW; a warp a row otherwise (from 32
+// entries on average: at 62 a row 0.32 ms against 0.34).  Hubs of 100,000, 60,000,
+// 20,000 and 40 of 3,000 (N = 300,000): Q 2.26 ms with a warp's four long rows in
+// turn, 1.33 with a warp a row, 0.27 now.  A warp's rows ascend, and so do their
 // instances: sums go out when the instance changes and at the end (one atomic a
 // row on B words took 1.5 ms of a batch of 36, N = 1.5 M).
+constexpr int64_t IJ_LONG = 64, IJ_DENSE = 32;
+constexpr int IJ_HUB_PARTS = 8;
+constexpr int64_t IJ_WARPS = 152 * (2048 / 32);  // resident at a time
+
 __device__ __forceinline__ void ij_row(const LevelDev& g, const int32_t* labels, int32_t c, int64_t b, int64_t e,
                                        int t, int nt, ull& I, ull& J) {
   for (int64_t q = b + t; q < e; q += nt) {
@@ -48,9 +57,9 @@ __device__ __forceinline__ void ij_row(const LevelDev& g, const int32_t* labels,
   }
 }
 
-__global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B) {
-  constexpr int G = 8;
-  constexpr int64_t LONG = 64;
+// hubs, nhubs: see k_build_rows.
+template <int G>
+__global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B, int32_t* hubs, ull* nhubs) {
   const int lane = threadIdx.x & 31, gl = lane % G;
   const int64_t groups = (int64_t)gridDim.x * blockDim.x / G;
   ull I = 0, J = 0;
@@ -68,6 +77,7 @@ __global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B) {
     const int64_t v = v0 + lane / G;
     const bool ok = v < g.N;
     const int64_t b = ok ? g.rowptr[v] : 0, e = ok ? g.rowptr[v + 1] : 0;
+    const bool hub = hubs && e - b > HUB_ROW;
     const int32_t c = ok ? labels[v] : 0;
     const int32_t inst = B > 1 ? node_inst(g, (int32_t)(ok ? v : v0)) : 0;
     const int32_t first = __shfl_sync(0xffffffffu, inst, 0);
@@ -76,19 +86,22 @@ __global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B) {
       flush();
       cur = first;
     }
-    if (e - b <= LONG) ij_row(g, labels, c, b, e, gl, G, I, J);
-    unsigned wide = __ballot_sync(0xffffffffu, gl == 0 && e - b > LONG);
-    while (wide) {
-      const int src = __ffs(wide) - 1;
-      wide &= wide - 1;
-      ull Iw = 0, Jw = 0;
-      ij_row(g, labels, __shfl_sync(0xffffffffu, c, src), __shfl_sync(0xffffffffu, b, src),
-             __shfl_sync(0xffffffffu, e, src), lane, 32, Iw, Jw);
-      Iw = warp_sum(Iw);
-      Jw = warp_sum(Jw);
-      if (lane == src) {
-        I += Iw;
-        J += Jw;
+    if (hub && gl == 0) hubs[atomicAdd(nhubs, 1ull)] = (int32_t)v;
+    if (!hub && (G == 32 || e - b <= IJ_LONG)) ij_row(g, labels, c, b, e, gl, G, I, J);
+    if constexpr (G < 32) {
+      unsigned wide = __ballot_sync(0xffffffffu, gl == 0 && !hub && e - b > IJ_LONG);
+      while (wide) {
+        const int src = __ffs(wide) - 1;
+        wide &= wide - 1;
+        ull Iw = 0, Jw = 0;
+        ij_row(g, labels, __shfl_sync(0xffffffffu, c, src), __shfl_sync(0xffffffffu, b, src),
+               __shfl_sync(0xffffffffu, e, src), lane, 32, Iw, Jw);
+        Iw = warp_sum(Iw);
+        Jw = warp_sum(Jw);
+        if (lane == src) {
+          I += Iw;
+          J += Jw;
+        }
       }
     }
     if (!alike) {  // rows of several instances: each lane's sums go out alone
@@ -98,6 +111,27 @@ __global__ void k_IJ(LevelDev g, const int32_t* labels, ull* IJ, int32_t B) {
     }
   }
   flush();
+}
+
+// The hubs' rows: blocks (x, 0 .. IJ_HUB_PARTS - 1) share one.
+__global__ void __launch_bounds__(256)
+    k_IJ_hubs(LevelDev g, const int32_t* labels, ull* IJ, int32_t B, const int32_t* hubs, const ull* nhubs) {
+  const int64_t count = (int64_t)*nhubs;
+  for (int64_t h = blockIdx.x; h < count; h += gridDim.x) {
+    const int32_t v = hubs[h];
+    const int64_t b = g.rowptr[v], e = g.rowptr[v + 1];
+    const int64_t part = (e - b + gridDim.y - 1) / gridDim.y;
+    const int64_t from = min(e, b + blockIdx.y * part), to = min(e, from + part);
+    ull I = 0, J = 0;
+    ij_row(g, labels, labels[v], from, to, threadIdx.x, blockDim.x, I, J);
+    I = warp_sum(I);
+    J = warp_sum(J);
+    if ((threadIdx.x & 31) == 0) {
+      const int32_t inst = B > 1 ? node_inst(g, v) : 0;
+      if (I) atomicAdd(&IJ[2 * inst], I);
+      if (J) atomicAdd(&IJ[2 * inst + 1], J);
+    }
+  }
 }
 
 // S_s += Sigma_{c,s}^2 over the table; per-block partial sums in shared
@@ -271,7 +305,9 @@ void modularity(Solver& S, const int32_t* labels0, double* Q) {
   configure_stores(S, G.N);
   sigma_rebuild(S, Level{g}, labels0);
   const int32_t Tn = S.Tn;
-  ull* acc = c.ws->get<ull>("q_acc", 2 * (size_t)B + 2 * (size_t)Tn);
+  // I and J per instance, S per null slice, the hubs' number
+  const size_t accs = 2 * (size_t)B + 2 * (size_t)Tn;
+  ull* acc = c.ws->get<ull>("q_acc", accs + 1);
   double* dQ = c.ws->get<double>("q_out", B);
   QInst* dqi = c.ws->get<QInst>("q_inst", B);
   std::vector<QInst> qi(B);
@@ -281,8 +317,18 @@ void modularity(Solver& S, const int32_t* labels0, double* Q) {
                   (int32_t)S.has_cw_h[i], (int32_t)S.has_gs_h[i]};
   }
   check_cuda(cudaMemcpyAsync(dqi, qi.data(), B * sizeof(QInst), cudaMemcpyHostToDevice, c.stream), "copy");
-  check_cuda(cudaMemsetAsync(acc, 0, (2 * (size_t)B + 2 * (size_t)Tn) * sizeof(ull), c.stream), "memset");
-  if (G.N > 0) launch(c, k_IJ, dim3(gsz(G.N * 8)), dim3(256), 0, g, labels0, acc, B);
+  check_cuda(cudaMemsetAsync(acc, 0, (accs + 1) * sizeof(ull), c.stream), "memset");
+  if (G.N > 0) {
+    const bool all_warps = G.N <= IJ_WARPS;
+    int32_t* hubs = G.hubs && !all_warps ? c.ws->get<int32_t>("q_hubs", G.nnz / HUB_ROW + 1) : nullptr;
+    if (all_warps || G.nnz > IJ_DENSE * G.N)
+      launch(c, k_IJ<32>, dim3(gsz(G.N * 32)), dim3(256), 0, g, labels0, acc, B, hubs, acc + accs);
+    else
+      launch(c, k_IJ<8>, dim3(gsz(G.N * 8)), dim3(256), 0, g, labels0, acc, B, hubs, acc + accs);
+    if (hubs)
+      launch(c, k_IJ_hubs, dim3(76, IJ_HUB_PARTS), dim3(256), 0, g, labels0, acc, B, (const int32_t*)hubs,
+             (const ull*)(acc + accs));
+  }
   const size_t smem = Tn <= 1024 ? 2 * (size_t)Tn * sizeof(ull) : 0;
   const int64_t span = S.sig.d ? S.sig.rows * S.sig.T : (int64_t)S.sig.h.cap;
   launch(c, k_S, dim3(gsz(span)), dim3(256), smem, S.sig, Tn, acc + 2 * B);
