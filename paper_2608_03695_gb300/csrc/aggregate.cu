@@ -508,27 +508,35 @@ __global__ void k_big_output(const int32_t* big, const int32_t* nbig_ptr, const 
   }
 }
 
-// Rows from the upper-bound layout to their final places (warp per row).
-__global__ void k_contract_compact(int32_t Np, const int64_t* eoff, const int32_t* ecnt, const int64_t* rowptr,
-                                   const int32_t* tcol, const long long* tw, int32_t* col, long long* W,
-                                   const int64_t* soff, const int32_t* scnt, const int64_t* sptr,
-                                   const int32_t* tsidx, const long long* tsval, int32_t* sidx, long long* sval) {
+// One row, by a warp, from the upper-bound layout (RowOut) to its final place.
+struct RowPlace {
+  const int64_t *rowptr, *sptr;
+  int32_t* col;
+  long long* W;
+  int32_t* sidx;
+  long long* sval;
+};
+
+__device__ __forceinline__ void contract_row_place(const RowOut& f, const RowPlace& t, int64_t x) {
   const int lane = threadIdx.x & 31;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t x = (((int64_t)blockIdx.x * blockDim.x) >> 5) + (threadIdx.x >> 5); x < Np; x += warps) {
-    const int64_t a = eoff[x], o = rowptr[x];
-    const int n = ecnt[x];
-    for (int k = lane; k < n; k += 32) {
-      col[o + k] = tcol[a + k];
-      W[o + k] = tw[a + k];
-    }
-    const int64_t sa = soff[x], so = sptr[x];
-    const int ns = scnt[x];
-    for (int k = lane; k < ns; k += 32) {
-      sidx[so + k] = tsidx[sa + k];
-      sval[so + k] = tsval[sa + k];
-    }
+  const int64_t a = f.eoff[x], o = t.rowptr[x];
+  const int n = f.ecnt[x];
+  for (int k = lane; k < n; k += 32) {
+    t.col[o + k] = f.tcol[a + k];
+    t.W[o + k] = f.tw[a + k];
   }
+  const int64_t sa = f.soff[x], so = t.sptr[x];
+  const int ns = f.scnt[x];
+  for (int k = lane; k < ns; k += 32) {
+    t.sidx[so + k] = f.tsidx[sa + k];
+    t.sval[so + k] = f.tsval[sa + k];
+  }
+}
+
+__global__ void k_contract_compact(int32_t Np, RowOut from, RowPlace to) {
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t x = (((int64_t)blockIdx.x * blockDim.x) >> 5) + (threadIdx.x >> 5); x < Np; x += warps)
+    contract_row_place(from, to, x);
 }
 
 __global__ void k_min_init(const int32_t* P, const int32_t* R, const int32_t* newid, int32_t N, int32_t* minid) {
@@ -564,10 +572,10 @@ __global__ void k_compose(const int32_t* R, const int32_t* newid, int64_t N0, in
 // The whole aggregation of a small level in one cooperative launch: the path
 // below is about 28 launches and three synchronisations (0.26 ms however small
 // the level); here they are eight grid barriers and one synchronisation, with
-// outputs allocated by upper bound.  Rows are summed by a warp or a block; a row
-// that needs more distinct targets than the block's table holds, or is so long
-// that one block would hold up the level, sends the level to the general path.
-// The next level's degree tiers are found on the way.
+// the rows' scratch allocated by upper bound.  Rows are summed by a warp or a
+// block; a row that needs more distinct targets than the block's table holds, or is
+// so long that one block would hold up the level, sends the level to the general
+// path.  The next level's degree tiers are found on the way.
 constexpr int64_t RESIDENT_ROW_MAX = 1 << 15;  // entries of a row one block sums
 
 struct AggCtl {
@@ -586,7 +594,7 @@ struct AggArgs {
   int32_t *tcol, *ecnt, *tsidx, *scnt_out;
   long long *tw, *tsval;
   int64_t *rowptr, *sptr;
-  int32_t *col, *sidx;
+  int32_t *col, *sidx;  // col: nullptr where the rows are moved by a launch of its own
   long long *W, *sval;
   int32_t* next_labels;
   int32_t *inst_next, *off_next;
@@ -867,17 +875,9 @@ __global__ void __launch_bounds__(RT, 1) k_aggregate(AggArgs a) {
     }
   }
   __syncthreads();
-  for (int32_t x = lo + w; x < hi; x += RW) {
-    const int64_t from = a.eoff[x], to = a.rowptr[x], sfrom = a.soff[x], sto = a.sptr[x];
-    const int n = a.ecnt[x], ns = a.scnt_out[x];
-    for (int k = lane; k < n; k += 32) {
-      a.col[to + k] = a.tcol[from + k];
-      a.W[to + k] = a.tw[from + k];
-    }
-    for (int k = lane; k < ns; k += 32) {
-      a.sidx[sto + k] = a.tsidx[sfrom + k];
-      a.sval[sto + k] = a.tsval[sfrom + k];
-    }
+  if (a.col) {
+    const RowPlace place{a.rowptr, a.sptr, a.col, a.W, a.sidx, a.sval};
+    for (int32_t x = lo + w; x < hi; x += RW) contract_row_place(o, place, x);
   }
   if (threadIdx.x < NTIERS && tiers[threadIdx.x]) atomicAdd(&a.ctl->tier[threadIdx.x], tiers[threadIdx.x]);
   if (tid == 0) {
@@ -922,6 +922,12 @@ static void next_level(const Level& L, Level& next, int32_t Np, int64_t mu, int6
 // Levels up to this many work units (entries, and RESIDENT_NODE_WORK a node) are
 // aggregated in one launch.
 constexpr int64_t RESIDENT_AGGREGATE_WORK = (int64_t)1 << 21;
+// Up to this many entries and strengths (12 bytes each) the rows go straight to
+// their places, in arrays sized by upper bound; past it they are moved once their
+// number is known.  A served window of 8 x 4,000 nodes, admitted at 19.2 MB, holds
+// 18.8 MB; 19.3 with 2^17, and 20.3 with every array by upper bound.  All of them
+// moved: n = 1,000, T = 4 1% longer.
+constexpr int64_t RESIDENT_PLACE_MAX = (int64_t)1 << 15;
 
 enum class Resident { DONE, SAME, GENERAL };  // SAME: nothing merged; GENERAL: not for one launch
 
@@ -955,10 +961,17 @@ static Resident aggregate_resident(Solver& S, const Level& L, const int32_t* P, 
   a.scnt_out = c.ws->get<int32_t>("ag_scnt_out", n1);
   a.rowptr = c.ws->get<int64_t>(slot + "_rowptr", n1);
   a.sptr = c.ws->get<int64_t>(slot + "_sptr", n1);
-  a.col = c.ws->get<int32_t>(slot + "_col", nnz);
-  a.W = c.ws->get<long long>(slot + "_W", nnz);
-  a.sidx = c.ws->get<int32_t>(slot + "_sidx", ns);
-  a.sval = c.ws->get<long long>(slot + "_sval", ns);
+  // The next level's rows stay allocated while it is solved (and the server admits
+  // requests by what a solve holds), so only few entries are given room by their
+  // upper bound.
+  const bool placed = L.nnz + L.ns <= RESIDENT_PLACE_MAX;
+  const auto place = [&](int64_t entries, int64_t strengths) {
+    a.col = c.ws->get<int32_t>(slot + "_col", entries);
+    a.W = c.ws->get<long long>(slot + "_W", entries);
+    a.sidx = c.ws->get<int32_t>(slot + "_sidx", strengths);
+    a.sval = c.ws->get<long long>(slot + "_sval", strengths);
+  };
+  if (placed) place(L.nnz, L.ns);
   a.next_labels = next_labels;
   a.B = S.B;
   if (L.d.inst) {
@@ -979,6 +992,12 @@ static Resident aggregate_resident(Solver& S, const Level& L, const int32_t* P, 
   std::memcpy(&h, readback(c, a.ctl, sizeof(AggCtl)), sizeof(AggCtl));
   if (h.np == N) return Resident::SAME;
   if (h.general) return Resident::GENERAL;
+  if (!placed) {
+    place(h.mu, h.ms);
+    launch(c, k_contract_compact, dim3(gsz((int64_t)h.np * 32)), dim3(256), 0, h.np,
+           RowOut{a.eoff, a.soff, a.tcol, a.tw, a.ecnt, a.tsidx, a.tsval, a.scnt_out},
+           RowPlace{a.rowptr, a.sptr, a.col, a.W, a.sidx, a.sval});
+  }
   if (node_of0)
     launch(c, k_compose, dim3(gsz(S.N0)), dim3(256), 0, (const int32_t*)S.R, (const int32_t*)a.newid, S.N0, node_of0);
   next_level(L, next, h.np, h.mu, h.ms, a.rowptr, a.col, a.W, a.sptr, a.sidx, a.sval, a.inst_next, a.off_next);
@@ -1122,10 +1141,8 @@ bool aggregate(Solver& S, const Level& L, const int32_t* P, Level& next, const s
   long long* W = c.ws->get<long long>(slot + "_W", mu);
   int32_t* sidx = c.ws->get<int32_t>(slot + "_sidx", ms);
   long long* sval = c.ws->get<long long>(slot + "_sval", ms);
-  launch(c, k_contract_compact, dim3(gsz((int64_t)Np * 32)), dim3(256), 0, Np, (const int64_t*)eoff,
-         (const int32_t*)ecnt, (const int64_t*)rowptr, (const int32_t*)tcol, (const long long*)tw, col, W,
-         (const int64_t*)soff, (const int32_t*)scnt_out, (const int64_t*)sptr, (const int32_t*)tsidx,
-         (const long long*)tsval, sidx, sval);
+  launch(c, k_contract_compact, dim3(gsz((int64_t)Np * 32)), dim3(256), 0, Np,
+         RowOut{eoff, soff, tcol, tw, ecnt, tsidx, tsval, scnt_out}, RowPlace{rowptr, sptr, col, W, sidx, sval});
 
   int32_t *inst_next = nullptr, *off_next = nullptr;
   if (L.d.inst) {
