@@ -551,8 +551,9 @@ _I64, _I32 = np.dtype(np.int64), np.dtype(np.int32)
 
 
 def _flat(a, dtype):
-    """`a` itself when it is such a contiguous array already."""
-    if type(a) is np.ndarray and a.dtype == dtype and a.flags.c_contiguous:
+    """`a` itself when it is such a contiguous array already (a scalar becomes an
+    array of one)."""
+    if type(a) is np.ndarray and a.dtype == dtype and a.flags.c_contiguous and a.ndim:
         return a
     return np.ascontiguousarray(a, dtype=dtype)
 
@@ -567,7 +568,10 @@ def _address(a):
 
 
 def _tensor_address(a):
-    return 0 if a is None else a.data_ptr()
+    """Address of a tensor's data, or of an array's beside tensors."""
+    if a is None:
+        return 0
+    return a.data_ptr() if hasattr(a, "data_ptr") else a.ctypes.data
 
 
 def _csr_array(snaps, device_ptrs=False, host_tensors=False):
