@@ -576,6 +576,7 @@ __global__ void k_compose(const int32_t* R, const int32_t* newid, int64_t N0, in
 // block; a row that needs more distinct targets than the block's table holds, or is
 // so long that one block would hold up the level, sends the level to the general
 // path.  The next level's degree tiers are found on the way.
+static_assert(R_PER_WARP >= 1 << CW_BITS, "a warp's share of the block's table holds a warp's row");
 constexpr int64_t RESIDENT_ROW_MAX = 1 << 15;  // entries of a row one block sums
 
 struct AggCtl {

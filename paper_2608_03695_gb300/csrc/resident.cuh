@@ -17,7 +17,7 @@ constexpr int RW = RT / 32;
 constexpr int R_SLOTS = TIER4_SMEM_SLOTS;
 constexpr int R_PER_WARP = R_SLOTS / RW;
 constexpr int R_BUCKET_ITEMS = 4;
-static_assert(R_PER_WARP == 1 << T2_BITS, "a warp's share of the block's table is tier 2's table");
+static_assert(R_PER_WARP >= 1 << T2_BITS, "a warp's share of the block's table holds tier 2's");
 
 __device__ __forceinline__ void resident_bar() {
   if (gridDim.x == 1)
