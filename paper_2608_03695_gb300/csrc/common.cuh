@@ -1,7 +1,9 @@
 // Device-side building blocks shared by the mslice kernels (sm_103a).
 #pragma once
-#include <cstdint>
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
+
+#include <cstdint>
 
 namespace mslice {
 
@@ -130,15 +132,16 @@ __device__ __forceinline__ void shared_add64(long long* p, long long x) {
 }
 
 // Counts a freshly taken slot against its region (rebuild trigger).  Threads of
-// a warp that take slots of the same region together count them with one
-// atomic: the nodes of a level's first table share a few regions, and one atomic
-// each (1.6 M on 16 words) took 0.5 ms where the inserts need 0.1.
+// a warp that take slots of the same region together (as many as happen to arrive
+// together: the count is right for any) count them with one atomic: the nodes of a
+// level's first table share a few regions, and one atomic each (1.6 M on 16 words)
+// took 0.5 ms where the inserts need 0.1.
 __device__ __forceinline__ void hash_took_slot(const HashView& h, ull key, uint64_t size) {
   if (!h.used) return;
   const uint32_t s = (uint32_t)key;
-  const unsigned peers = __match_any_sync(__activemask(), s);
-  if ((threadIdx.x & 31) != __ffs(peers) - 1) return;
-  const ull n = (ull)__popc(peers);
+  const auto peers = cooperative_groups::labeled_partition(cooperative_groups::coalesced_threads(), s);
+  if (peers.thread_rank() != 0) return;
+  const ull n = (ull)peers.size();
   // count the region once, when its taken slots pass half of it
   const ull taken = atomicAdd(&h.region_used[s], n) + n;
   if (2 * taken > size && 2 * (taken - n) <= size) atomicAdd(h.used, 1ull);
