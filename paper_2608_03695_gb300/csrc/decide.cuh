@@ -810,10 +810,8 @@ void decide_all(Ctx& c, const Pol& pol, const TierSegs& sg, const int32_t* tier_
   }
   if (tier_cnt[4] > 0) {
     // MSLICE_TIER4_SHARED=0: every tier-4 node uses global scratch
-    static const bool smem = [] {
-      const char* e = std::getenv("MSLICE_TIER4_SHARED");
-      return !(e && e[0] == '0');
-    }();
+    const char* e = std::getenv("MSLICE_TIER4_SHARED");
+    const bool smem = !(e && e[0] == '0');
     // 32 warps per tier-4 block where the group tiers hold few nodes (coarse
     // levels, where the hubs are the whole sub-round), 16 beside long group
     // tiers, whose blocks share the SMs
