@@ -285,12 +285,12 @@ struct RefPolicy {
     }
   }
   // randomised refinement: the key of target X when X is allowed and the
-  // key is >= 0 (cand() without its strict-gain filter)
+  // key is >= 0 (cand() without its strict-gain filter); not with L0
   __device__ bool rand_key(int32_t v, const VCtx& vc, int32_t X, long long W, i128& G) const {
     const Probe p = probe(v, vc, X);
     if (p.size == 1 && p.cls == q) return false;
     if (!p.wc) return false;
-    if (L0 || vc.single) {
+    if (vc.single) {
       const long long x = vc.k > 0 ? sst_resolve<DENSE>(kr, X, vc.s, p.first) : 0;
       G = (((i128)W) << P_BITS) - (i128)(vc.A * (u128)(ull)x);
     } else {
@@ -899,7 +899,7 @@ __global__ void k_ref_reset(Segs3 sg, int32_t* target) { ref_reset(sg, target); 
 
 // ---------------------------------------------------------------------------
 // The whole refinement of a small level in one cooperative launch: about 45
-// launches (0.35 ms, however small the level) become 4 K + 1 grid barriers.
+// launches (0.35 ms, however small the level) become 4 K grid barriers.
 // The right-hand sides of well-connectedness are summed over the members,
 //   sum_s Lambda_s K_{R,s} (K_{C,s} - K_{R,s})
 //     = sum_{v in R} sum_s Lambda_s k_{v,s} (K_{C,s} - K_{R,s}),
