@@ -35,6 +35,7 @@
 //   i128 own(v, vc, W_own)             score of staying
 //   void finish(v, best, W_best, G_own, vc)
 //   static constexpr int MIN_BLOCKS    resident blocks per SM the group tiers aim for
+//   static constexpr int BLOCK_MIN_BLOCKS  the same for tier 3
 // and, for the block tiers' slice-parallel scoring of aggregated nodes:
 //   int64_t slice_count(v)             entries of v's (snapshot, strength) list (0 at level 0)
 //   u128 null_part(v, vc, key, self, t, nt)  the null sum over entries t, t+nt, ...
@@ -433,21 +434,21 @@ __device__ __forceinline__ void group_decide_node(const Pol& pol, int32_t v, int
     const int j = gl / sub, slot = j < n ? CL[j] : 0;
     const int32_t key = j < n ? K[slot] : own;
     const u128 ns_sum =
-        lanes_sum_u128(key != own ? pol.null_part(v, vc, key, false, gl % sub, sub) : (u128)0, sub, gmask);
+        lanes_sum_u128(key != own ? pol.template null_part<4>(v, vc, key, false, gl % sub, sub) : (u128)0, sub, gmask);
     if (key != own && gl % sub == 0) c = pol.cand_ns(v, vc, key, V[slot], ns_sum);
   } else {
     for (int j = gl; j < n; j += G) {
       const int slot = CL[j];
       const int32_t key = K[slot];
       if (key != own) {
-        const Cand x = ns > 1 ? pol.cand_ns(v, vc, key, V[slot], pol.null_part(v, vc, key, false, 0, 1))
+        const Cand x = ns > 1 ? pol.cand_ns(v, vc, key, V[slot], pol.template null_part<4>(v, vc, key, false, 0, 1))
                               : pol.cand(v, vc, key, V[slot], pol.probe(v, vc, key));
         if (better(x, c)) c = x;
       }
     }
   }
   if (ns > 1 && pol.own_walks_slices()) {
-    const u128 ns_own = lanes_sum_u128(pol.null_part(v, vc, own, true, gl, G), G, gmask);
+    const u128 ns_own = lanes_sum_u128(pol.template null_part<4>(v, vc, own, true, gl, G), G, gmask);
     if (gl == 0) Gown = pol.own_ns(v, vc, table_get(K, V, BITS, own), ns_own);
   } else if (gl == 0) {
     Gown = pol.own(v, vc, table_get(K, V, BITS, own));
@@ -487,8 +488,9 @@ __device__ __forceinline__ Cand score_range(const Pol& pol, int32_t v, const typ
 // One node decided by the whole block with its table in shared memory
 // (hk/hv of at least 2^bits slots, all free on entry and left free; cl: room
 // for 2^bits / 2 slot numbers; ncand: a shared counter, 0 on entry and left
-// 0).  The node's distinct keys are listed as their slots are claimed.
-template <class Pol, int NT = BLOCK_THREADS>
+// 0).  The node's distinct keys are listed as their slots are claimed.  U: entries
+// of a strength list that a thread has in flight.
+template <class Pol, int NT = BLOCK_THREADS, int U = 1>
 __device__ __forceinline__ void block_decide_node(const Pol& pol, int32_t v, int32_t* hk, long long* hv, uint16_t* cl,
                                                   int32_t* ncand, Cand* red, ull* usm, i128* own_sm) {
   const typename Pol::VCtx vc = pol.vctx(v);
@@ -525,7 +527,7 @@ __device__ __forceinline__ void block_decide_node(const Pol& pol, int32_t v, int
       const int slot = j < n ? cl[j] : 0;
       const int32_t k = j < n ? hk[slot] : own;
       const bool walks = j < m && (stay || k != own);
-      u128 x = walks ? pol.null_part(v, vc, k, stay, threadIdx.x % sub, sub) : (u128)0;
+      u128 x = walks ? pol.template null_part<U>(v, vc, k, stay, threadIdx.x % sub, sub) : (u128)0;
       x = lanes_sum_u128(x, sub < 32 ? sub : 32, 0xffffffffu);
       if (sub > 32) {
         const int w = threadIdx.x >> 5;
@@ -595,7 +597,7 @@ __device__ __forceinline__ int block_claim(int32_t* queue, int count, int32_t* s
 }
 
 template <class Pol>
-__global__ void __launch_bounds__(BLOCK_THREADS)
+__global__ void __launch_bounds__(BLOCK_THREADS, Pol::BLOCK_MIN_BLOCKS)
     k_decide_block(Pol pol, const int32_t* list, const int32_t* count_ptr, int32_t* queue) {
   constexpr int SLOTS = 1 << TIER3_BITS;
   __shared__ int32_t hk[SLOTS];
@@ -642,7 +644,7 @@ __device__ __forceinline__ void gtable_add(int32_t* hk, long long* hv, int bits,
 
 // One node decided by a block of NT threads with its table in global scratch at
 // goff[v].
-template <class Pol, int NT>
+template <class Pol, int NT, int U = 1>
 __device__ __forceinline__ void block_decide_scratch(const Pol& pol, int32_t v, int32_t* gkeys, long long* gvals,
                                                      const int64_t* goff, unsigned* status, Cand* red, ull* usm,
                                                      i128* own_sm) {
@@ -672,7 +674,7 @@ __device__ __forceinline__ void block_decide_scratch(const Pol& pol, int32_t v, 
       const int32_t k = hk[i];
       if (k < 0 || k == own) continue;
       const u128 ns =
-          block_sum_u128<NT / 32>(pol.null_part(v, vc, k, false, threadIdx.x, NT), usm);
+          block_sum_u128<NT / 32>(pol.template null_part<U>(v, vc, k, false, threadIdx.x, NT), usm);
       if (threadIdx.x == 0) {
         const Cand x = pol.cand_ns(v, vc, k, hv[i], ns);
         if (better(x, c)) c = x;
@@ -681,7 +683,7 @@ __device__ __forceinline__ void block_decide_scratch(const Pol& pol, int32_t v, 
     i128 Go = 0;
     if (pol.own_walks_slices()) {
       const u128 ns =
-          block_sum_u128<NT / 32>(pol.null_part(v, vc, own, true, threadIdx.x, NT), usm);
+          block_sum_u128<NT / 32>(pol.template null_part<U>(v, vc, own, true, threadIdx.x, NT), usm);
       if (threadIdx.x == 0) Go = pol.own_ns(v, vc, table_get(hk, hv, bits, own), ns);
     } else if (threadIdx.x == 0) {
       Go = pol.own(v, vc, table_get(hk, hv, bits, own));

@@ -42,14 +42,16 @@ __device__ __forceinline__ u128 null_sum(const LevelDev& g, const u128* lam, con
   return t;
 }
 
-// The same over the entries t, t + nt, ... of v's list, four at a time: their
+// The same over the entries t, t + nt, ... of v's list, U at a time: their
 // table loads are in flight together before the first is used (a walk of one
-// entry at a time waits for two dependent loads each).  The group kernels keep
-// the plain walk: the registers of this one cost them a fifth of their speed.
-template <bool DENSE>
+// entry at a time waits for two dependent loads each).  The resident kernels take
+// four.  The large levels' kernels keep the plain walk: the registers of four cost
+// the group kernels a fifth of their speed, and took the dense block kernels from 64
+// registers to 74 (tier 3) and to 248 bytes of spills (tier 4): rows of 300 entries
+// with lists of 8 decided in 1.97 ms a round instead of 1.78 (N = 50,000).
+template <bool DENSE, int U>
 __device__ __forceinline__ u128 null_sum_part(const LevelDev& g, const u128* lam, const SigStore& h, int32_t v,
                                               int32_t c, bool self, int t, int nt) {
-  constexpr int U = 4;
   int64_t b, e;
   slice_range(g, v, b, e);
   u128 acc = 0;
@@ -84,6 +86,7 @@ __device__ __forceinline__ u128 null_sum_part(const LevelDev& g, const u128* lam
 template <bool DENSE, bool L0 = false>
 struct LMPolicy {
   static constexpr int MIN_BLOCKS = DENSE ? MSLICE_DENSE_MIN_BLOCKS : MSLICE_GROUP_MIN_BLOCKS;
+  static constexpr int BLOCK_MIN_BLOCKS = L0 ? 6 : 4;
   LevelDev g;
   const int32_t* labels;
   const int32_t* size;
@@ -162,8 +165,9 @@ struct LMPolicy {
   // slice-parallel scoring (block tiers, aggregated levels)
   __device__ int64_t slice_count(int32_t v) const { return L0 || g.is0 ? 0 : g.sptr[v + 1] - g.sptr[v]; }
   __device__ bool own_walks_slices() const { return true; }
+  template <int U>
   __device__ u128 null_part(int32_t v, const VCtx&, int32_t c, bool self, int t, int nt) const {
-    return null_sum_part<DENSE>(g, lam, sig, v, c, self, t, nt);
+    return null_sum_part<DENSE, U>(g, lam, sig, v, c, self, t, nt);
   }
   __device__ Cand cand_ns(int32_t, const VCtx& vc, int32_t c, long long W, const u128& ns) const {
     return Cand{(((i128)W) << P_BITS) - (i128)((u128)(ull)null_scale(g, vc.om) * ns), c};
@@ -633,6 +637,13 @@ __device__ __forceinline__ void lm_empty(const LevelDev& g, int32_t B, int32_t* 
 //   - Pruning that leaves three nodes in four in the lists is given up until
 //     the movement has fallen to a quarter, or for a number of rounds that
 //     doubles each time (communities can swap nodes for dozens of rounds).
+//   - After TRACK_FAILS levels of a kind (level 0, or aggregated) in a row whose
+//     pruning was given up like that, the next ones of that kind begin with a pause
+//     (see track_start): where margins are small beside the drift, every level of a
+//     solve records and prunes in vain.  The Constant Potts Model with gamma = 1 on
+//     T = 16, n = 100,000: 418 ms without this, 395 after 2 levels, 398 after 3; T = 64,
+//     n = 100,000, where later levels' pruning works, lost 7% after 1 level and up to
+//     2% after 2.
 //   - Levels with fewer entries, or with short rows (the decisions cost little
 //     more than the tracking), are not tracked, unless strength lists of two or
 //     more entries a node make their decisions dear (TRACK_MIN_LOOKUPS).
@@ -645,15 +656,21 @@ __device__ __forceinline__ void lm_empty(const LevelDev& g, int32_t B, int32_t* 
 constexpr int64_t TRACK_MIN_ENTRIES = 1 << 20, TRACK_MIN_DEGREE = 8;
 constexpr int64_t TRACK_MIN_LOOKUPS = 1 << 21;
 constexpr double TRACK_START = 1.0 / 16, TRACK_STOP = 1.0 / 4;
-constexpr int TRACK_FIRST_PAUSE = 8;
+constexpr int TRACK_FIRST_PAUSE = 8, TRACK_FAILS = 3;
 
 struct TrackState {
   int32_t mode, pause, next_pause, moved, pause_moved;
 };
 
-__host__ __device__ __forceinline__ TrackState track_next(const int32_t* prev, bool first, int32_t mode_init, long long moved,
-                                                 long long listed) {
-  TrackState s{mode_init, 0, TRACK_FIRST_PAUSE, 0, 0};
+// How a level's tracking starts: the mode of its first round, the rounds left
+// untracked at least, and the length of the next pause.
+struct TrackStart {
+  int32_t mode, pause, next_pause;
+};
+
+__host__ __device__ __forceinline__ TrackState track_next(const int32_t* prev, bool first, const TrackStart& start,
+                                                          long long moved, long long listed) {
+  TrackState s{start.mode, start.pause, start.next_pause, 0, 0};
   if (first) return s;
   const long long settled = prev[TRACK_SETTLED];
   const int32_t before = prev[TRACK_MODE], last = prev[TRACK_MOVED];
@@ -679,6 +696,22 @@ __host__ __device__ __forceinline__ TrackState track_next(const int32_t* prev, b
   else
     s.mode = (double)moved < TRACK_STOP * active ? TRACK_PRUNE : TRACK_OFF;
   return s;
+}
+
+// fails: levels of this kind in a row whose pruning was given up.
+inline TrackStart track_start(bool from_singletons, int fails) {
+  if (fails < TRACK_FAILS) return TrackStart{from_singletons ? TRACK_OFF : TRACK_RECORD, 0, TRACK_FIRST_PAUSE};
+  const int32_t pause = TRACK_FIRST_PAUSE << std::min(fails - TRACK_FAILS, 16);
+  return TrackStart{TRACK_OFF, pause, 2 * pause};
+}
+
+// The count after a level that ended in `state` with `listed` nodes in its last
+// round's lists; start: how it began.
+inline int track_fails(int fails, const TrackStart& start, const int32_t* state, long long listed) {
+  if (state[TRACK_MODE] == TRACK_PRUNE)
+    return listed > 3 * (long long)state[TRACK_SETTLED] ? fails + 1 : 0;
+  // (in a pause that began in this level)
+  return state[TRACK_PAUSE] > 0 && state[TRACK_NEXT_PAUSE] > start.next_pause ? fails + 1 : fails;
 }
 
 __device__ __forceinline__ void track_store(int32_t* state, const TrackState& s) {
@@ -748,7 +781,7 @@ struct ResidentIn {
   int r = 0, r_end = 0;
   bool first = false;        // r is the level's first round
   bool build = false;        // sizes and (dense) Sigma are to be built first
-  int32_t mode_init = 0;
+  TrackStart start{TRACK_OFF, 0, TRACK_FIRST_PAUSE};
   long long prev_moved = 0, prev_listed = 0;
   long long max_listed = 0;
 };

@@ -54,7 +54,8 @@ struct ResidentArgs {
   int32_t B;
   TrackView trk;       // of even rounds
   int32_t Tn;
-  int32_t mode_init, first;      // first: the level's first round is this launch's
+  TrackStart start;
+  int32_t first;                 // the level's first round is this launch's
   long long prev_moved, prev_listed;  // of the round before this launch
   uint64_t seed, it, lvl;
   int32_t r0, r_end, K;
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
       trk.Bp = a.trk.B + (int64_t)(1 - p) * a.Tn;
       if (threadIdx.x == 0) {
         const TrackState st =
-            track_next(a.trk.state + (1 - p) * TRACK_WORDS, a.first && r == a.r0, a.mode_init, moved, listed);
+            track_next(a.trk.state + (1 - p) * TRACK_WORDS, a.first && r == a.r0, a.start, moved, listed);
         mode_sh = st.mode;
         if (blockIdx.x == 0) track_store(trk.state, st);
       }
@@ -176,9 +177,9 @@ __global__ void __launch_bounds__(RT, 1) k_lm_rounds(Pol pol, ResidentArgs a) {
           sg,
           [&](int32_t v) {
             if (table_bits_for_degree(a.g.rowptr[v + 1] - a.g.rowptr[v]) <= TIER4_SMEM_BITS)
-              block_decide_node<Pol, RT>(pol, v, hk, hv, cl, &block_ncand, red, usm, &own_sm);
+              block_decide_node<Pol, RT, 4>(pol, v, hk, hv, cl, &block_ncand, red, usm, &own_sm);
             else
-              block_decide_scratch<Pol, RT>(pol, v, a.gkeys, a.gvals, a.goff, a.status, red, usm, &own_sm);
+              block_decide_scratch<Pol, RT, 4>(pol, v, a.gkeys, a.gvals, a.goff, a.status, red, usm, &own_sm);
           },
           [&](int32_t v) {
             group_decide_node<Pol, 32, T2_BITS, 2>(pol, v, hk + w * R_PER_WARP, hv + w * R_PER_WARP,
@@ -271,7 +272,7 @@ void resident_rounds(Solver& S, const Level& L, int32_t* labels, int it, int lvl
   a.B = S.B;
   a.trk = trk;
   a.Tn = S.Tn;
-  a.mode_init = in.mode_init;
+  a.start = in.start;
   a.first = in.first ? 1 : 0;
   a.prev_moved = in.prev_moved;
   a.prev_listed = in.prev_listed;

@@ -256,11 +256,11 @@ __global__ void k_count_sizes(const int32_t* size, int64_t N, ull* out) {
 // Round start (one block) of a tracked round: its tracking state, budgets and
 // counters, and the other parity's accumulators cleared for the round after.
 __global__ void __launch_bounds__(512) k_round_begin(TrackView trk, int32_t* state_prev, int32_t Tn, int first,
-                                                     int32_t mode_init, long long moved, long long listed,
+                                                     TrackStart start, long long moved, long long listed,
                                                      int32_t* counters) {
   __shared__ int32_t mode_sh;
   if (threadIdx.x == 0) {
-    const TrackState st = track_next(state_prev, first, mode_init, moved, listed);
+    const TrackState st = track_next(state_prev, first, start, moved, listed);
     mode_sh = st.mode;
     track_store(trk.state, st);
     trk.state[TRACK_PAST] = trk.state[TRACK_SETTLED] = 0;
@@ -719,7 +719,8 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
                                   L.ns <= 4 * (int64_t)N) ||
                                      (L.ns >= 2 * (int64_t)N && L.nnz + L.nnz / N * L.ns >= TRACK_MIN_LOOKUPS);
   const TrackView trk = !worth || tuning ? TrackView{} : track_view(S, L);
-  const int32_t mode_init = lvl == 0 && it == 0 && !S.warm ? TRACK_OFF : TRACK_RECORD;
+  int& fails = S.track_fails[lvl > 0];
+  const TrackStart start = track_start(lvl == 0 && it == 0 && !S.warm, fails);
   if (trk.state)
     check_cuda(cudaMemsetAsync(trk.state, 0, 2 * TRACK_WORDS * sizeof(int32_t), c.stream), "memset");
   // Batch: an instance whose round moved nothing is at a fixed point of
@@ -754,7 +755,7 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
       in.first = first_round;
       in.build = build;
       build = false;
-      in.mode_init = mode_init;
+      in.start = start;
       in.prev_moved = moved;
       in.prev_listed = listed;
       in.max_listed = 2 * few;  // (some slack, so that rounds do not change hands to and fro)
@@ -791,11 +792,11 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
     // lengths and the tracking mode go to the pinned buffer.
     const TrackView tr = track_at(trk, S.Tn, r);
     // (the mode k_round_begin comes to, from the same words)
-    const bool tracked = tr.state && track_next(state, first_round, mode_init, moved, listed).mode != TRACK_OFF;
+    const bool tracked = tr.state && track_next(state, first_round, start, moved, listed).mode != TRACK_OFF;
     const BucketLists bl{S.lists, (int64_t)S.N0, S.cursors, tier_offsets(S), S.bseg};
     if (tr.state)
       launch(c, k_round_begin, dim3(1), dim3(512), 0, tr, track_at(trk, S.Tn, r + 1).state, S.Tn, (int)first_round,
-             mode_init, moved, listed, S.counters);
+             start, moved, listed, S.counters);
     else
       check_cuda(cudaMemsetAsync(S.counters, 0, 3 * sizeof(int32_t), c.stream), "memset");
     bucket_tracked(S, L, 0, it, lvl, r, active, tr);
@@ -866,6 +867,7 @@ MoveOut local_move(Solver& S, const Level& L, int32_t* labels, int it, int lvl, 
     if (r == max_rounds) out.capped = true;
   }
   S.lm_moves += out.moves;
+  if (trk.state) fails = track_fails(fails, start, state, listed);
   return out;
 }
 

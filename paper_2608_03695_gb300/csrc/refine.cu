@@ -164,6 +164,7 @@ __global__ void k_wc(LevelDev g, const int32_t* sizeR, const long long* Wout, co
 template <bool DENSE, bool L0 = false>
 struct RefPolicy {
   static constexpr int MIN_BLOCKS = DENSE ? MSLICE_DENSE_MIN_BLOCKS : MSLICE_GROUP_MIN_BLOCKS;
+  static constexpr int BLOCK_MIN_BLOCKS = L0 ? 6 : 4;
   LevelDev g;
   const int32_t* P;
   const int32_t* R;
@@ -264,8 +265,9 @@ struct RefPolicy {
   // slice-parallel scoring (block tiers, aggregated levels); own() is 0
   __device__ int64_t slice_count(int32_t v) const { return L0 || g.is0 ? 0 : g.sptr[v + 1] - g.sptr[v]; }
   __device__ bool own_walks_slices() const { return false; }
+  template <int U>
   __device__ u128 null_part(int32_t v, const VCtx&, int32_t X, bool, int t, int nt) const {
-    return null_sum_part<DENSE>(g, lam, kr, v, X, false, t, nt);
+    return null_sum_part<DENSE, U>(g, lam, kr, v, X, false, t, nt);
   }
   __device__ Cand cand_ns(int32_t, const VCtx& vc, int32_t X, long long W, const u128& ns) const {
     const unsigned long long d = desc[X];
@@ -1033,9 +1035,9 @@ __global__ void __launch_bounds__(RT, 1) k_refine(RefPolicy<DENSE> pol, RefArgs 
             if (!pol.begin(v)) {
               if (threadIdx.x == 0) pol.skip(v);
             } else if (table_bits_for_degree(a.g.rowptr[v + 1] - a.g.rowptr[v]) <= TIER4_SMEM_BITS) {
-              block_decide_node<RefPolicy<DENSE>, RT>(pol, v, hk, hv, cl, &block_ncand, red, usm, &own_sm);
+              block_decide_node<RefPolicy<DENSE>, RT, 4>(pol, v, hk, hv, cl, &block_ncand, red, usm, &own_sm);
             } else {
-              block_decide_scratch<RefPolicy<DENSE>, RT>(pol, v, a.gkeys, a.gvals, a.goff, a.status, red, usm, &own_sm);
+              block_decide_scratch<RefPolicy<DENSE>, RT, 4>(pol, v, a.gkeys, a.gvals, a.goff, a.status, red, usm, &own_sm);
             }
           },
           [&](int32_t v) {

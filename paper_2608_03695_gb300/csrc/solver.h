@@ -98,6 +98,7 @@ struct Solver {
   // given labels
   long long* track_base = nullptr;
   std::vector<long long> track_base_h;
+  int track_fails[2] = {0, 0};  // levels in a row whose pruning was given up: level 0, aggregated levels
   double total_strength = 0;
   bool warm = false;
   int32_t* wqueue = nullptr;       // work counters of the decision kernels, one per degree tier
